@@ -26,7 +26,7 @@ struct perm_run_s {
     int device = 0, num_sms = 0;
     bool key64 = false;
     int thresh = perm::kSnapshot;
-    int log2h = 0, slots = 0, ctas = 0, worker_warps = 0, lanes = 0, stride = 32, stack_cache = 16;
+    int log2h = 0, slots = 0, ctas = 0, worker_warps = 0, lanes = 0, stack_cache = 16;
     size_t smem = 0;
     int arena_mode = 0;            // perm::ArenaMode
     long long arena_cta_bytes = 0;
@@ -93,6 +93,7 @@ void free_all(perm_handle h) {
 
 // Parts of one tour that may grow on other walks at once (shared copies), and the
 // larger bound used once no tour of the run has finished for kStallNs.
+constexpr int kAutoWalks = 32;          // walks per CTA of the automatic layout
 constexpr int kDefaultShareCap = 4;
 constexpr int kBoostShareCap = 1024;
 constexpr long long kStallNs = 5000000;
@@ -215,12 +216,13 @@ int create_impl(perm_handle *out, const perm_config *cfg, const ForcedLayout *fo
     }
     h->own_stream = true;
 
-    // layout: walks per warp (lanes), worker warps per CTA, CTAs.  Each thread
-    // grows one walk; the walks of an SM are spread over about four warps so
-    // that every scheduler has a walk's dependent chain to issue from.
+    // layout: walks per warp (lanes), walk warps per CTA, CTAs.  A group of lanes grows
+    // one walk; the walks of an SM are spread over up to 8 warps, so that every
+    // scheduler has two walks' dependent chains to issue from.
     const bool snap = (h->thresh == perm::kSnapshot);
     const size_t budget = force ? force->smem_budget : prop.sharedMemPerBlockOptin;
-    auto pow2_at_least = [](int v) { int p = 1; while (p < v) p <<= 1; return p; };
+    const int max_l = perm::walks_per_warp_max(d), max_w = perm::kMaxWalkWarps;
+    const size_t walk_b = perm::walk_bytes(key64, n_max, log2h, h->stack_cache);
     // where the walks' hashes, site lists and stack rings live: shared memory, or a
     // global arena when asked for or when not one walk per CTA fits beside the head
     const size_t head_b = perm::cta_head_bytes(n_max, snap);
@@ -230,23 +232,19 @@ int create_impl(perm_handle *out, const perm_config *cfg, const ForcedLayout *fo
     };
     int arena_mode = arena_for(force ? 1 : cfg->walk_memory);
     if (!force && cfg->walk_memory == 0 &&
-        perm::cta_smem_bytes(d, key64, n_max, log2h, h->stack_cache, 1, snap, 1) > budget)
+        head_b + walk_b > budget)
         arena_mode = arena_for(2);
-    auto smem_for = [&](int warps, int stride) {
+    auto smem_for = [&](int walks) {
         if (arena_mode == perm::kArenaWalks) return head_b;
         if (arena_mode == perm::kArenaAll) return (size_t)0;
-        return perm::cta_smem_bytes(d, key64, n_max, log2h, h->stack_cache, warps, snap, stride);
+        return head_b + walk_b * (size_t)walks;
     };
     if (!force && cfg->max_ctas == -1) {
-        // dense packing: the fewest CTAs (of up to 8 x 32 walks) that hold one walk
+        // dense packing: the fewest CTAs (of up to 8 full warps) that hold one walk
         // per sequence, so that runs sharing the device take few SMs each
         long long per_cta = 0;
-        for (int w = 1; w <= 8; ++w)
-            for (int l = 32; l >= 1; --l)
-                if (smem_for(w, pow2_at_least(l)) <= budget) {
-                    per_cta = std::max(per_cta, (long long)w * l);
-                    break;
-                }
+        for (int t = max_w * max_l; t >= 1; --t)
+            if (smem_for(t) <= budget) { per_cta = t; break; }
         if (per_cta > 0) {
             const long long need = ((long long)n_seq + per_cta - 1) / per_cta;
             h->num_sms = (int)std::max(1LL, std::min((long long)h->num_sms, need));
@@ -263,39 +261,37 @@ int create_impl(perm_handle *out, const perm_config *cfg, const ForcedLayout *fo
     if (helpers < 0) helpers = can_help && !lpw ? std::max(0LL, (long long)h->num_sms * 32 - tslots) : 0;
     long long slots = tslots + helpers;
     const long long slots_wanted = slots;
-    int warps = 0, lanes = 0, stride = 0;
+    int warps = 0, lanes = 0;
+    // walks of a CTA over its warps: over as many of the 8 as there are walks
+    auto spread = [&](int t) {
+        lanes = (t + max_w - 1) / max_w;
+        warps = (t + lanes - 1) / lanes;
+    };
     if (force) {
-        // every CTA of the batch grid may join this run: the most walks up to
-        // 4 warps x 8 (the automatic layout's bound) that fit the shared memory
-        for (int w = 4; w >= 1 && !warps; --w)
-            for (int l = 8; l >= 1; --l)
-                if (smem_for(w, pow2_at_least(l)) <= budget) { warps = w; lanes = l; stride = pow2_at_least(l); break; }
+        // every CTA of the batch grid may join this run: the most walks up to 32 (the
+        // automatic layout's bound) that fit the shared memory
+        for (int t = kAutoWalks; t >= 1 && !warps; --t) {
+            spread(t);
+            if (smem_for(warps * lanes) > budget) warps = 0;
+        }
         slots = (long long)force->ctas * warps * lanes;
         if (!warps || slots > (1LL << 30)) { cudaStreamDestroy(h->stream); delete h; return PERM_EUNSUPPORTED; }
         h->num_sms = force->ctas;
     }
     for (; !force;) {
         const long long per_cta = (slots + h->num_sms - 1) / h->num_sms;
-        int best_w = 0, best_l = 0, best_s = 0;
-        for (int w = 1; w <= 8; ++w) {
-            int l = (int)((per_cta + w - 1) / w);
-            if (lpw) { if (l > lpw) continue; l = lpw < l ? lpw : l; }
-            // automatic: at most 4 walk warps of 8 walks.  A warp's walks take
-            // different paths through the step, so its iteration time grows with its
-            // walks, and past about 32 walks per SM more walks buy little and lengthen
-            // the start-up (cubic lattice, n_max 512, 8192 sequences: 4 x 8 walks per
-            // SM run in 0.57 s, 5 x 8 in 0.63 s)
-            else if (l > 8 || w > 4) continue;
-            if (l > 32 || (long long)w * l < per_cta) continue;
-            const int st = pow2_at_least(l);
-            if (smem_for(w, st) > budget) continue;
-            // prefer about four warps; among fitting choices keep the first that reaches it
-            if (best_w == 0 || (best_w < 4 && w <= 4) || (lpw && w < best_w)) {
-                best_w = w; best_l = l; best_s = st;
+        // automatic: at most 32 walks per SM.  More lengthen the start-up and buy little
+        const int cap = lpw ? max_w * std::min(lpw, max_l) : kAutoWalks;
+        if (per_cta <= cap) {
+            if (lpw) {
+                lanes = (int)std::min<long long>(per_cta, std::min(lpw, max_l));
+                warps = (int)((per_cta + lanes - 1) / lanes);
+            } else {
+                spread((int)per_cta);
             }
-            if (!lpw && w >= 4) break;
+            if (smem_for(warps * lanes) <= budget) break;
+            warps = 0;
         }
-        if (best_w) { warps = best_w; lanes = best_l; stride = best_s; break; }
         if (slots <= 1) break;
         slots = slots - (slots + 7) / 8;        // does not fit: fewer concurrent walks
     }
@@ -313,15 +309,13 @@ int create_impl(perm_handle *out, const perm_config *cfg, const ForcedLayout *fo
     h->tour_slots = force ? (int)slots : (int)std::min(tslots, slots);
     h->worker_warps = warps;
     h->lanes = lanes;
-    h->stride = stride;
     h->slots = (int)slots;
-    h->smem = smem_for(warps, stride);
+    h->smem = smem_for(warps * lanes);
     // the batch kernel grows its members with the shared-memory body only
     if (force && arena_mode != perm::kArenaNone) { cudaStreamDestroy(h->stream); delete h; return PERM_EUNSUPPORTED; }
     h->arena_mode = arena_mode;
     if (arena_mode != perm::kArenaNone) {
-        const size_t wb = perm::cta_warp_bytes(key64, n_max, log2h, h->stack_cache, stride);
-        h->arena_cta_bytes = (long long)(wb * (size_t)warps + (arena_mode == perm::kArenaAll ? head_b : 0));
+        h->arena_cta_bytes = (long long)(walk_b * (size_t)(warps * lanes) + (arena_mode == perm::kArenaAll ? head_b : 0));
         h->arena_cta_bytes = (h->arena_cta_bytes + 255) & ~255LL;
         // at most 64 GB of walk state
         if ((double)h->arena_cta_bytes * h->ctas > 64e9) { cudaStreamDestroy(h->stream); delete h; return PERM_ENOMEM; }
@@ -409,7 +403,7 @@ static RunDev make_params(perm_handle h) {
     RunDev P;
     std::memset(&P, 0, sizeof(P));
     P.d = h->cfg.d; P.n_max = h->cfg.n_max; P.n_seq = h->cfg.n_seq; P.alg = h->cfg.alg;
-    P.log2h = h->log2h; P.S = h->lanes; P.stride = h->stride;
+    P.log2h = h->log2h; P.S = h->lanes;
     P.worker_warps = h->worker_warps; P.slots = h->slots; P.tour_slots = h->tour_slots;
     P.stack_cache = h->stack_cache;
     P.arena_mode = h->arena_mode; P.arena = h->arena; P.arena_cta_bytes = h->arena_cta_bytes;

@@ -9,10 +9,13 @@
 //     probability 1 - r, a survivor's weight is multiplied by 1/r.
 //
 // Layout conventions shared by the kernels:
-//   - A walk's occupancy hash and its per-site slot list live in shared memory,
-//     interleaved by lane: element i of lane l is at [i * S + l] (S = lanes per
-//     warp), so that every lane always hits its own bank.
-//   - Keys pack the lattice coordinates of a site; 0 is the empty slot.
+//   - A group of lanes holds one walk: 4 lanes on the square lattice, 8 on the cubic
+//     one.  Every lane of a group carries the walk's state; lane j of the group
+//     stands for direction j.
+//   - A walk's occupancy hash, its per-site slot list and its stack ring are
+//     contiguous.  The hash is made of 16-byte buckets.
+//   - Keys pack the lattice coordinates of a site; 0 is the empty slot.  The key of
+//     neighbour j is the site's key plus a constant of the direction.
 //   - Directions: j = 0..2d-1 -> axis j/2, sign + for even j (+x,-x,+y,-y,+z,-z).
 #pragma once
 
@@ -45,13 +48,16 @@ __device__ __forceinline__ Philox4 philox4x32_10(uint32_t c0, uint32_t c1, uint3
 
 // ---------------------------------------------------------------------------
 // Site keys.  Key32<2>: 16-bit fields x+32768 | (y+32768)<<16, |x|,|y| <= 32766.
-// Key32<3>: 10-bit fields (c+512) mod 1024, for walks with n_max <= 512: every
-// stored site has |c| <= 511 (field 1..1023, never 0); a probe at |c| = 512
-// gives field 0 and cannot match a stored site.  Key64<3>: 21-bit fields.
+// Key32<3>: c+512 at bits 0, 11 and 22, for walks with n_max <= 512: every stored
+// site has |c| <= 511 (field 1..1023, never 0); a probe at c = -512 gives field 0,
+// one at +512 sets the guard bit above the field (for z it leaves field 0), so
+// neither matches a stored site, and adding a direction's constant never borrows
+// from or carries into another field.  Key64<3>: 21-bit fields.
 // ---------------------------------------------------------------------------
 template <int D, typename Key> struct KeyCodec;
 
 template <> struct KeyCodec<2, uint32_t> {
+    static constexpr int kField = 16;
     __device__ __forceinline__ static uint32_t encode(int x, int y, int) {
         return (uint32_t)(x + 32768) | ((uint32_t)(y + 32768) << 16);
     }
@@ -63,18 +69,21 @@ template <> struct KeyCodec<2, uint32_t> {
 };
 
 template <> struct KeyCodec<3, uint32_t> {
+    static constexpr int kField = 11;
     __device__ __forceinline__ static uint32_t encode(int x, int y, int z) {
-        return ((uint32_t)(x + 512) & 1023u) | (((uint32_t)(y + 512) & 1023u) << 10) |
-               (((uint32_t)(z + 512) & 1023u) << 20);
+        return (uint32_t)(x + 512) + ((uint32_t)(y + 512) << 11) + ((uint32_t)(z + 512) << 22);
     }
+    // (the end-point of a walk of 512 steps along z reads z = -512 for +512: the
+    // same square)
     __device__ __forceinline__ static void decode(uint32_t k, int &x, int &y, int &z) {
-        x = (int)(k & 1023u) - 512;
-        y = (int)((k >> 10) & 1023u) - 512;
-        z = (int)((k >> 20) & 1023u) - 512;
+        x = (int)(k & 2047u) - 512;
+        y = (int)((k >> 11) & 2047u) - 512;
+        z = (int)(k >> 22) - 512;
     }
 };
 
 template <> struct KeyCodec<3, unsigned long long> {
+    static constexpr int kField = 21;
     __device__ __forceinline__ static unsigned long long encode(int x, int y, int z) {
         return (unsigned long long)(uint32_t)(x + (1 << 20)) |
                ((unsigned long long)(uint32_t)(y + (1 << 20)) << 21) |
@@ -87,85 +96,72 @@ template <> struct KeyCodec<3, unsigned long long> {
     }
 };
 
-__device__ __forceinline__ uint32_t hash_home(uint32_t k, int log2h) {
-    return (k * 0x9E3779B1u) >> (32 - log2h);
-}
-__device__ __forceinline__ uint32_t hash_home(unsigned long long k, int log2h) {
-    const uint32_t f = (uint32_t)k ^ (uint32_t)(k >> 29) ^ (uint32_t)(k >> 53);
-    return (f * 0x9E3779B1u) >> (32 - log2h);
-}
-
-// Neighbour j of (x, y, z).
-__device__ __forceinline__ void step_coords(int j, int &x, int &y, int &z) {
-    const int s = (j & 1) ? -1 : 1;
-    if (j < 2) x += s; else if (j < 4) y += s; else z += s;
-}
-
-// Open addressing with triangular probing: the i-th probe of key k is slot
-// home(k) + i(i+1)/2 mod 2^log2h, which visits every slot once in the first
-// 2^log2h probes.  Against linear probing it breaks up the runs of occupied
-// slots that a walk's clustered sites leave, so the longest probe of a warp's
-// walks (the warp waits for it) is shorter: on random square-lattice walks of up
-// to 511 steps, 3.5 rounds against 4.6 for the longest of six walks' neighbour
-// probes.  Deletion in LIFO order stays exact for any fixed probe sequence.
-//
-// Insert a key known to be absent; returns its slot, or -1 if the probe
-// sequence ran through the whole table (full: impossible at load factor <= 1/2).
-template <typename Key>
-__device__ __forceinline__ int hash_insert(Key *tab, int S, int lane, int log2h, Key k) {
-    const uint32_t mask = (1u << log2h) - 1u;
-    uint32_t s = hash_home(k, log2h);
-    for (int it = 0; it <= (int)mask; ++it) {
-        Key *p = tab + (s * (uint32_t)S + (uint32_t)lane);
-        if (*p == (Key)0) { *p = k; return (int)s; }
-        s = (s + (uint32_t)it + 1u) & mask;
-    }
-    return -1;
-}
-
-// ---------------------------------------------------------------------------
-// a_+ (Sec. 1): probe the 2d neighbours of the end-point (triangular probing).
-// Returns the free mask; slot[j] is the empty slot that ended the probe of a
-// free direction j (its insertion slot while the table is unchanged).  Each
-// round loads all 2d slots and updates the probes with selects (no branches);
-// at load factor <= 1/2 almost every probe ends in the first round.
-// ---------------------------------------------------------------------------
+// What a step in direction j adds to a site's key.
 template <int D, typename Key>
-__device__ __forceinline__ int probe_neighbours(const Key *tab, int S, int lane, int log2h,
-                                                int x, int y, int z, int (&slot)[2 * D],
-                                                bool &overflow, int back = -1) {
-    const uint32_t mask = (1u << log2h) - 1u;
-    Key key[2 * D];
-    uint32_t s[2 * D];
-#pragma unroll
-    for (int j = 0; j < 2 * D; ++j) {
-        int xx = x, yy = y, zz = z;
-        step_coords(j, xx, yy, zz);
-        key[j] = KeyCodec<D, Key>::encode(xx, yy, zz);
-        s[j] = hash_home(key[j], log2h);
-        slot[j] = 0;
+__device__ __forceinline__ Key step_key(int j) {
+    const Key one = (Key)1 << (KeyCodec<D, Key>::kField * (j >> 1));
+    return (j & 1) ? (Key)0 - one : one;
+}
+
+// ---------------------------------------------------------------------------
+// The occupancy hash: 2^log2b buckets of 16 bytes (4 keys of 32 bits or 2 of 64),
+// probed triangularly from the key's home: the i-th bucket is home + i(i+1)/2 mod
+// 2^log2b, which visits every bucket once.  A key sits in the first bucket of its
+// sequence with room, in that bucket's first empty place.  Keys are deleted in
+// LIFO order only, so a bucket's keys always fill its first places, every bucket
+// that a key passed over is full while the key lives, and a probe may stop at the
+// first bucket that is not full.  One 16-byte load settles a probe unless the
+// bucket is full: at the load of at most 1/2 that a walk reaches at n_max, one
+// bucket of four in seven is full, against one slot in two with one key per probe.
+// ---------------------------------------------------------------------------
+template <typename Key> struct Buckets {
+    static constexpr int kKeys = 16 / (int)sizeof(Key);
+    static constexpr int kLog2 = sizeof(Key) == 4 ? 2 : 1;
+};
+
+__device__ __forceinline__ uint32_t hash_home(uint32_t k, int log2b) {
+    return (k * 0x9E3779B1u) >> (32 - log2b);
+}
+__device__ __forceinline__ uint32_t hash_home(unsigned long long k, int log2b) {
+    const uint32_t f = (uint32_t)k ^ (uint32_t)(k >> 29) ^ (uint32_t)(k >> 53);
+    return (f * 0x9E3779B1u) >> (32 - log2b);
+}
+
+// One bucket: whether it holds k, whether it is full, its first empty place.
+__device__ __forceinline__ void look_bucket(const uint32_t *tab, uint32_t b, uint32_t k, bool &hit, bool &full, int &e) {
+    const uint4 v = *reinterpret_cast<const uint4 *>(tab + 4u * b);
+    hit = v.x == k || v.y == k || v.z == k || v.w == k;
+    full = v.w != 0u;
+    e = (v.x != 0u) + (v.y != 0u) + (v.z != 0u);
+}
+__device__ __forceinline__ void look_bucket(const unsigned long long *tab, uint32_t b, unsigned long long k, bool &hit,
+                                            bool &full, int &e) {
+    const ulonglong2 v = *reinterpret_cast<const ulonglong2 *>(tab + 2u * b);
+    hit = v.x == k || v.y == k;
+    full = v.y != 0ull;
+    e = v.x != 0ull;
+}
+
+// Every lane of the warp probes for its own key in its own walk's table (want:
+// the lane takes part).  Returns true if the key is absent; `slot` is then where
+// it would be inserted.  `overflow`: the probe ran through the whole table
+// (impossible at a load of at most 1/2).
+template <typename Key>
+__device__ __forceinline__ bool probe(const Key *tab, int log2b, Key k, bool want, int &slot, bool &overflow) {
+    const uint32_t mask = (1u << log2b) - 1u;
+    uint32_t b = hash_home(k, log2b);
+    bool absent = false, pend = want;
+    for (uint32_t it = 0;; ++it) {
+        bool hit, full;
+        int e;
+        look_bucket(tab, b, k, hit, full, e);
+        if (pend && !hit && !full) { absent = true; slot = (int)(b * (uint32_t)Buckets<Key>::kKeys) + e; }
+        pend = pend && !hit && full;
+        if (!__any_sync(0xFFFFFFFFu, pend)) break;
+        if (it >= mask) { overflow = pend; break; }
+        b = (b + it + 1u) & mask;
     }
-    // direction `back` leads to the walk's previous site, occupied by definition:
-    // no probe
-    uint32_t pending = ((1u << (2 * D)) - 1u) & ~(back >= 0 ? 1u << back : 0u), freem = 0u;
-    for (int it = 0; it <= (int)mask; ++it) {
-        Key v[2 * D];
-#pragma unroll
-        for (int j = 0; j < 2 * D; ++j) v[j] = tab[s[j] * (uint32_t)S + (uint32_t)lane];
-#pragma unroll
-        for (int j = 0; j < 2 * D; ++j) {
-            const bool pend = (pending >> j) & 1u;
-            const bool hit = v[j] == key[j];
-            const bool emp = v[j] == (Key)0;          // keys are never 0
-            slot[j] = (pend && emp) ? (int)s[j] : slot[j];
-            freem |= (uint32_t)(pend && emp) << j;
-            pending &= ~((uint32_t)(pend && (hit || emp)) << j);
-            s[j] = (s[j] + (uint32_t)it + 1u) & mask; // harmless for resolved probes
-        }
-        if (pending == 0u) break;
-    }
-    overflow = pending != 0u;
-    return (int)freem;
+    return absent;
 }
 
 // ---------------------------------------------------------------------------
@@ -180,30 +176,27 @@ __device__ __forceinline__ int probe_neighbours(const Key *tab, int S, int lane,
 // settle it.  The decision then equals the one taken on the double-precision
 // r at every node.
 //
-// The estimate: x = M / (1 + Wsum/W), with the two doubles entering through
-// their mantissas rounded to 24 bits (nearest, ties to even; a carry bumps the
-// exponent) and their exponents.  Each quotient is a product with the
-// hardware's approximate reciprocal (rcp.approx, at most one unit in the last
-// place, i.e. relative error <= 2^-23) rounded once more; the other operations
-// are correctly rounded single-precision ones.  Relative errors: the two
-// mantissas 2^-24 each, the quotient 3 2^-24, the sum 1 + rho 2^-24 (plus rho's
-// own 5 2^-24 scaled by rho/(1 + rho) < 1), M 2^-24 and the final quotient
-// 3 2^-24, with the three roundings of the double-precision r (<= 4 2^-53):
-// |x - r| <= 10.02 2^-24 x.  Every margin below allows at least 15 2^-24 x.
-// Doubles with no such bound (W zero, negative, subnormal or not finite; Wsum
-// negative, subnormal or not finite; Wsum/W above 2^100) set `odd` and take
-// the exact path, and so does M of 2^32 or more (M enters through a 32-bit
-// conversion: a 64-bit one costs as much as a double-precision operation).
-// Every operation here is single-precision or integer arithmetic: a double-
-// precision one takes 64 cycles or more on this part.
+// The estimate: x = (M m_w) / (m_w + m_s 2^(e_s - e_w)), with the two doubles
+// entering through their mantissas truncated to 24 bits and their exponents.  The
+// quotient is a product with the hardware's approximate reciprocal (rcp.approx, at
+// most one unit in the last place, i.e. relative error <= 2^-23); the other
+// operations are correctly rounded single-precision ones (the scaling by a power
+// of two is exact).  Relative errors of x, in 2^-24: the truncated mantissas 2
+// each (x depends on W/Wsum with a logarithmic derivative below 1), M 1, M m_w 1,
+// the sum 1, the reciprocal 2, the last product 1, with the three roundings of the
+// double-precision r (<= 4 2^-53): |x - r| <= 10.02 2^-24 x.  Every margin below
+// allows at least 15 2^-24 x.  Doubles with no such bound (W zero, negative,
+// subnormal or not finite; Wsum negative, subnormal or not finite; Wsum/W above
+// 2^100) set `odd` and take the exact path, and so does M of 2^32 or more (M
+// enters through a 32-bit conversion: a 64-bit one costs as much as a
+// double-precision operation).  Every operation here is single-precision or integer
+// arithmetic: a double-precision one takes 64 cycles or more on this part.  (With
+// mantissas rounded to nearest and two reciprocals, M / (1 + Wsum/W), the bound was
+// the same and the chain one reciprocal and a dozen integer operations longer.)
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ uint32_t mant24_bits(unsigned long long b, int &ef) {
-    const uint32_t hi = (uint32_t)(b >> 32) & 0xFFFFFu, lo = (uint32_t)b;
-    uint32_t keep = (hi << 3) | (lo >> 29);          // top 23 fraction bits
-    const uint32_t rem = lo & 0x1FFFFFFFu;           // the 29 bits dropped
-    if (rem > 0x10000000u || (rem == 0x10000000u && (keep & 1u))) keep += 1u;
-    if (keep == (1u << 23)) { keep = 0u; ef += 1; }
-    return (127u << 23) | keep;
+// The top 24 bits of a double's mantissa as a float in [1, 2).
+__device__ __forceinline__ float mant24(uint32_t hi, uint32_t lo) {
+    return __uint_as_float((__funnelshift_l(lo, hi, 3) & 0x7FFFFFu) | 0x3F800000u);
 }
 
 // 1/v to within one unit in the last place (v normal and positive).
@@ -213,26 +206,24 @@ __device__ __forceinline__ float rcp_approx(float v) {
     return r;
 }
 
-__device__ __forceinline__ float ratio_estimate(double W, double Wsum, unsigned long long M, bool &odd) {
-    const unsigned long long wb = (unsigned long long)__double_as_longlong(W);
-    const unsigned long long sb = (unsigned long long)__double_as_longlong(Wsum);
-    int ew = (int)((uint32_t)(wb >> 52) & 0x7FFu), es = (int)((uint32_t)(sb >> 52) & 0x7FFu);
-    const bool s_zero = (sb == 0ull);
-    bool bad = (wb >> 63) != 0ull || (sb >> 63) != 0ull || ew == 0 || ew == 0x7FF || es == 0x7FF ||
-               (es == 0 && !s_zero);
-    const float mw = __uint_as_float(mant24_bits(wb, ew));
-    const float ms = __uint_as_float(mant24_bits(sb, es));
-    const float q = __fmul_rn(ms, rcp_approx(mw));    // in (0.5, 2)
+// M as the estimate takes it (-1: beyond the estimate's range).
+__device__ __forceinline__ float tours_float(unsigned long long M) {
+    return (M >> 32) != 0ull ? -1.0f : __uint2float_rn((uint32_t)M);
+}
+
+__device__ __forceinline__ float ratio_estimate(double W, double Wsum, float Mf, bool &odd) {
+    const uint32_t wh = (uint32_t)__double2hiint(W), wl = (uint32_t)__double2loint(W);
+    const uint32_t sh = (uint32_t)__double2hiint(Wsum), sl = (uint32_t)__double2loint(Wsum);
+    const int ew = (int)(wh >> 20), es = (int)(sh >> 20);      // sign bit and exponent
+    const bool s_zero = (sh | sl) == 0u;
+    const float mw = mant24(wh, wl);
+    // below 2^-100 the ratio only moves the sum by less than 2^-99 of it
     int e = es - ew;
-    bad = bad || (!s_zero && e > 100);
-    // below 2^-100 the ratio only moves 1 + rho by less than 2^-99
+    odd = (uint32_t)(ew - 1) >= 2046u || ((uint32_t)(es - 1) >= 2046u && !s_zero) || (!s_zero && e > 100) || Mf < 0.0f;
     e = e < -100 ? -100 : (e > 100 ? 100 : e);
-    float rho = __fmul_rn(q, __uint_as_float((uint32_t)(e + 127) << 23));   // exact scaling
-    rho = s_zero ? 0.0f : rho;
-    const float s = __fadd_rn(1.0f, rho);
-    const float Mf = __uint2float_rn((uint32_t)M);
-    odd = bad || (M >> 32) != 0ull;
-    return __fmul_rn(Mf, rcp_approx(s));
+    float ms = __fmul_rn(mant24(sh, sl), __uint_as_float((uint32_t)(e + 127) << 23));   // exact scaling
+    ms = s_zero ? 0.0f : ms;
+    return __fmul_rn(__fmul_rn(Mf, mw), rcp_approx(__fadd_rn(mw, ms)));
 }
 
 // r exactly as defined, in double precision: three correctly rounded operations
@@ -260,42 +251,30 @@ __device__ __forceinline__ double widen(float f) {
 // ---------------------------------------------------------------------------
 // The decision of Sec. 2 on the estimate x (enrichment: c = floor r iff
 // u0 < ceil(r) - r, at most a_+ copies; pruning: survive iff u0 < r, with
-// u0 = w0 2^-32).  Sets `amb` when x cannot settle it:
+// u0 = w0 2^-32).  Both are the floor of one sum: for r >= 1, c = floor(r + u0); for
+// r < 1, c = floor(r + 1 - u0) (1: survive).  Sets `amb` when x cannot settle it:
 //  - the branch: x >= 1 + 2^-19 gives r > 1, x <= 1 - 2^-19 gives r < 1;
-//  - x (1 - 2^-20) >= a_+ + 1 gives floor r > a_+, so c = a_+ whatever u0;
-//  - floor and ceil: x farther than x 2^-20 from an integer gives
-//    floor r = floor x;
-//  - the u0 comparisons, on w0 against the threshold P = (ceil x - x) 2^32 or
-//    P = x 2^32 (exact in single precision), which is within 2565 x of the
-//    threshold of r: |w0 - P| > 4096 x + 512 settles them (the 512 covers the
-//    rounding of w0 to single precision and of the difference, 128 each).
+//  - the floor: the sum y for x lies within x 2^-20 + 2^-23 of an integer k <= a_+
+//    (past a_+ both neighbours of k give c = a_+).  The sum for r is within
+//    10.02 x 2^-24 (the estimate) + 2^-25 (u0 to single precision) + (x + 1) 2^-24
+//    (the sum's rounding) of y, which is less.  (r an integer: c = r whatever u0, and
+//    so is floor(r + u0).)
+// x enters capped at 16, past every a_+ + 1.  Selects, no branches: a warp's walks
+// take different sides, and a branch costs a lone warp 25 cycles or more.  (The same
+// decision by ceilings and thresholds on w0 took 144 cycles of a lone warp, this
+// one 60.)
 // Returns c (0: pruned); `surv` marks a survivor of pruning.
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ int decide_estimate(float x, int a, uint32_t w0, bool &surv, bool &amb) {
-    const float w0f = __uint2float_rn(w0);
-    const float margin = __fmaf_rn(x, 4096.0f, 512.0f);
-    int c = 0;
-    surv = false;
-    amb = false;
-    if (x >= 1.0f + 0x1p-19f) {
-        if (__fmul_rn(x, 1.0f - 0x1p-20f) >= (float)(a + 1)) {
-            c = a;
-        } else {
-            const float fl = floorf(x), ce = __fadd_rn(fl, 1.0f);
-            const float fr = __fsub_rn(x, fl), p = __fsub_rn(ce, x);          // both exact
-            const float dlt = __fsub_rn(w0f, __fmul_rn(p, 4294967296.0f));
-            amb = fminf(fr, p) <= __fmul_rn(x, 0x1p-20f) || fabsf(dlt) <= margin;
-            const float craw = dlt < 0.0f ? fl : ce;
-            c = (craw >= (float)a) ? a : (int)craw;
-        }
-    } else if (x <= 1.0f - 0x1p-19f) {
-        const float dlt = __fsub_rn(w0f, __fmul_rn(x, 4294967296.0f));
-        amb = fabsf(dlt) <= margin;
-        surv = dlt < 0.0f;
-        c = surv ? 1 : 0;
-    } else {
-        amb = true;
-    }
+    const float uf = __fmul_rn(__uint2float_rn(w0), 0x1p-32f), vf = __fmul_rn(__uint2float_rn(~w0), 0x1p-32f);
+    const float xc = fminf(x, 16.0f), lim = (float)a;
+    const bool up = xc >= 1.0f;
+    const float y = __fadd_rn(xc, up ? uf : vf);
+    const float k = __fsub_rn(__fadd_rn(y, 12582912.0f), 12582912.0f);        // y to the nearest integer
+    const float tol = __fmaf_rn(xc, 0x1p-20f, 0x1p-23f);
+    amb = fabsf(__fsub_rn(xc, 1.0f)) < 0x1p-19f || (fabsf(__fsub_rn(y, k)) <= tol && k <= lim);
+    const int c = (int)fminf(k > y ? __fsub_rn(k, 1.0f) : k, lim);
+    surv = !up && c > 0;
     return c;
 }
 
@@ -314,20 +293,15 @@ __device__ __forceinline__ int decide_exact(double r, int a, uint32_t w0, bool &
     return surv ? 1 : 0;
 }
 
-// Partial Fisher-Yates: c distinct free steps from the free list (3 bits per
-// entry), draws by multiply-high on w1 (one dependent chain, stopped after c).
-__device__ __forceinline__ uint32_t choose_steps(int c, int a, uint32_t freelist, uint32_t w1) {
-    uint32_t x = w1, list = freelist;
-    for (int i = 0; i < c; ++i) {
-        const uint32_t m = (uint32_t)(a - i);
-        const unsigned long long prod = (unsigned long long)x * m;
-        const int j = i + (int)(prod >> 32);
-        x = (uint32_t)prod;
-        const uint32_t vi = (list >> (3 * i)) & 7u, vj = (list >> (3 * j)) & 7u;
-        const uint32_t t = vi ^ vj;
-        list ^= (t << (3 * i)) | (t << (3 * j));
-    }
-    return (c == 0) ? 0u : list;
+// Step i of a partial Fisher-Yates shuffle of the free list (3 bits per entry, a
+// entries): entry i changes places with one drawn from i..a-1 by multiply-high on x,
+// which keeps the product's low word for the next draw.
+__device__ __forceinline__ void choose_step(int i, int a, uint32_t &list, uint32_t &x) {
+    const unsigned long long prod = (unsigned long long)x * (uint32_t)(a - i);
+    const int si = 3 * i, sj = 3 * (i + (int)(prod >> 32));
+    x = (uint32_t)prod;
+    const uint32_t t = ((list >> si) ^ (list >> sj)) & 7u;
+    list ^= (t << si) ^ (t << sj);                  // the same place: the two cancel
 }
 
 }  // namespace perm

@@ -1,12 +1,27 @@
 // perm_kernels.cu -- persistent flatPERM growth kernel (Algorithms 1 and 2 of
 // Campbell and Janse van Rensburg, "Parallel PERM", Sec. 3) for sm_103a.
 //
-// One thread grows one walk ("slot"); a warp holds up to 32 walks.  Per walk,
-// shared memory holds the occupancy hash (triangular probing, deleted in LIFO
-// order on backtrack), the hash slot of every site, and the top of the stack
-// of waiting copies (the rest spills to global memory).  Each thread runs the
-// tours handed to it one after another; a tour is a depth-first traversal of
-// the tree of copies made by enrichment (Sec. 2).
+// A group of lanes grows one walk ("slot"): 4 lanes on the square lattice, 8 on the
+// cubic one, so a warp holds up to 8 or 4 walks.  Every lane of a group carries the
+// walk's state; lane j probes neighbour j, deletes every 4th (8th) site of a
+// backtrack, and issues one of the node's table updates.  Per walk, shared memory
+// holds the occupancy hash (16-byte buckets, keys deleted in LIFO order on
+// backtrack), the hash slot of every site, and the top of the stack of waiting
+// copies (the rest spills to global memory).  Each walk runs the tours handed to
+// it one after another; a tour is a depth-first traversal of the tree of copies
+// made by enrichment (Sec. 2).
+//
+// What bounds it: the walks are few (one per sequence, at most 32 an SM here), so
+// each warp's dependent instruction stream sets the rate, not memory, issue slots
+// or arithmetic.  On this part a lone warp pays 25 cycles or more for a branch, 45
+// for a vote and a branch on it, 20-60 for a reduction, 33 for a shared-memory load,
+// 64 for every double-precision instruction whatever its active lanes (measured, one
+// warp).  One lane per walk ran all four (six) probes, the table updates and a dozen
+// branches of a node one after another, 7 walks to a warp; a group of lanes does them
+// side by side, and the node is one straight line.  GB300, group of lanes against
+// one lane per walk: 12 walks to n = 16, 24 000 tours 48.5 -> 31.5 ms; square n = 512,
+// 4096 sequences, 96 tours each of a continued run 193 -> 126 ms, 256 tours from
+// empty tables 561 -> 302 ms; cubic n = 512, 8192 sequences, 128 tours 491 -> 253 ms.
 //
 // Threshold sources for Algorithm 2 (one shared table W, Fig. 1):
 //  - snapshot: every node adds its weight to the global table with a
@@ -33,9 +48,7 @@ namespace perm {
 
 namespace {
 
-constexpr int kStride = 32;        // interleave stride of the snapshot-state kernel
-constexpr int kUnwind = 8;         // hash deletions per walk per iteration
-constexpr int kNodePasses = 2;     // nodes a walk may grow per iteration
+constexpr int kUnwindSites = 16;   // hash deletions per walk per iteration
 constexpr int kPoolExtra = 4;      // extra tour tickets fetched per warp (snapshot)
 constexpr int kChunk = 8;          // stack records moved per spill or fill (ring >= 2 kChunk)
 constexpr int kReloadBatch = 8;    // snapshot entries a refresher lane loads before storing them
@@ -82,33 +95,48 @@ __device__ __forceinline__ void set_status(int *status, int code) {
 
 __device__ __forceinline__ size_t align16(size_t b) { return (b + 15) & ~(size_t)15; }
 
-__host__ __device__ __forceinline__ size_t warp_region_bytes(int n_max, int log2h, int K,
-                                                             size_t key_bytes, int stride) {
-    const size_t hash_b = ((((size_t)1 << log2h) * stride * key_bytes) + 15) & ~(size_t)15;
-    const size_t sites_b = (((size_t)n_max * stride * 2) + 15) & ~(size_t)15;
-    const size_t stk_b = (((size_t)K * stride * 4) + 15 & ~(size_t)15) + (size_t)K * stride * 8;
-    return hash_b + sites_b + stk_b;
+// A walk's region: hash, site list, stack ring (records, then their weights).
+__host__ __device__ __forceinline__ size_t walk_hash_bytes(int log2h, size_t key_bytes) {
+    return ((size_t)1 << log2h) * key_bytes;              // a multiple of 16: 2^4 slots or more
+}
+__host__ __device__ __forceinline__ size_t walk_sites_bytes(int n_max) { return ((size_t)n_max * 2 + 15) & ~(size_t)15; }
+__host__ __device__ __forceinline__ size_t walk_region_bytes(int n_max, int log2h, int K, size_t key_bytes) {
+    return walk_hash_bytes(log2h, key_bytes) + walk_sites_bytes(n_max) + (size_t)K * 12;
 }
 
 __host__ __device__ __forceinline__ size_t head_region_bytes(int n_max, bool snapshot) {
     const size_t L = (size_t)n_max + 1;
-    size_t b = 64 + 2 * 64 * 8;   // header + two a/c tables
+    size_t b = 64 + 1024;         // header + constants (fill_constants)
     if (snapshot) b += 8 * L;     // the snapshot of W_n
     return (b + 15) & ~(size_t)15;
 }
 
-// Weight factors for the two scale steps dE of the lattice (row t: dE = dE_lo + t):
-// [a*8 + c] = (a/c) 2^-dE for c >= 1 (enrichment), [a*8 + 0] = a 2^-dE (exact).
-__device__ void fill_aoc(double *aoc, int d, int tid, int nthreads) {
+// The constants of a CTA's head region: weight factors for the two scale steps dE of
+// the lattice (t: dE = dE_lo + t), [t*48 + (a-1)*8 + c] = (a/c) 2^-dE for c >= 1
+// (enrichment), c = 0: a 2^-dE (exact); and after the 96 factors the free list of
+// every free mask (directions in order, 3 bits each).
+constexpr int kFactors = 96;
+__device__ void fill_constants(double *aoc, int d, int tid, int nthreads) {
     const int dE_lo = (d == 2) ? 1 : 2;
-    for (int i = tid; i < 128; i += nthreads) {
-        const int t = i >> 6, a = (i >> 3) & 7, c = i & 7;
-        double v = 0.0;
+    for (int i = tid; i < kFactors; i += nthreads) {
+        const int t = i / 48, a = (i % 48) / 8 + 1, c = i & 7;
         const double s = __longlong_as_double((long long)((unsigned long long)(1023 - dE_lo - t) << 52));
-        if (a >= 1 && c >= 1) v = __dmul_rn(__ddiv_rn((double)a, (double)c), s);
-        else if (a >= 1) v = __dmul_rn((double)a, s);
-        aoc[i] = v;
+        aoc[i] = c >= 1 ? __dmul_rn(__ddiv_rn((double)a, (double)c), s) : __dmul_rn((double)a, s);
     }
+    uint32_t *lists = reinterpret_cast<uint32_t *>(aoc + kFactors);
+    for (int m = tid; m < 64; m += nthreads) {
+        uint32_t list = 0u;
+        int cnt = 0;
+        for (int j = 0; j < 6; ++j)
+            if (m >> j & 1) { list |= (uint32_t)j << (3 * cnt); ++cnt; }
+        lists[m] = list;
+    }
+}
+
+// E(n+1) - E(n) - dE_lo: which of the lattice's two scale steps length n takes.
+template <int D>
+__device__ __forceinline__ int scale_row(int n) {
+    return D == 2 ? (((3 * n) & 7) + 3) >> 3 : ((n & 3) + 1) >> 2;
 }
 
 // Original PERM's cut-offs (Sec. 2) as a node reads them: per length (T_n, t_n)
@@ -121,137 +149,136 @@ struct Cutoffs {
     unsigned long long K;
 };
 
-struct NodeOut {
-    int outcome, a, mask, c;
-    uint32_t dirs;
+// What the nodes of a walk compute from M, the tours started: once per tour and
+// snapshot (a double-precision division takes as long as a node).
+struct Tours {
+    unsigned long long M;
+    float Mf;                  // tours_float(M)
+    double inv1, inv3, inv5;   // 1/M rounded to double, and 3 and 5 times that
+};
+__device__ __forceinline__ void set_tours(Tours &t, unsigned long long M) {
+    t.M = M;
+    t.Mf = tours_float(M);
+    t.inv1 = __drcp_rn(__ull2double_rn(M));
+    t.inv3 = __dmul_rn(3.0, t.inv1);
+    t.inv5 = __dmul_rn(5.0, t.inv1);
+}
+
+struct Decision {
+    int c;               // copies (0: pruned)
     double r;            // r as the decision used it (single-precision estimate or exact)
     double child_w;
-    bool overflow;
     bool exact;          // the decision was taken on r in double precision
 };
 
+// r exactly as defined and the decision on it (out of line: one node in 10^4 or fewer).
+__device__ __noinline__ Decision decide_node_exact(int a, double W, double Wsum, unsigned long long M, uint32_t w0,
+                                                   double a_sc) {
+    Decision o;
+    bool surv = false;
+    o.exact = true;
+    o.r = ratio_exact(W, Wsum, M);
+    o.c = decide_exact(o.r, a, w0, surv);
+    if (surv) o.child_w = __dmul_rn(__dmul_rn(W, __ddiv_rn(1.0, o.r)), a_sc);
+    else o.child_w = __dmul_rn(__ddiv_rn(W, (double)(o.c > 0 ? o.c : 1)), a_sc);
+    return o;
+}
+
+// The decision at a node with a >= 1 free neighbours (Sec. 2): r, the copies, the
+// children's weight.  Wsum: sum of the weights recorded at length n before this
+// node; refine: round the survivor's quotient by M correctly (one more step of the
+// division).  valid: the lane has a node to decide (the others' results are not used);
+// force_exact: decide on the double-precision r.  Shared by the persistent kernel
+// and the snapshot-state kernel; every lane of a walk's group takes the same decision.
+// One straight line with selects but for the exact path: a branch costs a lone warp
+// 25 cycles or more, a double-precision instruction 64 whatever its active lanes.
+template <int D>
+__device__ __forceinline__ Decision decide_node(int n, int a, double W, double Wsum, const Tours &t, bool refine,
+                                                uint32_t w0, const double *aoc, bool valid, bool force_exact) {
+    Decision o;
+    o.exact = false;
+    bool odd = false, amb = false, surv = false;
+    const double sum = __dadd_rn(Wsum, W);
+    const float x = ratio_estimate(W, Wsum, t.Mf, odd);
+    o.r = n == 0 ? 1.0 : widen(x);
+    const int dE = scale_row<D>(n) + (D == 2 ? 1 : 2);
+    const double *row = aoc + 48 * (dE - (D == 2 ? 1 : 2)) + 8 * (a - 1);
+    int c = decide_estimate(x, a, w0, surv, amb);
+    if (n == 0) { c = 1; surv = false; }                 // r = 1 at the empty walk
+    const bool exact = valid && n != 0 && (amb || odd || force_exact);
+    // a survivor carries W/r = [W_n]^sample = (Wsum + W)/M, a child of an enrichment
+    // (W/c) a_+ 2^-dE: one double-precision product for both, on the critical path
+    // alone.  The survivor's factor (1/M) a_+ 2^-dE (a node past the empty walk has
+    // a_+ <= 5) is one of three products kept per M, its exponent shifted (exact: 1/M
+    // is far from the subnormals); the weight is within 2^-51 of the quotient
+    double base = W, fac = row[c];
+    if (refine) {
+        // q = sum (1/M), then q + (sum - q M)/M: the quotient to half a unit
+        const double Md = __ull2double_rn(t.M), q = __dmul_rn(sum, t.inv1);
+        base = surv ? __fma_rn(__fma_rn(-q, Md, sum), t.inv1, q) : W;
+        fac = surv ? row[0] : fac;
+    } else {
+        const double f0 = a == 3 ? t.inv3 : (a == 5 ? t.inv5 : t.inv1);
+        const int sh = (a == 2 ? 1 : (a == 4 ? 2 : 0)) - dE;
+        const double fs = __hiloint2double(__double2hiint(f0) + (sh << 20), __double2loint(f0));
+        base = surv ? sum : W;
+        fac = surv ? fs : fac;
+    }
+    o.child_w = __dmul_rn(base, fac);
+    o.c = c;
+    // the estimate cannot settle a comparison: r exactly as defined
+    if (exact) o = decide_node_exact(a, W, Wsum, t.M, w0, row[0]);
+    return o;
+}
+
+// Original PERM's decision (Sec. 2, cut-offs T_n, t_n) at a node past the empty walk:
+// copies above T_n, survival with probability 1/q (weight times q) below t_n, one
+// copy between them.
+template <int D>
+__device__ __forceinline__ Decision decide_cutoffs(int n, int a, double W, uint32_t w0, const double *aoc,
+                                                   const Cutoffs &cuts) {
+    Decision o;
+    const double *row = aoc + 48 * scale_row<D>(n) + 8 * (a - 1);
+    const double2 tc = __ldg(cuts.cut + n);
+    o.exact = false;
+    const bool above = W > tc.x, below = W < tc.y;
+    o.c = above ? (cuts.copies < a ? cuts.copies : a) : (below && !((unsigned long long)w0 < cuts.K) ? 0 : 1);
+    o.r = above ? (double)cuts.copies : (below ? cuts.inv_q : 1.0);
+    o.child_w = __dmul_rn(below && !above ? __dmul_rn(W, cuts.q) : W, row[above ? o.c : 0]);
+    return o;
+}
+
+// A reduction into global memory by the lanes that take part, without a branch around it
+// (the compiler's costs a lone warp 40 cycles, the predicated instruction 20).
+__device__ __forceinline__ void red_add(double *p, double v, bool take) {
+    asm volatile("{\n.reg .pred q;\nsetp.ne.s32 q, %2, 0;\n@q red.relaxed.gpu.global.add.f64 [%0], %1;\n}"
+                 :: "l"(p), "d"(v), "r"((int)take) : "memory");
+}
+__device__ __forceinline__ void red_inc(unsigned long long *p, bool take) {
+    asm volatile("{\n.reg .pred q;\nsetp.ne.s32 q, %2, 0;\n@q red.relaxed.gpu.global.add.u64 [%0], %1;\n}"
+                 :: "l"(p), "l"(1ull), "r"((int)take) : "memory");
+}
+
 // The whole warp copies a donor's sites 0..bdp (key and hash slot) into a cell.
 template <typename Key>
-__device__ __noinline__ void copy_sites_to_cell(const Key *hash, const uint16_t *sites, int ST, int src,
-                                                int bdp, Key *ck, uint16_t *cs, int lane) {
+__device__ __noinline__ void copy_sites_to_cell(const Key *hash, const uint16_t *sites, int bdp, Key *ck, uint16_t *cs,
+                                                int lane) {
     for (int k = lane; k <= bdp; k += 32) {
-        const uint16_t sl = sites[(uint32_t)k * ST + src];
-        ck[k] = hash[(uint32_t)sl * ST + src];
+        const uint16_t sl = sites[k];
+        ck[k] = hash[sl];
         cs[k] = sl;
     }
 }
 
 // The whole warp places a taker's sites 0..dp from a cell at their hash slots.
 template <typename Key>
-__device__ __noinline__ void place_sites_from_cell(Key *hash, uint16_t *sites, int ST, int src, int dp,
-                                                   const Key *ck, const uint16_t *cs, int lane) {
+__device__ __noinline__ void place_sites_from_cell(Key *hash, uint16_t *sites, int dp, const Key *ck, const uint16_t *cs,
+                                                   int lane) {
     for (int k = lane; k <= dp; k += 32) {
         const uint16_t sl = __ldcg(cs + k);
-        hash[(uint32_t)sl * ST + src] = __ldcg(ck + k);
-        sites[(uint32_t)k * ST + src] = sl;
+        hash[sl] = __ldcg(ck + k);
+        sites[k] = sl;
     }
-}
-
-// One node's growth step (Sec. 1 and Sec. 2): a_+, r, decision, steps, child
-// weight.  Wsum: sum of the weights recorded at length n before this node;
-// M: tours started.  force_exact: take every decision on the double-precision r.
-// Shared by the persistent kernel and the snapshot-state kernel.
-template <int D, typename Key>
-__device__ __forceinline__ NodeOut grow_node(const Key *hash, int stride, int lane, int log2h, int n,
-                                             int n_max, int cx, int cy, int cz, double W, double Wsum,
-                                             unsigned long long M, unsigned long long ordinal,
-                                             uint32_t seq, uint32_t tour, uint32_t k0, uint32_t k1,
-                                             const double *aoc, int (&eslot)[2 * D],
-                                             const Cutoffs &cuts, double invM = 0.0, int back = -1,
-                                             bool force_exact = false) {
-    NodeOut o;
-    o.a = 0; o.mask = 0; o.c = 0; o.dirs = 0u; o.child_w = 0.0; o.overflow = false; o.exact = false;
-    // three independent chains: the node's random block, the estimate of r, and the probes
-    const Philox4 w = philox4x32_10((uint32_t)ordinal, (uint32_t)(ordinal >> 32), tour, seq, k0, k1);
-    bool odd = false;
-    const float x = ratio_estimate(W, Wsum, M, odd);
-    o.r = n == 0 ? 1.0 : widen(x);
-    if (n == n_max) { o.outcome = kLeafNmax; return o; }
-    bool ovf = false;
-    const int fm = probe_neighbours<D, Key>(hash, stride, lane, log2h, cx, cy, cz, eslot, ovf, back);
-    o.overflow = ovf;
-    o.mask = fm;
-    const int a = __popc(fm);
-    o.a = a;
-    if (a == 0) { o.outcome = kTrapped; return o; }
-    uint32_t freelist = 0u;
-    int cnt = 0;
-#pragma unroll
-    for (int j = 0; j < 2 * D; ++j) {
-        if (fm >> j & 1) { freelist |= (uint32_t)j << (3 * cnt); ++cnt; }
-    }
-    const int dE = scale_exp(D, n + 1) - scale_exp(D, n);
-    const int dE_lo = (D == 2) ? 1 : 2;
-    const double *row = aoc + 64 * (dE - dE_lo);
-    const double a_sc = row[a * 8];                      // a_+ 2^-dE, exact
-    int c;
-    bool surv = false;
-    if (n == 0) {
-        c = 1;                                           // r = 1 at the empty walk
-        o.child_w = __dmul_rn(W, a_sc);
-    } else if (cuts.cut != nullptr) {
-        // original PERM (Sec. 2, cut-offs T_n, t_n): copies above T_n, survival with
-        // probability 1/q (weight times q) below t_n, one copy between them
-        const double2 tc = __ldg(cuts.cut + n);
-        if (W > tc.x) {
-            c = cuts.copies < a ? cuts.copies : a;
-            o.r = (double)cuts.copies;
-            o.child_w = __dmul_rn(W, row[a * 8 + c]);
-        } else if (W < tc.y) {
-            surv = (unsigned long long)w.x < cuts.K;
-            c = surv ? 1 : 0;
-            o.r = cuts.inv_q;
-            o.child_w = __dmul_rn(__dmul_rn(W, cuts.q), a_sc);
-        } else {
-            c = 1;
-            o.r = 1.0;
-            o.child_w = __dmul_rn(W, a_sc);
-        }
-    } else {
-        bool amb = false;
-        c = decide_estimate(x, a, w.x, surv, amb);
-        if (amb || odd || force_exact) {
-            // the estimate cannot settle a comparison: r exactly as defined
-            const double R = ratio_exact(W, Wsum, M);
-            c = decide_exact(R, a, w.x, surv);
-            o.r = R;
-            o.exact = true;
-            if (surv) o.child_w = __dmul_rn(__dmul_rn(W, __ddiv_rn(1.0, R)), a_sc);
-            else if (c > 0) o.child_w = __dmul_rn(__ddiv_rn(W, (double)c), a_sc);
-        } else {
-            // a survivor carries W/r = [W_n]^sample = (Wsum + W)/M, a child of an
-            // enrichment (W/c) a_+ 2^-dE: one double-precision product for both.
-            // invM (when nonzero) is 1/M rounded to double; the survivor's factor
-            // (1/M) a_+ 2^-dE is formed beside the sum Wsum + W, so that its weight
-            // (within 2^-51 of the quotient, relative) takes two dependent double
-            // operations.  The tests of invM and of the outcome are integer ones
-            double base = W, fac = row[a * 8 + c];
-            if (surv) {
-                base = __dadd_rn(Wsum, W);
-                if (__double_as_longlong(invM) != 0ll) fac = __dmul_rn(invM, a_sc);
-                else { base = __ddiv_rn(base, __ull2double_rn(M)); fac = a_sc; }
-            }
-            o.child_w = __dmul_rn(base, fac);
-        }
-    }
-    if (c == 0) { o.outcome = kPruned; o.child_w = 0.0; return o; }
-    o.c = c;
-    o.dirs = choose_steps(c, a, freelist, w.y);
-    o.outcome = kChildren;
-    return o;
-}
-
-template <int D>
-__device__ __forceinline__ int select_slot(const int (&eslot)[2 * D], int dir) {
-    int s = eslot[0];
-#pragma unroll
-    for (int j = 1; j < 2 * D; ++j) if (j == dir) s = eslot[j];
-    return s;
 }
 
 // ---------------------------------------------------------------------------
@@ -279,23 +306,26 @@ constexpr int kStalledBit = 4;
 // that the walks' hashes, site lists and stacks are reached by shared-memory
 // instructions rather than generic ones (a generic load that lands in shared
 // memory waits longer, and in the long-scoreboard queue).
+template <int D> constexpr int kGroupLanes = D == 2 ? 4 : 8;   // lanes that hold one walk
+
 template <int D, typename Key, int MODE, bool SHARED>
 __device__ __forceinline__ void grow_run(const RunDev &P, unsigned char *smem, const BatchLeave *bl,
                                          int cta_walks) {
+    constexpr int G = kGroupLanes<D>;
     const int L = P.n_max + 1;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const bool snapshot = (MODE == kSnapshot);
     const int K = P.stack_cache;
 
     // The CTA's state: the head region (header, constant tables, snapshot of W_n)
-    // and one region per walk warp (occupancy hashes, site lists, stack rings).
-    // Both sit in shared memory, or, for walks too long for it, the walk regions
-    // (and, if even the head does not fit, the head too) in this CTA's slice of a
-    // global arena, served through L1 and L2.  Each walk's data is touched by its
-    // own thread only, so the same code runs on either.
-    const int ST = P.stride;
+    // and one region per walk (occupancy hash, site list, stack ring).  Both sit in
+    // shared memory, or, for walks too long for it, the walk regions (and, if even
+    // the head does not fit, the head too) in this CTA's slice of a global arena,
+    // served through L1 and L2.  A walk's data is touched by its own warp only, and
+    // the lanes of the warp order their accesses by __syncwarp(), so the same code
+    // runs on either.
     const size_t hbytes = head_region_bytes(P.n_max, snapshot);
-    const size_t wbytes = warp_region_bytes(P.n_max, P.log2h, K, sizeof(Key), ST);
+    const size_t wbytes = walk_region_bytes(P.n_max, P.log2h, K, sizeof(Key));
     unsigned char *hbase = smem, *wbase = smem + hbytes;
     if (!SHARED && P.arena_mode != kArenaNone) {
         unsigned char *a = P.arena + (size_t)blockIdx.x * (size_t)P.arena_cta_bytes;
@@ -304,20 +334,17 @@ __device__ __forceinline__ void grow_run(const RunDev &P, unsigned char *smem, c
     }
     CtaHead *head = reinterpret_cast<CtaHead *>(hbase);
     double *aoc = reinterpret_cast<double *>(hbase + 64);
-    unsigned char *p = hbase + 64 + 1024;
-    double *Wsnap = nullptr;
-    if (snapshot) {
-        Wsnap = reinterpret_cast<double *>(p); p += 8 * (size_t)L;
-    }
+    const uint32_t *lists = reinterpret_cast<const uint32_t *>(aoc + kFactors);
+    double *Wsnap = snapshot ? reinterpret_cast<double *>(hbase + 64 + 1024) : nullptr;
 
     // zero everything (empty hashes, empty stacks), then the constant tables
     for (size_t i = threadIdx.x; i < hbytes / 16; i += blockDim.x)
         reinterpret_cast<uint4 *>(hbase)[i] = make_uint4(0u, 0u, 0u, 0u);
-    for (size_t i = threadIdx.x; i < wbytes * P.worker_warps / 16; i += blockDim.x)
+    for (size_t i = threadIdx.x; i < wbytes * (size_t)(P.S * P.worker_warps) / 16; i += blockDim.x)
         reinterpret_cast<uint4 *>(wbase)[i] = make_uint4(0u, 0u, 0u, 0u);
     if (P.arena_mode != kArenaNone) __threadfence_block();
     __syncthreads();
-    fill_aoc(aoc, D, threadIdx.x, blockDim.x);
+    fill_constants(aoc, D, threadIdx.x, blockDim.x);
     const long long limit = P.tour_limit;
     if (snapshot) {
         unsigned long long Ms = *(volatile unsigned long long *)P.tickets;
@@ -410,35 +437,43 @@ __device__ __forceinline__ void grow_run(const RunDev &P, unsigned char *smem, c
     // ----------------------------------------------------------------------
     // worker warps
     // ----------------------------------------------------------------------
-    unsigned char *wb = wbase + wbytes * warp;
-    Key *hash = reinterpret_cast<Key *>(wb);
-    uint16_t *sites = reinterpret_cast<uint16_t *>(
-        wb + (((((size_t)1 << P.log2h) * ST * sizeof(Key)) + 15) & ~(size_t)15));
-    uint32_t *smeta = reinterpret_cast<uint32_t *>(reinterpret_cast<unsigned char *>(sites) +
-                                                   ((((size_t)P.n_max * ST * 2) + 15) & ~(size_t)15));
-    double *sw = reinterpret_cast<double *>(reinterpret_cast<unsigned char *>(smeta) +
-                                            ((((size_t)K * ST * 4) + 15) & ~(size_t)15));
-
+    const int grp = lane / G, j = lane % G, lead = lane - j;   // group, direction, the group's first lane
+    const bool first = j == 0;
+    const unsigned lt_mask = (1u << lead) - 1u;
     const int gwarp = blockIdx.x * P.worker_warps + warp;
-    const int slot = gwarp * P.S + lane;
-    const bool active = lane < P.S && slot < P.slots && warp * P.S + lane < cta_walks;
+    const int slot = gwarp * P.S + grp;
+    const bool active = grp < P.S && slot < P.slots && warp * P.S + grp < cta_walks;
     const int sidx = active ? slot : 0;
+    const size_t hash_b = walk_hash_bytes(P.log2h, sizeof(Key)), sites_b = walk_sites_bytes(P.n_max);
+    // (the lanes of a group without a walk read the warp's first one and write nothing)
+    unsigned char *warp_base = wbase + wbytes * (size_t)(warp * P.S);
+    unsigned char *wb = warp_base + wbytes * (size_t)(grp < P.S ? grp : 0);
+    Key *hash = reinterpret_cast<Key *>(wb);
+    uint16_t *sites = reinterpret_cast<uint16_t *>(wb + hash_b);
+    uint32_t *smeta = reinterpret_cast<uint32_t *>(wb + hash_b + sites_b);
+    double *sw = reinterpret_cast<double *>(wb + hash_b + sites_b + (size_t)K * 4);
+    const int log2b = P.log2h - Buckets<Key>::kLog2;
+    const Key origin = KeyCodec<D, Key>::encode(0, 0, 0);
+    const Key dkey = step_key<D, Key>(j < 2 * D ? j : 0);
+
     uint32_t *gmeta = P.gstk_meta + (size_t)sidx * P.n_max;
     double *gwt = P.gstk_w + (size_t)sidx * P.n_max;
-    const unsigned lt_mask = (1u << lane) - 1u;
     const Cutoffs cuts{P.cut, P.cut_copies, P.cut_q, P.cut_inv_q, P.cut_K};
-    const int dE_lo = (D == 2) ? 1 : 2;
-    (void)dE_lo;
+    const bool cutoffs = P.cut != nullptr;
 
+    // the walk's state: the same in every lane of its group
     int state = active ? kNeed : kDone;
-    int n = 0, cx = 0, cy = 0, cz = 0, maxn = 0;
+    int n = 0, maxn = 0;
+    Key cur = origin;          // key of the end-point
     double W = 1.0;
-    unsigned long long ordinal = 0ull, g = 0ull;
+    uint32_t ord = 0u;         // nodes of this part so far; a node's 64-bit ordinal is did 2^32 + ord
+    unsigned long long g = 0ull;
+    // the random blocks of the G nodes from ordinal pbase on: lane j holds the first two
+    // words of node pbase + j's (a block a pass for every lane would be G times the work)
+    uint32_t pbase = (uint32_t)-G, pw0 = 0u, pw1 = 0u;
     uint32_t seq = 0u, tour = 0u;
     int top = 0, sbase = 0;
     int un_lo = 0, un_hi = -1, pend_dir = 0, pend_depth = 0;
-    int back = -1;             // the direction from the end-point to the previous site (-1: empty walk)
-    bool tour_end = false;
     double pend_w = 0.0;
     unsigned long long my_steps = 0ull, my_copies = 0ull, my_exact = 0ull;
     int my_max_stack = 0;
@@ -459,43 +494,223 @@ __device__ __forceinline__ void grow_run(const RunDev &P, unsigned char *smem, c
     // no tour tickets left; a helper (of a batch, or a walk beyond the run's tour walks)
     // takes none and grows waiting copies only
     bool exhausted = (bl != nullptr && bl->helper) || sidx >= P.tour_slots;
-    int my_hungry = 0;         // lane 0: this warp's share of P.hungry
+    int my_hungry = 0;         // this warp's share of P.hungry
     unsigned idle_ns = 500u;   // back-off of a warp with nothing to grow
     int frow = 0, fmaxn = 0;   // tour-sum row to flush at a part's end, and its depth
     bool do_flush = false, shared_flush = false;
     const uint32_t dq_mask = (1u << P.dq_log2cap) - 1u;
-    // a hand-over made in this iteration's node passes, copied after them
-    int don_cell = -1, don_bdp = 0;
-    uint32_t don_round = 0u;
     // a donation cell: 32-byte header, the keys of sites 0..n_max, then their slots
     const size_t cell_key_bytes = align16(((size_t)P.n_max + 1) * sizeof(Key));
     unsigned long long my_iters = 0ull;
-    unsigned long long inv_of = 0ull;   // the snapshot M whose reciprocal inv_ms holds
-    double inv_ms = 0.0;
+    Tours tours;               // tours started as this walk's nodes see them
+    set_tours(tours, 1ull);
+    bool fresh_need = true;    // the walk has ended its tour since it last looked for work
     double *Wrow = P.Wn;
     unsigned long long *Srow = P.Sn;
     double *Rrow = P.Rn;
+    double *acc = Wrow;        // the row this lane adds a node's weight to (lane 0: W_n, lane 1: the tour's sums)
 
+    const bool extras = P.Rn != nullptr || P.cut != nullptr;
     const long long t_start = global_ns();
-    for (long long iter = 0;; ++iter) {
-        const bool late = (iter & 255) == 0 && global_ns() - t_start > P.max_ns;
-        if (__any_sync(kFull, late)) {
-            if (lane == 0) set_status(P.status, PERM_ETIMEOUT);
-            break;
+    for (uint32_t iter = 0u;; ++iter) {
+        if ((iter & 7u) == 0u) {
+        if ((iter & 255u) == 0u) {
+            const bool late = global_ns() - t_start > P.max_ns;
+            if (__any_sync(kFull, late)) {
+                if (lane == 0) set_status(P.status, PERM_ETIMEOUT);
+                break;
+            }
+            // in a batch launch a failed run stops at once, so that its CTAs move on
+            // (the whole warp leaves together: one lane's read decides)
+            if (bl != nullptr && __shfl_sync(kFull, *(volatile int *)P.status, 0) != 0) break;
         }
-        // in a batch launch a failed run stops at once, so that its CTAs move on
-        // (the whole warp leaves together: one lane's read decides)
-        if (bl != nullptr && (iter & 255) == 0 && __shfl_sync(kFull, *(volatile int *)P.status, 0) != 0) break;
-        // ---------------- tour tickets ----------------
-        if (state == kNeed && xbusy) {
-            if (*(volatile unsigned int *)(P.outst + myrow) == kRowFree) xbusy = false;
-            else if (rows_per_walk == 2 && *(volatile unsigned int *)(P.outst + (myrow ^ 1)) == kRowFree) {
-                myrow ^= 1;
-                xbusy = false;
+        // ---------------- hand-overs: waiting copies for idle walks ----------------
+        // A walk with two waiting records or more hands its oldest one to an idle walk:
+        // that subtree grows there, and its weights still go to this tour's row `own`.
+        // Its first lane decides and writes the cell's header; the whole warp copies the
+        // sites 0..bdp with the slot that an in-order rebuild would give each, so the
+        // taker places them without probing.
+        // (looked at every eighth iteration)
+        if (snapshot && P.share && __shfl_sync(kFull, *(volatile int *)&head->want_don, 0) > 0) {
+            // at most P.share parts of one tour grow at once (a soft cap: the parts of a
+            // tour stay few, so each still sees its siblings' samples)
+            bool can = first && state == kNode && top - bot >= 2;
+            if (can && !(did == 0u && !donated))
+                can = *(volatile unsigned int *)(P.outst + own) < (unsigned)*(volatile int *)&head->cap;
+            unsigned dm = __ballot_sync(kFull, can);
+            while (dm) {
+                const int src = __ffs(dm) - 1;
+                dm &= dm - 1u;
+                int cell = -1, bdp = 0;
+                uint32_t round = 0u;
+                if (lane == src) {
+                    const int bi = bot & (K - 1);
+                    const uint32_t bm = bot < sbase ? __ldcg(gmeta + bot) : smeta[bi];
+                    const double bw = bot < sbase ? __ldcg(gwt + bot) : sw[bi];
+                    bdp = (int)(bm & 0xFFFFu);
+                    if (P.n_max - bdp >= kMinShareGap && atomicSub(&head->want_don, 1) > 0) {
+                        unsigned long long pos = 0ull;
+                        bool got = false;
+                        for (int attempt = 0; attempt < 8; ++attempt) {
+                            const unsigned long long t0 = *(volatile unsigned long long *)P.dq_tail;
+                            const uint32_t c0 = (uint32_t)t0 & dq_mask;
+                            if (*(volatile unsigned int *)(P.dq_free + c0) != (uint32_t)(t0 >> P.dq_log2cap)) break;
+                            if (atomicCAS(P.dq_tail, t0, t0 + 1ull) == t0) { pos = t0; got = true; break; }
+                        }
+                        if (got) {
+                            if (did == 0u && !donated) P.outst[own] = 2u;
+                            else atomicAdd(P.outst + own, 1u);
+                            cell = (int)((uint32_t)pos & dq_mask);
+                            round = (uint32_t)(pos >> P.dq_log2cap);
+                            unsigned char *cb = P.dq_cells + (size_t)cell * (size_t)P.dq_cell_bytes;
+                            *reinterpret_cast<uint4 *>(cb) = make_uint4((uint32_t)own, seq, tour, (uint32_t)bdp);
+                            *reinterpret_cast<uint2 *>(cb + 16) = make_uint2(bm, 0u);
+                            *reinterpret_cast<double *>(cb + 24) = bw;
+                        } else {
+                            atomicAdd(&head->want_don, 1);
+                        }
+                    }
+                }
+                cell = __shfl_sync(kFull, cell, src);
+                if (cell < 0) continue;
+                bdp = __shfl_sync(kFull, bdp, src);
+                unsigned char *cb = P.dq_cells + (size_t)cell * (size_t)P.dq_cell_bytes;
+                unsigned char *sb = warp_base + wbytes * (size_t)(src / G);
+                copy_sites_to_cell<Key>(reinterpret_cast<const Key *>(sb), reinterpret_cast<const uint16_t *>(sb + hash_b),
+                                        bdp, reinterpret_cast<Key *>(cb + 32),
+                                        reinterpret_cast<uint16_t *>(cb + 32 + cell_key_bytes), lane);
+                __threadfence();
+                __syncwarp();
+                if (lane == src) *(volatile unsigned int *)(P.dq_ready + cell) = round + 1u;
+                if (lead == src) {
+                    if (did == 0u) donated = true;
+                    bot += 1;
+                    if (sbase < bot) sbase = bot;
+                }
+            }
+        }
+        }
+        // ---------------- walks that ended their tour, or have none ----------------
+        // (looked after at once when a tour has ended; a walk that then found nothing to
+        // grow looks again every eighth iteration: the reads and atomics take several
+        // round trips to L2, which the warp's other walks wait for)
+        if (__any_sync(kFull, state == kFlush || (state == kNeed && (fresh_need || (iter & 7u) == 0u)))) {
+        // ---------------- end of a tour (part): per-tour sums into Q (whole warp) ----------------
+        if (__any_sync(kFull, state == kFlush)) {
+            const bool fl = state == kFlush, whole = did == 0u && !donated;
+            // empty the ended walks' hashes, the whole warp one walk at a time: every
+            // bucket, or, of a short walk, its sites' slots
+            unsigned em = __ballot_sync(kFull, fl && first);
+            while (em) {
+                const int src = __ffs(em) - 1;
+                em &= em - 1u;
+                const int hi = __shfl_sync(kFull, un_hi, src);
+                unsigned char *hb = warp_base + wbytes * (size_t)(src / G);
+                const int vecs = (int)(hash_b / 16);
+                if (vecs <= 2 * (hi + 1)) {
+                    for (int i = lane; i < vecs; i += 32) reinterpret_cast<uint4 *>(hb)[i] = make_uint4(0u, 0u, 0u, 0u);
+                } else {
+                    const uint16_t *st = reinterpret_cast<const uint16_t *>(hb + hash_b);
+                    for (int i = lane; i <= hi; i += 32) reinterpret_cast<Key *>(hb)[st[i]] = (Key)0;
+                }
+            }
+            if (fl) my_steps += ord;
+            // the sums of a tour whose parts grew on several walks: this part's must be in
+            // the row before the count of its parts says so (a tour that stayed on this
+            // walk needs the warp's own order only)
+            if (__any_sync(kFull, fl && !whole)) __threadfence();
+            __syncwarp();
+            unsigned om = 0u, left = 0u;
+            if (fl && !whole && first) {
+                // parts of the tour grew elsewhere: the last part to end flushes
+                om = atomicMax(P.tmaxn + own, (unsigned)maxn);
+                __threadfence();
+                left = atomicSub(P.outst + own, 1u);
+                __threadfence();
+            }
+            __syncwarp();
+            om = __shfl_sync(kFull, om, lead);
+            left = __shfl_sync(kFull, left, lead);
+            bool other_row = false;
+            if (fl) {
+                frow = own;
+                shared_flush = !whole;
+                do_flush = whole || left == 1u;
+                fmaxn = whole ? maxn : (int)(om > (unsigned)maxn ? om : (unsigned)maxn);
+                // the row stays with the parts still growing: the next tour takes the
+                // walk's other row, if that one is free
+                other_row = !do_flush && did == 0u;
+                if (other_row) myrow ^= rows_per_walk - 1;
+            }
+            unsigned row_use = kRowFree;
+            if (other_row && first) row_use = *(volatile unsigned int *)(P.outst + myrow);
+            row_use = __shfl_sync(kFull, row_use, lead);
+            if (other_row) xbusy = row_use != kRowFree;
+            unsigned flm = __ballot_sync(kFull, fl && do_flush && first);
+            while (flm) {
+                const int src = __ffs(flm) - 1;
+                flm &= flm - 1u;
+                const int s_slot = __shfl_sync(kFull, frow, src);
+                const int s_maxn = __shfl_sync(kFull, fmaxn, src);
+                const int s_seq = __shfl_sync(kFull, cur_seq, src);
+                double *Xr = P.X + (size_t)s_slot * L;
+                double *Qr = (P.alg == PERM_ALG1) ? P.Qn + (size_t)(s_seq < 0 ? 0 : s_seq) * L : P.Qn;
+                // eight loads in flight per lane, then the squares go straight to Q_n
+                for (int k0 = 0; k0 <= s_maxn; k0 += 32 * 8) {
+                    double x[8];
+#pragma unroll
+                    for (int u = 0; u < 8; ++u) {
+                        const int k = k0 + u * 32 + lane;
+                        x[u] = (k <= s_maxn) ? __ldcg(Xr + k) : 0.0;
+                    }
+#pragma unroll
+                    for (int u = 0; u < 8; ++u) {
+                        const int k = k0 + u * 32 + lane;
+                        if (__double_as_longlong(x[u]) != 0ll) {     // (an integer test: no -0.0 here)
+                            atomicAdd(&Qr[k], __dmul_rn(x[u], x[u]));
+                            __stcg(Xr + k, 0.0);
+                        }
+                    }
+                }
+            }
+            __syncwarp();
+            if (fl) {
+                if (do_flush) {
+                    if (first) {
+                        if (shared_flush) {
+                            P.tmaxn[frow] = 0u;
+                            __threadfence();       // (after the barrier above: the emptied row too)
+                            *(volatile unsigned int *)(P.outst + frow) = kRowFree;
+                        }
+                        atomicAdd(P.finished, 1ull);
+                    }
+                    if (P.alg == PERM_ALG1) {
+                        seq_t += 1;
+                        if (first) P.seq_M[cur_seq] = (unsigned long long)seq_t;
+                    }
+                }
+                own = myrow; did = 0u; donated = false; do_flush = false;
+                state = kNeed;
+            }
+            fresh_need = true;
+        }
+        fresh_need = false;
+        const bool blocked = state == kNeed && xbusy;
+        if (__any_sync(kFull, blocked)) {
+            unsigned r0 = 0u, r1 = 0u;
+            if (blocked && first) {
+                r0 = *(volatile unsigned int *)(P.outst + myrow);
+                if (rows_per_walk == 2) r1 = *(volatile unsigned int *)(P.outst + (myrow ^ 1));
+            }
+            r0 = __shfl_sync(kFull, r0, lead);
+            r1 = __shfl_sync(kFull, r1, lead);
+            if (blocked) {
+                if (r0 == kRowFree) xbusy = false;
+                else if (r1 == kRowFree) { myrow ^= 1; xbusy = false; }
             }
         }
         const bool want_t = state == kNeed && !xbusy && !exhausted;
-        const unsigned need = __ballot_sync(kFull, want_t);
+        const unsigned need = __ballot_sync(kFull, want_t && first);
         if (need) {
             if (P.alg == PERM_ALG2) {
                 const unsigned cnt = __popc(need);
@@ -552,17 +767,25 @@ __device__ __forceinline__ void grow_run(const RunDev &P, unsigned char *smem, c
                     if ((long long)g >= limit) {
                         if (P.share) exhausted = true;   // idle: may still take shared copies
                         else state = kDone;
-                        if (bl != nullptr && (atomicOr(bl->closed + P.run_index, 1) & 3) == 0)
+                        if (bl != nullptr && first && (atomicOr(bl->closed + P.run_index, 1) & 3) == 0)
                             atomicSub(bl->runs_open, 1);
                     } else {
-                        seq = (uint32_t)(g % (unsigned long long)P.n_seq);
-                        tour = (uint32_t)(g / (unsigned long long)P.n_seq);
+                        if ((g >> 32) == 0ull) {           // (a 64-bit division takes several times as long)
+                            tour = (uint32_t)g / (uint32_t)P.n_seq;
+                            seq = (uint32_t)g - tour * (uint32_t)P.n_seq;
+                        } else {
+                            seq = (uint32_t)(g % (unsigned long long)P.n_seq);
+                            tour = (uint32_t)(g / (unsigned long long)P.n_seq);
+                        }
                     }
                 }
-            } else if (state == kNeed) {
+            } else {
                 // Algorithm 1: a walk owns a sequence until its tours are done
-                if (cur_seq < 0 || seq_t >= P.seq_target) {
-                    const unsigned long long s = atomicAdd(P.tickets, 1ull);
+                const bool ask = state == kNeed && (cur_seq < 0 || seq_t >= P.seq_target);
+                unsigned long long s = 0ull;
+                if (ask && first) s = atomicAdd(P.tickets, 1ull);
+                s = __shfl_sync(kFull, s, lead);
+                if (ask) {
                     if (s >= (unsigned long long)P.n_seq) {
                         state = kDone;
                     } else {
@@ -582,20 +805,24 @@ __device__ __forceinline__ void grow_run(const RunDev &P, unsigned char *smem, c
                 }
             }
             if (state == kNeed && !waiting && !xbusy && !exhausted && (P.alg == PERM_ALG2 || cur_seq >= 0)) {
-                // start a tour at the empty walk (Sec. 1: W(empty) = 1)
-                n = 0; cx = cy = cz = 0; maxn = 0; W = 1.0; ordinal = 0ull; back = -1;
+                // start a tour at the empty walk (Sec. 1: W(empty) = 1); the walk's hash
+                // is empty, so the origin takes the first place of its home bucket
+                n = 0; cur = origin; maxn = 0; W = 1.0; ord = 0u; pbase = (uint32_t)-G;
                 top = 0; sbase = 0; bot = 0;
                 own = myrow; did = 0u; donated = false;
-                const int s0 = hash_insert<Key>(hash, ST, lane, P.log2h,
-                                                KeyCodec<D, Key>::encode(0, 0, 0));
-                if (s0 < 0) { set_status(P.status, PERM_EOVERFLOW); state = kDone; }
-                else { sites[lane] = (uint16_t)s0; state = kNode; }
+                acc = first ? Wrow : P.X + (size_t)own * L;
+                if (first) {
+                    const uint32_t s0 = hash_home(origin, log2b) * (uint32_t)Buckets<Key>::kKeys;
+                    hash[s0] = origin;
+                    sites[0] = (uint16_t)s0;
+                }
+                state = kNode;
             }
         }
         if (P.share) {
             // ---------------- shared copies: idle walks take queued ones ----------------
             const bool idle = state == kNeed && (waiting || xbusy || exhausted);
-            const unsigned hm = __ballot_sync(kFull, idle);
+            const unsigned hm = __ballot_sync(kFull, idle && first);
             // one lane's read of the queue length decides for the warp (the block
             // below exchanges values across all lanes)
             if (hm && __shfl_sync(kFull, *(volatile int *)&head->queued, 0) > 0) {
@@ -615,24 +842,26 @@ __device__ __forceinline__ void grow_run(const RunDev &P, unsigned char *smem, c
                 take = __shfl_sync(kFull, take, leader);
                 const unsigned rk = __popc(hm & lt_mask);
                 bool claiming = idle && rk < take;
-                unsigned long long pos = 0ull;
-                uint32_t cell = 0u, round = 0u;
+                const unsigned long long pos = base + rk;
+                const uint32_t cell = (uint32_t)pos & dq_mask;
+                const uint32_t round = (uint32_t)(pos >> P.dq_log2cap);
                 int cdp = -1;
-                if (claiming) {
-                    pos = base + rk;
-                    cell = (uint32_t)pos & dq_mask;
-                    round = (uint32_t)(pos >> P.dq_log2cap);
-                    bool ok = false;
+                bool ok = false;
+                if (claiming && first) {
                     for (int spin = 0; spin < kCellSpin; ++spin) {
                         if (*(volatile unsigned int *)(P.dq_ready + cell) == round + 1u) { ok = true; break; }
                         __nanosleep(32);
                     }
+                    __threadfence();
+                }
+                __syncwarp();
+                ok = __shfl_sync(kFull, (int)ok, lead) != 0;
+                if (claiming) {
                     if (!ok || pos + 1ull >= (1ull << 32)) {
                         set_status(P.status, ok ? PERM_EOVERFLOW : PERM_ETIMEOUT);
                         state = kDone;
                         claiming = false;
                     } else {
-                        __threadfence();
                         cdp = (int)__ldcg(reinterpret_cast<const unsigned int *>(P.dq_cells + (size_t)cell *
                                                                                 (size_t)P.dq_cell_bytes) + 3);
                     }
@@ -640,7 +869,7 @@ __device__ __forceinline__ void grow_run(const RunDev &P, unsigned char *smem, c
                 // the walk up to the branch point (Sec. 1), each site straight into the
                 // slot it had in the donor's hash; the whole warp places one taker's
                 // sites at a time (the taker's hash is empty: it had no walk)
-                unsigned cm = __ballot_sync(kFull, claiming);
+                unsigned cm = __ballot_sync(kFull, claiming && first);
                 while (cm) {
                     const int src = __ffs(cm) - 1;
                     cm &= cm - 1u;
@@ -649,9 +878,10 @@ __device__ __forceinline__ void grow_run(const RunDev &P, unsigned char *smem, c
                     const unsigned char *cb = P.dq_cells + (size_t)scell * (size_t)P.dq_cell_bytes;
                     const Key *ck = reinterpret_cast<const Key *>(cb + 32);
                     const uint16_t *cs = reinterpret_cast<const uint16_t *>(cb + 32 + cell_key_bytes);
-                    place_sites_from_cell<Key>(hash, sites, ST, src, sdp, ck, cs, lane);
+                    unsigned char *tb = warp_base + wbytes * (size_t)(src / G);
+                    place_sites_from_cell<Key>(reinterpret_cast<Key *>(tb), reinterpret_cast<uint16_t *>(tb + hash_b),
+                                               sdp, ck, cs, lane);
                 }
-                __syncwarp();
                 if (claiming) {
                     const unsigned char *cb = P.dq_cells + (size_t)cell * (size_t)P.dq_cell_bytes;
                     const uint4 h0 = __ldcg(reinterpret_cast<const uint4 *>(cb));
@@ -659,382 +889,304 @@ __device__ __forceinline__ void grow_run(const RunDev &P, unsigned char *smem, c
                     const double cw = __longlong_as_double(__ldcg(reinterpret_cast<const long long *>(cb + 24)));
                     const int dp = (int)h0.w;
                     const uint32_t meta = h1.x;
-                    __threadfence();
-                    *(volatile unsigned int *)(P.dq_free + cell) = round + 1u;
                     own = (int)h0.x; seq = h0.y; tour = h0.z;
                     g = (unsigned long long)tour * (unsigned long long)P.n_seq + seq;
                     did = (uint32_t)(pos + 1ull);
-                    ordinal = (unsigned long long)did << 32;
+                    ord = 0u; pbase = (uint32_t)-G;
                     donated = false; maxn = 0;
                     top = 0; sbase = 0; bot = 0;
+                    acc = first ? Wrow : P.X + (size_t)own * L;
                     const int cnt = (int)((meta >> 16) & 7u);
                     const uint32_t dirs = meta >> 19;
                     pend_dir = (int)(dirs & 7u);
                     pend_w = cw;
                     pend_depth = dp;
                     if (cnt > 1) {
-                        smeta[lane] = (uint32_t)dp | ((uint32_t)(cnt - 1) << 16) | ((dirs >> 3) << 19);
-                        sw[lane] = cw;
+                        if (first) {
+                            smeta[0] = (uint32_t)dp | ((uint32_t)(cnt - 1) << 16) | ((dirs >> 3) << 19);
+                            sw[0] = cw;
+                        }
                         top = 1;
                     }
-                    un_lo = dp + 1; un_hi = dp; tour_end = false;
+                    un_lo = dp + 1; un_hi = dp;
                     waiting = false;
                     state = kUnwindState;      // resumes at the branch point below
                 }
+                // every lane has read the cells: they may be written again
+                __threadfence();
+                __syncwarp();
+                if (claiming && first) *(volatile unsigned int *)(P.dq_free + cell) = round + 1u;
             }
-            const int hcount = __popc(__ballot_sync(kFull, state == kNeed && (waiting || xbusy || exhausted)));
-            if (lane == 0 && hcount != my_hungry) {
-                atomicAdd(P.hungry, hcount - my_hungry);
+            const int hcount = __popc(__ballot_sync(kFull, first && state == kNeed && (waiting || xbusy || exhausted)));
+            if (hcount != my_hungry) {
+                if (lane == 0) atomicAdd(P.hungry, hcount - my_hungry);
                 my_hungry = hcount;
             }
             // walks with no tickets left stop once every tour of the launch has
-            // finished (or the run has failed)
-            if (state == kNeed && exhausted &&
-                ((long long)*(volatile unsigned long long *)&head->fin >= limit || *(volatile int *)&head->status != 0 ||
-                 (!xbusy && *(volatile int *)&head->may_leave != 0)))
-                state = kDone;
+            // finished (or the run has failed); one lane's reads decide
+            const bool over = (long long)*(volatile unsigned long long *)&head->fin >= limit ||
+                              *(volatile int *)&head->status != 0;
+            const bool leave = *(volatile int *)&head->may_leave != 0;
+            const int go = __shfl_sync(kFull, (over ? 1 : 0) | (leave ? 2 : 0), 0);
+            if (state == kNeed && exhausted && ((go & 1) || (!xbusy && (go & 2)))) state = kDone;
         }
-        const unsigned live = __ballot_sync(kFull, state != kDone);
-        if (!live) break;
-        ++my_iters;
-        if (__all_sync(kFull, state == kDone || (state == kNeed && (waiting || xbusy || exhausted)))) {
+        }
+        if (!__any_sync(kFull, state == kNode || state == kUnwindState)) {
+            // nothing to grow: the warp backs off, or leaves
+            if (!__any_sync(kFull, state != kDone)) break;
             __nanosleep(idle_ns);
             idle_ns = idle_ns < 4000u ? 2u * idle_ns : 4000u;
-        } else {
-            idle_ns = 500u;
+            fresh_need = true;
+            ++my_iters;
+            continue;
         }
+        ++my_iters;
 
-        // ---------------- nodes: up to kNodePasses per iteration ----------------
-        // A walk whose node made children grows its next node in the same
-        // iteration, so that the warp-wide parts of the loop are shared by more
-        // nodes; a walk that reached a leaf waits for the backtrack below.
-        for (int pass = 0; pass < kNodePasses; ++pass) {
-        if (pass > 0 && !__any_sync(kFull, state == kNode)) break;
-        // the snapshot's M for this pass, and its reciprocal (taken by the whole warp
-        // once per new snapshot: double-precision arithmetic is slow on this part)
-        unsigned long long Ms_p = 0ull;
-        if (snapshot) {
-            Ms_p = __shfl_sync(kFull, *(volatile unsigned long long *)&head->Ms, 0);
-            if (Ms_p != inv_of) { inv_of = Ms_p; inv_ms = __drcp_rn(__ull2double_rn(Ms_p)); }
-        }
-        if (state == kNode) {
-            // the sum of the weights recorded at this length before the node (a
-            // snapshot, or the global table's value returned by the node's own add)
-            // and the tours started, this one included
-            double Wsum;
-            unsigned long long Mb;
+        // ---------------- one node of every walk that has one ----------------
+        // One straight line with few branches, each of them for something rare: on this
+        // part a lone warp pays 25 cycles or more for a branch, taken or not, 45 for a vote
+        // and a branch on it.
+        {
+            __syncwarp();                       // the walks' hashes as the last iteration left them
+            // (two loads of the whole warp right after the barrier, one instruction each: the
+            // lanes of a group read the same value while the refresher writes)
+            unsigned long long Mn = g + 1ull;
+            double Wsum = 0.0;
+            const bool isn = state == kNode;
             if (snapshot) {
-                // fire-and-forget reductions into the global table (no value comes back)
-                atomicAdd(P.Wn + n, W);
-                atomicAdd(P.Sn + n, 1ull);
+                const unsigned long long Ms = *(volatile unsigned long long *)&head->Ms;
                 Wsum = *(volatile double *)&Wsnap[n];
-                Mb = Ms_p > g + 1ull ? Ms_p : g + 1ull;
+                Mn = Ms > Mn ? Ms : Mn;
+            }
+            const bool grows_on = isn && n < P.n_max;
+            // a_+ (Sec. 1): lane j of the group probes neighbour j
+            const bool probes = grows_on && j < 2 * D;
+            const Key nkey = cur + dkey;
+            uint32_t bucket = hash_home(nkey, log2b);
+            bool hit, full;
+            int place;
+            look_bucket(hash, bucket, nkey, hit, full, place);
+            // the node's weight goes into the tables with reductions that return nothing, one
+            // lane each (fresh form: the W_n one returns the sum before it)
+            if (snapshot) {
+                red_add(acc + n, W, isn && j < 2);
             } else {
-                Wsum = atomicAdd(&Wrow[n], W);
-                atomicAdd(&Srow[n], 1ull);
+                double before = 0.0;
+                unsigned long long Mt = 0ull;
+                if (isn && first) {
+                    before = atomicAdd(&Wrow[n], W);
+                    if (P.alg == PERM_ALG2) Mt = *(volatile unsigned long long *)P.tickets;
+                }
+                red_add(acc + n, W, isn && j == 1);
+                Wsum = __shfl_sync(kFull, before, lead);
                 if (P.alg == PERM_ALG2) {
-                    unsigned long long Mt = *(volatile unsigned long long *)P.tickets;
+                    Mt = __shfl_sync(kFull, Mt, lead);
                     if ((long long)Mt > limit) Mt = (unsigned long long)limit;
-                    Mb = Mt > g + 1ull ? Mt : g + 1ull;
-                } else {
-                    Mb = (unsigned long long)seq_t + 1ull;
+                    Mn = Mt > Mn ? Mt : Mn;
                 }
             }
-            atomicAdd(P.X + (size_t)own * L + n, W);
-            if (P.Rn != nullptr) {
-                // the observable of Sec. 1, eq. 5: W |omega_n|^2 (exact integer square)
-                const long long r2 = (long long)cx * cx + (long long)cy * cy + (long long)cz * cz;
-                atomicAdd(Rrow + n, __dmul_rn(W, (double)r2));
+            red_inc(Srow + n, isn && j == 2);
+            maxn = (isn && n > maxn) ? n : maxn;
+            // a full bucket without the key, a used-up block of random words, a new M: one
+            // vote for the three
+            bool more = probes && full && !hit;
+            if (__any_sync(kFull, isn && (more || ord - pbase >= (uint32_t)G || Mn != tours.M))) {
+                if (isn && Mn != tours.M) set_tours(tours, Mn);
+                if (__any_sync(kFull, isn && ord - pbase >= (uint32_t)G)) {
+                    pbase = ord;
+                    if (isn && ord >= 0xFFFFFFF0u) set_status(P.status, PERM_EOVERFLOW);
+                    const Philox4 w = philox4x32_10(ord + (uint32_t)j, did, tour, seq, P.key0, P.key1);
+                    pw0 = w.x; pw1 = w.y;
+                }
+                const uint32_t bmask = (1u << log2b) - 1u;
+                for (uint32_t it = 0u; __any_sync(kFull, more); ++it) {
+                    if (it >= bmask) { if (more) set_status(P.status, PERM_EOVERFLOW); break; }
+                    if (more) {
+                        bucket = (bucket + it + 1u) & bmask;
+                        look_bucket(hash, bucket, nkey, hit, full, place);
+                        more = full && !hit;
+                    }
+                }
             }
-            maxn = n > maxn ? n : maxn;
-            ++my_steps;
+            const bool free_j = probes && !hit && !full;
+            const int nslot = (int)(bucket * (uint32_t)Buckets<Key>::kKeys) + place;
+            const int fm = (int)((__ballot_sync(kFull, free_j) >> lead) & ((1u << G) - 1u));
+            const int a = __popc(fm), a1 = a > 0 ? a : 1;
+            const bool decides = grows_on && a > 0;
+            // the node's random words, from the lane that holds its block
+            const int wl = lead + (int)((ord - pbase) & (uint32_t)(G - 1));
+            const uint32_t w0 = __shfl_sync(kFull, pw0, wl), w1 = __shfl_sync(kFull, pw1, wl);
+            Decision o = decide_node<D>(n, a1, W, Wsum, tours, !snapshot, w0, aoc, decides && !cutoffs, false);
+            if (extras) {
+                if (cutoffs && n > 0) o = decide_cutoffs<D>(n, a1, W, w0, aoc, cuts);
+                if (P.Rn != nullptr) {
+                    // the observable of Sec. 1, eq. 5: W |omega_n|^2 (exact integer square)
+                    int cx, cy, cz;
+                    KeyCodec<D, Key>::decode(cur, cx, cy, cz);
+                    const long long r2 = (long long)cx * cx + (long long)cy * cy + (long long)cz * cz;
+                    red_add(Rrow + n, __dmul_rn(W, (double)r2), isn && j == 3);
+                }
+            }
+            const int c = decides ? o.c : 0;
+            if (o.exact && decides) my_exact += 1ull;
+            // the first child's step, its key and its place in the hash, from the lane that probed it
+            uint32_t list = lists[fm], xw = w1;
+            choose_step(0, a1, list, xw);
+            const int dir0 = (int)(list & 7u);
+            const Key ckey = __shfl_sync(kFull, nkey, lead + dir0);
+            const int cslot = __shfl_sync(kFull, nslot, lead + dir0);
+            if (c > 1)
+                for (int i = 1; i < c; ++i) choose_step(i, a, list, xw);
+            const uint32_t dirs = list;
 
-            int eslot[2 * D];
-#pragma unroll
-            for (int j = 0; j < 2 * D; ++j) eslot[j] = 0;
-            const NodeOut o = grow_node<D, Key>(hash, ST, lane, P.log2h, n, P.n_max, cx, cy, cz, W, Wsum,
-                                                Mb, ordinal, seq, tour, P.key0, P.key1, aoc, eslot, cuts,
-                                                (snapshot && Mb == Ms_p) ? inv_ms : 0.0, back);
-            if (o.overflow) set_status(P.status, PERM_EOVERFLOW);
-            my_exact += o.exact ? 1ull : 0ull;
-
-            if (P.trace != nullptr && (ordinal % (unsigned long long)P.trace_every) == 0ull &&
+            const unsigned long long ordinal = ((unsigned long long)did << 32) | ord;
+            if (P.trace != nullptr && isn && first && (ordinal % (unsigned long long)P.trace_every) == 0ull &&
                 ((unsigned long long)tour % (unsigned long long)P.trace_tour_every) == 0ull) {
                 const unsigned long long idx = atomicAdd(P.trace_count, 1ull);
                 if (idx < (unsigned long long)P.trace_cap) {
                     perm_trace_record *rec = P.trace + idx;
-                    rec->n = n; rec->a_plus = o.a; rec->free_mask = o.mask; rec->c = o.c;
-                    rec->outcome = o.outcome; rec->exact = o.exact ? 1 : 0;
+                    rec->n = n; rec->a_plus = a; rec->free_mask = fm; rec->c = c;
+                    rec->outcome = !grows_on ? kLeafNmax : (a == 0 ? kTrapped : (c == 0 ? kPruned : kChildren));
+                    rec->exact = decides && o.exact ? 1 : 0;
                     for (int i = 0; i < 6; ++i)
-                        rec->dirs[i] = (i < o.c) ? (int)((o.dirs >> (3 * i)) & 7u) : -1;
+                        rec->dirs[i] = (i < c) ? (int)((dirs >> (3 * i)) & 7u) : -1;
                     rec->seq = seq; rec->tour = tour;
-                    rec->ordinal = ordinal; rec->M = Mb;
-                    rec->W = W; rec->Wsum = Wsum; rec->r = o.r; rec->child_w = o.child_w;
+                    rec->ordinal = ordinal; rec->M = tours.M;
+                    rec->W = W; rec->Wsum = Wsum; rec->r = o.r; rec->child_w = c > 0 ? o.child_w : 0.0;
                     int32_t *cc = P.trace_coords + (size_t)idx * L * D;
-                    for (int k = 0; k < n; ++k) {
+                    for (int k = 0; k <= n; ++k) {
                         int x, y, z;
-                        KeyCodec<D, Key>::decode(hash[(uint32_t)sites[(uint32_t)k * ST + lane] * ST + lane], x, y, z);
+                        KeyCodec<D, Key>::decode(k < n ? hash[sites[k]] : cur, x, y, z);
                         cc[k * D] = x; cc[k * D + 1] = y;
                         if (D == 3) cc[k * D + 2] = z;
                     }
-                    cc[n * D] = cx; cc[n * D + 1] = cy;
-                    if (D == 3) cc[n * D + 2] = cz;
                 }
             }
 
-            if ((uint32_t)ordinal == 0xFFFFFFFFu) set_status(P.status, PERM_EOVERFLOW);
-            ordinal += 1ull;
-            if (o.outcome == kChildren) {
-                const int c = o.c;
+            if (c > 1) {
+                // copies 1..c-1 wait in one record (depth, count, steps, weight)
+                const unsigned gmask = ((1u << G) - 1u) << lead;
                 my_copies += (unsigned long long)(c - 1);
-                if (c > 1) {
-                    // copies 1..c-1 wait in one record (depth, count, steps, weight)
-                    if (top - sbase == K) {
-                        // ring full: the oldest kChunk records go to global memory
+                if (top - sbase == K) {
+                    // ring full: the oldest kChunk records go to global memory
 #pragma unroll
-                        for (int i = 0; i < kChunk; ++i) {
-                            const int idx = sbase + i;
-                            gmeta[idx] = smeta[(uint32_t)(idx & (K - 1)) * ST + lane];
-                            gwt[idx] = sw[(uint32_t)(idx & (K - 1)) * ST + lane];
-                        }
-                        sbase += kChunk;
+                    for (int i = 0; i < kChunk; i += G) {
+                        const int idx = sbase + i + j;
+                        gmeta[idx] = smeta[idx & (K - 1)];
+                        gwt[idx] = sw[idx & (K - 1)];
                     }
-                    if (top >= P.n_max) {
-                        set_status(P.status, PERM_EOVERFLOW);
-                    } else {
-                        const uint32_t rest = (o.dirs >> 3) & ((1u << (3 * (c - 1))) - 1u);
+                    sbase += kChunk;
+                    __syncwarp(gmask);
+                }
+                if (top >= P.n_max) {
+                    set_status(P.status, PERM_EOVERFLOW);
+                } else {
+                    if (first) {
+                        const uint32_t rest = (dirs >> 3) & ((1u << (3 * (c - 1))) - 1u);
                         const int ti = top & (K - 1);
-                        smeta[(uint32_t)ti * ST + lane] = (uint32_t)n | ((uint32_t)(c - 1) << 16) | (rest << 19);
-                        sw[(uint32_t)ti * ST + lane] = o.child_w;
-                        ++top;
-                        my_max_stack = top - bot > my_max_stack ? top - bot : my_max_stack;
+                        smeta[ti] = (uint32_t)n | ((uint32_t)(c - 1) << 16) | (rest << 19);
+                        sw[ti] = o.child_w;
                     }
+                    ++top;
+                    my_max_stack = top - bot > my_max_stack ? top - bot : my_max_stack;
                 }
-                const int dir0 = (int)(o.dirs & 7u);
-                const int s0 = select_slot<D>(eslot, dir0);
-                step_coords(dir0, cx, cy, cz);
-                back = dir0 ^ 1;
-                n += 1;
-                if (n < P.n_max) {
-                    hash[(uint32_t)s0 * ST + lane] = KeyCodec<D, Key>::encode(cx, cy, cz);
-                    sites[(uint32_t)n * ST + lane] = (uint16_t)s0;
-                }
-                W = o.child_w;
-                if (snapshot && P.share && don_cell < 0 && top - bot >= 2 && *(volatile int *)&head->want_don > 0) {
-                    // hand the oldest waiting copy record to an idle walk: its subtree
-                    // grows there, and its weights still go to this tour's row `own`.
-                    // The header is written now; the walk's sites 0..bdp go into the
-                    // cell after the node passes, copied by the whole warp
-                    const uint32_t bi = (uint32_t)(bot & (K - 1)) * ST + lane;
-                    const uint32_t bm = bot < sbase ? gmeta[bot] : smeta[bi];
-                    const double bw = bot < sbase ? gwt[bot] : sw[bi];
-                    const int bdp = (int)(bm & 0xFFFFu);
-                    // at most P.share parts of one tour grow at once (a soft cap: the
-                    // parts of a tour stay few, so each still sees its siblings' samples)
-                    bool room = true;
-                    if (!(did == 0u && !donated))
-                        room = *(volatile unsigned int *)(P.outst + own) < (unsigned)*(volatile int *)&head->cap;
-                    if (room && P.n_max - bdp >= kMinShareGap && atomicSub(&head->want_don, 1) > 0) {
-                        unsigned long long pos = 0ull;
-                        bool got = false;
-                        for (int attempt = 0; attempt < 8; ++attempt) {
-                            const unsigned long long t0 = *(volatile unsigned long long *)P.dq_tail;
-                            const uint32_t c0 = (uint32_t)t0 & dq_mask;
-                            if (*(volatile unsigned int *)(P.dq_free + c0) != (uint32_t)(t0 >> P.dq_log2cap)) break;
-                            if (atomicCAS(P.dq_tail, t0, t0 + 1ull) == t0) { pos = t0; got = true; break; }
-                        }
-                        if (got) {
-                            if (did == 0u && !donated) { P.outst[own] = 2u; donated = true; }
-                            else atomicAdd(P.outst + own, 1u);
-                            const uint32_t cell = (uint32_t)pos & dq_mask;
-                            unsigned char *cb = P.dq_cells + (size_t)cell * (size_t)P.dq_cell_bytes;
-                            *reinterpret_cast<uint4 *>(cb) = make_uint4((uint32_t)own, seq, tour, (uint32_t)bdp);
-                            *reinterpret_cast<uint2 *>(cb + 16) = make_uint2(bm, 0u);
-                            *reinterpret_cast<double *>(cb + 24) = bw;
-                            don_cell = (int)cell;
-                            don_round = (uint32_t)(pos >> P.dq_log2cap);
-                            don_bdp = bdp;
-                            bot += 1;
-                            if (sbase < bot) sbase = bot;
-                        } else {
-                            atomicAdd(&head->want_don, 1);
-                        }
-                    }
-                }
-            } else {
-                // leaf: resume the most recent waiting copy, or end the tour
-                if (top == sbase && sbase > bot) {
-                    // ring empty: bring back up to kChunk records, all loads in flight
-                    // before the first store (one round trip to L2, not kChunk)
-                    const int lo = sbase - kChunk > bot ? sbase - kChunk : bot;
-                    uint32_t fmeta[kChunk];
-                    double fw[kChunk];
-#pragma unroll
-                    for (int i = 0; i < kChunk; ++i) {
-                        const int idx = lo + i;
-                        fmeta[i] = idx < sbase ? __ldcg(gmeta + idx) : 0u;
-                        fw[i] = idx < sbase ? __ldcg(gwt + idx) : 0.0;
-                    }
-#pragma unroll
-                    for (int i = 0; i < kChunk; ++i) {
-                        const int idx = lo + i;
-                        if (idx < sbase) {
-                            smeta[(uint32_t)(idx & (K - 1)) * ST + lane] = fmeta[i];
-                            sw[(uint32_t)(idx & (K - 1)) * ST + lane] = fw[i];
-                        }
-                    }
-                    sbase = lo;
-                }
-                const int hi = n < P.n_max - 1 ? n : P.n_max - 1;
-                if (top == bot) {
-                    un_lo = 0; un_hi = hi; tour_end = true;
-                } else {
-                    const int ti = (top - 1) & (K - 1);
-                    const uint32_t meta = smeta[(uint32_t)ti * ST + lane];
-                    const int dp = (int)(meta & 0xFFFFu);
-                    const int cnt = (int)((meta >> 16) & 7u);
-                    const uint32_t dirs = meta >> 19;
-                    pend_dir = (int)(dirs & 7u);
-                    pend_w = sw[(uint32_t)ti * ST + lane];
-                    pend_depth = dp;
-                    if (cnt <= 1) --top;
-                    else smeta[(uint32_t)ti * ST + lane] = (uint32_t)dp | ((uint32_t)(cnt - 1) << 16) | ((dirs >> 3) << 19);
-                    un_lo = dp + 1; un_hi = hi; tour_end = false;
-                }
-                state = kUnwindState;
             }
-        }
-        }
+            ord += isn ? 1u : 0u;
+            const bool extend = c > 0, leaf = isn && c == 0;
+            cur = extend ? ckey : cur;
+            W = extend ? o.child_w : W;
+            const int n_leaf = n;
+            n += extend ? 1 : 0;
+            if (first && extend && n < P.n_max) {
+                hash[cslot] = ckey;
+                sites[n] = (uint16_t)cslot;
+            }
 
-        // ---------------- hand-overs: the whole warp copies each donor's sites ----------------
-        // A donor's sites 0..bdp are still in its hash (this iteration's deletions come
-        // below), each in the slot an in-order rebuild would give it, so the cell holds
-        // (key, slot) per site and the taker places them without probing.
-        if (P.share) {
-            unsigned dm = __ballot_sync(kFull, don_cell >= 0);
-            if (dm) __syncwarp();          // every lane sees the donors' sites
-            while (dm) {
-                const int src = __ffs(dm) - 1;
-                dm &= dm - 1u;
-                const int scell = __shfl_sync(kFull, don_cell, src);
-                const int sbdp = __shfl_sync(kFull, don_bdp, src);
-                unsigned char *cb = P.dq_cells + (size_t)scell * (size_t)P.dq_cell_bytes;
-                Key *ck = reinterpret_cast<Key *>(cb + 32);
-                uint16_t *cs = reinterpret_cast<uint16_t *>(cb + 32 + cell_key_bytes);
-                copy_sites_to_cell<Key>(hash, sites, ST, src, sbdp, ck, cs, lane);
-                __syncwarp();
-                if (lane == src) {
-                    __threadfence();
-                    *(volatile unsigned int *)(P.dq_ready + scell) = don_round + 1u;
-                }
-            }
-            don_cell = -1;
-        }
-
-        // ---------------- backtrack: LIFO deletions, then resume ----------------
-        if (state == kUnwindState) {
-#pragma unroll
-            for (int i = 0; i < kUnwind; ++i) {
-                const int k = un_hi - i;
-                if (k >= un_lo) hash[(uint32_t)sites[(uint32_t)k * ST + lane] * ST + lane] = (Key)0;
-            }
-            un_hi -= kUnwind;
-            if (un_hi < un_lo) {
-                if (tour_end) {
+            // ---------------- a leaf, or a backtrack still under way ----------------
+            // The most recent waiting copy, or the end of the tour; LIFO deletions, the
+            // group's lanes side by side; then the walk resumes.
+            if (leaf || state == kUnwindState) {
+                const unsigned gmask = ((1u << G) - 1u) << lead;
+                if (leaf) {
+                    if (top == sbase && sbase > bot) {
+                        // ring empty: bring back up to kChunk records, the group's lanes side by side
+                        const int lo = sbase - kChunk > bot ? sbase - kChunk : bot;
+                        for (int idx = lo + j; idx < sbase; idx += G) {
+                            smeta[idx & (K - 1)] = __ldcg(gmeta + idx);
+                            sw[idx & (K - 1)] = __ldcg(gwt + idx);
+                        }
+                        sbase = lo;
+                        __syncwarp(gmask);
+                    }
+                    un_hi = n_leaf < P.n_max - 1 ? n_leaf : P.n_max - 1;
                     state = kFlush;
-                } else {
-                    const int dp = pend_depth;
-                    KeyCodec<D, Key>::decode(hash[(uint32_t)sites[(uint32_t)dp * ST + lane] * ST + lane], cx, cy, cz);
-                    step_coords(pend_dir, cx, cy, cz);
-                    back = pend_dir ^ 1;
-                    n = dp + 1;
-                    if (n < P.n_max) {
-                        const int s = hash_insert<Key>(hash, ST, lane, P.log2h, KeyCodec<D, Key>::encode(cx, cy, cz));
-                        if (s < 0) { set_status(P.status, PERM_EOVERFLOW); state = kDone; }
-                        else sites[(uint32_t)n * ST + lane] = (uint16_t)s;
-                    }
-                    W = pend_w;
-                    if (state != kDone) state = kNode;
-                }
-            }
-        }
-
-        // ---------------- end of a tour (part): per-tour sums into Q (whole warp) ----------------
-        if (__any_sync(kFull, state == kFlush)) {
-            if (state == kFlush) {
-                if (did == 0u && !donated) {
-                    // the whole tour grew on this walk
-                    frow = own; fmaxn = maxn; do_flush = true; shared_flush = false;
-                } else {
-                    // parts of the tour grew elsewhere: the last part to end flushes
-                    const unsigned om = atomicMax(P.tmaxn + own, (unsigned)maxn);
-                    __threadfence();
-                    const unsigned left = atomicSub(P.outst + own, 1u);
-                    do_flush = (left == 1u);
-                    shared_flush = true;
-                    frow = own;
-                    fmaxn = (int)(om > (unsigned)maxn ? om : (unsigned)maxn);
-                    if (!do_flush && did == 0u) {
-                        // the row stays with the parts still growing: the next tour
-                        // takes the walk's other row, if that one is free
-                        myrow ^= rows_per_walk - 1;
-                        xbusy = *(volatile unsigned int *)(P.outst + myrow) != kRowFree;
+                    if (top != bot) {
+                        const int ti = (top - 1) & (K - 1);
+                        const uint32_t meta = smeta[ti];
+                        const int dp = (int)(meta & 0xFFFFu);
+                        const int cnt = (int)((meta >> 16) & 7u);
+                        const uint32_t rest = meta >> 19;
+                        pend_dir = (int)(rest & 7u);
+                        pend_w = sw[ti];
+                        pend_depth = dp;
+                        __syncwarp(gmask);      // every lane has read the record
+                        if (cnt <= 1) --top;
+                        else if (first) smeta[ti] = (uint32_t)dp | ((uint32_t)(cnt - 1) << 16) | ((rest >> 3) << 19);
+                        un_lo = dp + 1;
+                        state = kUnwindState;
                     }
                 }
-            }
-            unsigned fm = __ballot_sync(kFull, state == kFlush && do_flush);
-            __threadfence();
-            __syncwarp();
-            while (fm) {
-                const int src = __ffs(fm) - 1;
-                fm &= fm - 1u;
-                const int s_slot = __shfl_sync(kFull, frow, src);
-                const int s_maxn = __shfl_sync(kFull, fmaxn, src);
-                const int s_seq = __shfl_sync(kFull, cur_seq, src);
-                double *Xr = P.X + (size_t)s_slot * L;
-                double *Qr = (P.alg == PERM_ALG1) ? P.Qn + (size_t)(s_seq < 0 ? 0 : s_seq) * L : P.Qn;
-                // eight loads in flight per lane, then the squares go straight to Q_n
-                for (int k0 = 0; k0 <= s_maxn; k0 += 32 * 8) {
-                    double x[8];
+                if (state == kUnwindState) {
+                    const Key rkey = hash[sites[pend_depth]] + step_key<D, Key>(pend_dir);
+                    constexpr int kUnwind = kUnwindSites / G;
+                    int sl[kUnwind];
 #pragma unroll
-                    for (int u = 0; u < 8; ++u) {
-                        const int k = k0 + u * 32 + lane;
-                        x[u] = (k <= s_maxn) ? __ldcg(Xr + k) : 0.0;
+                    for (int i = 0; i < kUnwind; ++i) {
+                        const int k = un_hi - j - i * G;
+                        sl[i] = k >= un_lo ? (int)sites[k] : -1;
                     }
 #pragma unroll
-                    for (int u = 0; u < 8; ++u) {
-                        const int k = k0 + u * 32 + lane;
-                        if (__double_as_longlong(x[u]) != 0ll) {     // (an integer test: no -0.0 here)
-                            atomicAdd(&Qr[k], __dmul_rn(x[u], x[u]));
-                            __stcg(Xr + k, 0.0);
+                    for (int i = 0; i < kUnwind; ++i)
+                        if (sl[i] >= 0) hash[sl[i]] = (Key)0;
+                    un_hi -= kUnwindSites;
+                    __syncwarp(gmask);
+                    if (un_hi < un_lo) {
+                        n = pend_depth + 1;
+                        cur = rkey;
+                        W = pend_w;
+                        state = kNode;
+                        if (n < P.n_max) {
+                            // the new end-point's place (every lane of the group looks at the same
+                            // buckets): the first bucket of its sequence that is not full
+                            const uint32_t bmask = (1u << log2b) - 1u;
+                            uint32_t b = hash_home(rkey, log2b);
+                            look_bucket(hash, b, rkey, hit, full, place);
+                            for (uint32_t it = 0u; full && it < bmask; ++it) {
+                                b = (b + it + 1u) & bmask;
+                                look_bucket(hash, b, rkey, hit, full, place);
+                            }
+                            __syncwarp(gmask);
+                            if (full) {
+                                set_status(P.status, PERM_EOVERFLOW);
+                                state = kDone;
+                            } else if (first) {
+                                const uint32_t rs = b * (uint32_t)Buckets<Key>::kKeys + (uint32_t)place;
+                                hash[rs] = rkey;
+                                sites[n] = (uint16_t)rs;
+                            }
                         }
                     }
                 }
             }
-            __threadfence();
             __syncwarp();
-            if (state == kFlush) {
-                if (do_flush) {
-                    if (shared_flush) {
-                        P.tmaxn[frow] = 0u;
-                        __threadfence();
-                        *(volatile unsigned int *)(P.outst + frow) = kRowFree;
-                    }
-                    atomicAdd(P.finished, 1ull);
-                    if (P.alg == PERM_ALG1) {
-                        seq_t += 1;
-                        P.seq_M[cur_seq] = (unsigned long long)seq_t;
-                    }
-                }
-                own = myrow; did = 0u; donated = false; do_flush = false;
-                state = kNeed;
-            }
         }
     }
     if (P.share && lane == 0 && my_hungry != 0) atomicAdd(P.hungry, -my_hungry);
 
-    // statistics, then tell the refresher this warp is done
-    unsigned long long tot = my_steps, cps = my_copies, exn = my_exact;
+    // statistics (a walk cut short by an error counts its part so far), then tell the
+    // refresher this warp is done
+    if (state == kNode || state == kUnwindState) my_steps += ord;
+    unsigned long long tot = first ? my_steps : 0ull, cps = first ? my_copies : 0ull, exn = first ? my_exact : 0ull;
     int ms = my_max_stack;
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) {
@@ -1203,47 +1355,75 @@ __global__ void batch_init_kernel(const BatchDev B) {
 }
 
 // ---------------------------------------------------------------------------
-// Growth step on caller-given snapshot states (one thread per state).
+// Growth step on caller-given snapshot states (one group of lanes per state, one
+// warp per block, as the persistent kernel's node).
 // ---------------------------------------------------------------------------
 template <int D, typename Key>
 __global__ void __launch_bounds__(32) debug_step_kernel(int n_max, int log2h, int B,
         const int32_t *coords, const int32_t *len, const double *Wv, const double *Wsv,
         const uint64_t *Mv, const uint64_t *ordv, const uint32_t *seqv, const uint32_t *tourv,
         uint32_t k0, uint32_t k1, int force_exact, int32_t *out_i, double *out_r, double *out_w) {
+    constexpr int G = kGroupLanes<D>, kPer = 32 / G;
     extern __shared__ __align__(16) unsigned char smem[];
-    const int H = 1 << log2h;
-    Key *hash = reinterpret_cast<Key *>(smem);
-    double *aoc = reinterpret_cast<double *>(smem + (size_t)H * kStride * sizeof(Key));
-    const int lane = threadIdx.x;
-    fill_aoc(aoc, D, lane, 32);
-    for (int s = 0; s < H; ++s) hash[(size_t)s * kStride + lane] = (Key)0;
+    double *aoc = reinterpret_cast<double *>(smem);
+    const uint32_t *lists = reinterpret_cast<const uint32_t *>(aoc + kFactors);
+    const int lane = threadIdx.x, grp = lane / G, j = lane % G, lead = lane - j;
+    const int H = 1 << log2h, log2b = log2h - Buckets<Key>::kLog2;
+    Key *all = reinterpret_cast<Key *>(smem + 1024);
+    Key *hash = all + (size_t)H * grp;
+    fill_constants(aoc, D, lane, 32);
+    for (int s = lane; s < H * kPer; s += 32) all[s] = (Key)0;
     __syncwarp();
-    const int b = blockIdx.x * 32 + lane;
-    if (b >= B) return;
-    int32_t *oi = out_i + (size_t)b * 11;
-    const int n = len[b];
-    if (n < 0 || n > n_max) { oi[0] = -1; return; }
-    const int32_t *cb = coords + (size_t)b * (n_max + 1) * D;
+    const int b = blockIdx.x * kPer + grp;
+    const bool have = b < B;
+    const int n = have ? len[b] : -1;
+    const bool good = n >= 0 && n <= n_max;
+    if (have && !good && j == 0) out_i[(size_t)b * 11] = -1;
+    const int32_t *cb = coords + (size_t)(good ? b : 0) * (n_max + 1) * D;
+    // the walk's sites in order (the one at depth n_max is never inserted)
     bool ovf = false;
-    const int top = n < n_max - 1 ? n : n_max - 1;
-    for (int k = 0; k <= top; ++k) {
-        const Key key = KeyCodec<D, Key>::encode(cb[k * D], cb[k * D + 1], D == 3 ? cb[k * D + 2] : 0);
-        if (hash_insert<Key>(hash, kStride, lane, log2h, key) < 0) ovf = true;
+    const int last = good ? (n < n_max - 1 ? n : n_max - 1) : -1;
+    for (int k = 0; __any_sync(kFull, k <= last); ++k) {
+        Key key = KeyCodec<D, Key>::encode(0, 0, 0);
+        if (k <= last) key = KeyCodec<D, Key>::encode(cb[k * D], cb[k * D + 1], D == 3 ? cb[k * D + 2] : 0);
+        int slot = 0;
+        bool o = false;
+        const bool absent = probe<Key>(hash, log2b, key, k <= last, slot, o);
+        ovf = ovf || (k <= last && !absent);
+        __syncwarp();
+        if (j == 0 && absent) hash[slot] = key;
+        __syncwarp();
     }
-    const int cx = cb[n * D], cy = cb[n * D + 1], cz = (D == 3) ? cb[n * D + 2] : 0;
-    int eslot[2 * D];
-    const Cutoffs none{nullptr, 1, 1.0, 1.0, 0ull};
-    const NodeOut o = grow_node<D, Key>(hash, kStride, lane, log2h, n, n_max, cx, cy, cz, Wv[b],
-                                        Wsv[b], Mv[b], ordv[b], seqv[b], tourv[b], k0, k1, aoc, eslot,
-                                        none, 0.0, -1, force_exact != 0);
-    oi[0] = (ovf || o.overflow) ? -2 : o.outcome;
-    oi[1] = o.a;
-    oi[2] = o.mask;
-    oi[3] = o.c;
-    for (int i = 0; i < 6; ++i) oi[4 + i] = (i < o.c) ? (int)((o.dirs >> (3 * i)) & 7u) : -1;
-    oi[10] = o.exact ? 1 : 0;
+    Key cur = KeyCodec<D, Key>::encode(0, 0, 0);
+    if (good) cur = KeyCodec<D, Key>::encode(cb[n * D], cb[n * D + 1], D == 3 ? cb[n * D + 2] : 0);
+    const double W = good ? Wv[b] : 1.0, Wsum = good ? Wsv[b] : 1.0;
+    const unsigned long long M = good ? Mv[b] : 1ull, ordinal = good ? ordv[b] : 0ull;
+    const Philox4 w = philox4x32_10((uint32_t)ordinal, (uint32_t)(ordinal >> 32), good ? tourv[b] : 0u,
+                                    good ? seqv[b] : 0u, k0, k1);
+    int slot = 0;
+    const bool grows_on = good && n < n_max;
+    const bool free_j = probe<Key>(hash, log2b, cur + step_key<D, Key>(j < 2 * D ? j : 0), grows_on && j < 2 * D, slot, ovf);
+    const int fm = (int)((__ballot_sync(kFull, free_j) >> lead) & ((1u << G) - 1u));
+    ovf = ((__ballot_sync(kFull, ovf) >> lead) & ((1u << G) - 1u)) != 0u;
+    const int a = __popc(fm);
+    const bool decides = grows_on && a > 0;
+    Tours t;
+    set_tours(t, M);
+    const Decision o = decide_node<D>(good ? n : 0, a > 0 ? a : 1, W, Wsum, t, true, w.x, aoc, decides,
+                                      decides && force_exact != 0);
+    if (!good || j != 0) return;
+    const int c = decides ? o.c : 0;
+    uint32_t dirs = lists[fm], xw = w.y;
+    for (int i = 0; i < c; ++i) choose_step(i, a, dirs, xw);
+    int32_t *oi = out_i + (size_t)b * 11;
+    oi[0] = ovf ? -2 : (!grows_on ? kLeafNmax : (a == 0 ? kTrapped : (c == 0 ? kPruned : kChildren)));
+    oi[1] = a;
+    oi[2] = fm;
+    oi[3] = c;
+    for (int i = 0; i < 6; ++i) oi[4 + i] = (i < c) ? (int)((dirs >> (3 * i)) & 7u) : -1;
+    oi[10] = decides && o.exact ? 1 : 0;
     out_r[b] = o.r;
-    out_w[b] = o.child_w;
+    out_w[b] = c > 0 ? o.child_w : 0.0;
 }
 
 __global__ void philox_kernel(int B, const uint32_t *ctr, uint32_t k0, uint32_t k1, uint32_t *out) {
@@ -1261,18 +1441,13 @@ __global__ void finalize_kernel(unsigned long long *tickets, long long limit) {
 
 }  // namespace
 
-size_t cta_smem_bytes(int d, bool key64, int n_max, int log2h, int stack_cache, int worker_warps,
-                      bool snapshot, int stride) {
-    (void)d;
-    return head_region_bytes(n_max, snapshot) +
-           warp_region_bytes(n_max, log2h, stack_cache, key64 ? 8 : 4, stride) * (size_t)worker_warps;
-}
-
 size_t cta_head_bytes(int n_max, bool snapshot) { return head_region_bytes(n_max, snapshot); }
 
-size_t cta_warp_bytes(bool key64, int n_max, int log2h, int stack_cache, int stride) {
-    return warp_region_bytes(n_max, log2h, stack_cache, key64 ? 8 : 4, stride);
+size_t walk_bytes(bool key64, int n_max, int log2h, int stack_cache) {
+    return walk_region_bytes(n_max, log2h, stack_cache, key64 ? 8 : 4);
 }
+
+int walks_per_warp_max(int d) { return 32 / (d == 2 ? kGroupLanes<2> : kGroupLanes<3>); }
 
 namespace {
 template <int D, typename Key, int MODE>
@@ -1293,11 +1468,9 @@ template <int D, typename Key, int MODE>
 cudaError_t launch_one(const RunDev &P, int ctas, cudaStream_t stream) {
     const bool snapshot = (MODE == kSnapshot);
     // shared memory holds what the arena does not
-    const size_t smem = P.arena_mode == kArenaAll ? 0
-                      : (P.arena_mode == kArenaWalks ? head_region_bytes(P.n_max, snapshot)
-                                                     : cta_smem_bytes(D, sizeof(Key) == 8, P.n_max, P.log2h,
-                                                                      P.stack_cache, P.worker_warps, snapshot,
-                                                                      P.stride));
+    const size_t head = P.arena_mode == kArenaAll ? 0 : head_region_bytes(P.n_max, snapshot);
+    const size_t smem = head + (P.arena_mode != kArenaNone ? 0 : walk_region_bytes(P.n_max, P.log2h, P.stack_cache, sizeof(Key)) *
+                                                                     (size_t)(P.S * P.worker_warps));
     cudaError_t e = allow_smem<D, Key, MODE>();
     if (e != cudaSuccess) return e;
     const int threads = 32 * (P.worker_warps + (snapshot ? 1 : 0));
@@ -1374,10 +1547,10 @@ cudaError_t launch_debug_step(int d, int n_max, int B, const int32_t *coords, co
                               double *out_r, double *out_w, cudaStream_t stream) {
     int log2h = 4;
     while ((1 << log2h) < 2 * n_max) ++log2h;
-    const int blocks = (B + 31) / 32;
-    if (blocks == 0) return cudaSuccess;
-    const size_t key_b = 4;
-    const size_t smem = ((size_t)1 << log2h) * kStride * key_b + 128 * 8;
+    if (B <= 0) return cudaSuccess;
+    const int per = walks_per_warp_max(d);               // states per block of one warp
+    const int blocks = (B + per - 1) / per;
+    const size_t smem = 1024 + walk_hash_bytes(log2h, 4) * (size_t)per;
     if (d == 2) {
         cudaError_t e = cudaFuncSetAttribute(debug_step_kernel<2, uint32_t>,
                                              cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);

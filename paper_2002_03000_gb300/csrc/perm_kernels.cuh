@@ -18,8 +18,7 @@ struct RunDev {
     int d, n_max, n_seq, alg;
     int run_index;       // position in a batch launch's run table (0 otherwise)
     int log2h;           // per-walk hash size 2^log2h
-    int S;               // lanes per warp that hold walks
-    int stride;          // interleave stride of per-walk shared arrays (power of 2, >= S)
+    int S;               // walks per warp
     int worker_warps;    // per CTA
     int slots;           // walks on the device
     int tour_slots;      // walks that start tours (slots below it); the rest are helpers
@@ -117,11 +116,13 @@ int member_reset(perm_handle h);
 // run's current tables (cumulative, as perm_run).
 int member_extend(perm_handle h, int64_t extra_tours_per_seq, int run_index, RunDev *P);
 
-// Shared-memory bytes of one CTA (everything in shared memory), and its parts.
-size_t cta_smem_bytes(int d, bool key64, int n_max, int log2h, int stack_cache, int worker_warps,
-                      bool snapshot, int stride);
+// Bytes of a CTA's head region, and of one walk's region.
 size_t cta_head_bytes(int n_max, bool snapshot);
-size_t cta_warp_bytes(bool key64, int n_max, int log2h, int stack_cache, int stride);
+size_t walk_bytes(bool key64, int n_max, int log2h, int stack_cache);
+// Walks that a warp holds at most (a walk takes a group of its lanes), and walk
+// warps of a CTA.
+int walks_per_warp_max(int d);
+constexpr int kMaxWalkWarps = 8;
 
 cudaError_t launch_grow(const RunDev &P, int thresh_mode, bool key64, int ctas,
                         cudaStream_t stream);

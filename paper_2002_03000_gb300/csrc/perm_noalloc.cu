@@ -18,6 +18,7 @@
 // the last call's contents; each call clears what must start at zero.  Two
 // calls whose work overlaps on the GPU (different streams, or different host
 // threads on one device) race on it and both results are then invalid.
+#include <algorithm>
 #include <cstring>
 #include <mutex>
 
@@ -96,34 +97,29 @@ extern "C" int perm_run_static(const perm_config *cfg, int64_t tours_per_seq, do
         return PERM_EDEVICE;
     const size_t optin = (size_t)smem_optin;
 
-    // layout: one walk per thread, 32 walks per warp at most, as many warps per
-    // CTA as shared memory allows, one CTA per SM
+    // layout: walks over up to 8 warps per CTA, as many as shared memory allows, one
+    // CTA per SM
     const bool snap = (cfg->threshold == PERM_THRESH_SNAPSHOT);
     int log2h = 4;
     while ((1 << log2h) < 2 * n_max) ++log2h;
     const int K = 16;
-    int stride = 32;
-    size_t head = 0, per_warp = 0;
-    for (;; stride /= 2) {
-        head = perm::cta_smem_bytes(d, key64, n_max, log2h, K, 0, snap, stride);
-        per_warp = perm::cta_smem_bytes(d, key64, n_max, log2h, K, 1, snap, stride) - head;
-        if (head + per_warp <= optin || stride == 1) break;
-    }
-    if (head + per_warp > optin) return PERM_EUNSUPPORTED;
-    int max_warps = (int)((optin - head) / per_warp);
-    if (max_warps > 4) max_warps = 4;
+    const size_t head = perm::cta_head_bytes(n_max, snap), walk = perm::walk_bytes(key64, n_max, log2h, K);
+    if (head + walk > optin) return PERM_EUNSUPPORTED;
+    const long long most = std::min((long long)((optin - head) / walk),
+                                    (long long)perm::kMaxWalkWarps * perm::walks_per_warp_max(d));
 
     long long slots = cfg->slots ? cfg->slots : n_seq;
     if (slots > n_seq) slots = n_seq;
     if (slots > fit) slots = fit;
-    const long long cap = (long long)num_sms * max_warps * stride;
-    if (slots > cap) slots = cap;
-    const long long per_cta = (slots + num_sms - 1) / num_sms;
-    int warps = (int)((per_cta + stride - 1) / stride);
-    if (warps > max_warps) warps = max_warps;
-    if (warps < 1) warps = 1;
-    int lanes = (int)((per_cta + warps - 1) / warps);
-    if (lanes > stride) lanes = stride;
+    if (slots > num_sms * most) slots = num_sms * most;
+    long long per_cta = (slots + num_sms - 1) / num_sms;
+    int lanes = 1, warps = 1;
+    for (;; --per_cta) {                        // whole warps of `lanes` walks, within shared memory
+        lanes = (int)((per_cta + perm::kMaxWalkWarps - 1) / perm::kMaxWalkWarps);
+        warps = (int)((per_cta + lanes - 1) / lanes);
+        if ((long long)lanes * warps <= most) break;
+    }
+    slots = std::min(slots, (long long)num_sms * lanes * warps);
     const int ctas = (int)((slots + (long long)warps * lanes - 1) / ((long long)warps * lanes));
 
     unsigned char *p = static_cast<unsigned char *>(base);
@@ -148,7 +144,7 @@ extern "C" int perm_run_static(const perm_config *cfg, int64_t tours_per_seq, do
     perm::RunDev P;
     std::memset(&P, 0, sizeof(P));
     P.d = d; P.n_max = n_max; P.n_seq = n_seq; P.alg = PERM_ALG2;
-    P.log2h = log2h; P.S = lanes; P.stride = stride; P.worker_warps = warps;
+    P.log2h = log2h; P.S = lanes; P.worker_warps = warps;
     P.slots = (int)slots; P.tour_slots = (int)slots; P.stack_cache = K;
     P.key0 = (uint32_t)cfg->seed ^ cfg->run_id;
     P.key1 = (uint32_t)(cfg->seed >> 32);

@@ -86,8 +86,10 @@ typedef struct {
                           copy's weights still count for that tour (Sec. 2: the copies
                           grow independently).  k >= 1: at most k parts of one tour grow
                           at once; 0 = on with the default cap (4); -1 = off.  Once no
-                          tour of the run has finished for 5 ms (a start-up tree too
-                          large for a few walks), the cap rises to 1024 */
+                          tour of the run has finished for 0.7 ms (a start-up tree too
+                          large for a few walks), and at a run's end (no tour left to
+                          start, at most one in eight of the run's tours unfinished),
+                          the cap rises to 1024 */
     int stack_ring;    /* waiting-copy records per walk kept in shared memory (the rest
                           spill to global memory 8 at a time): 16, 32, 64 or 128;
                           0 = default (16) */

@@ -48,7 +48,7 @@ struct perm_run_s {
     unsigned char *dq_cells = nullptr;
     unsigned long long *dq_head = nullptr, *dq_tail = nullptr;
     unsigned int *dq_ready = nullptr, *dq_free = nullptr, *outst = nullptr, *tmaxn = nullptr;
-    int *hungry = nullptr;
+    int *hungry = nullptr;         // [0] walks waiting for work, [1] cells waiting for a walk, [2] cells in use
     double2 *cut = nullptr;        // original PERM's cut-offs (nullptr: flatPERM)
     int cut_copies = 1;
     double cut_q = 1.0;
@@ -92,11 +92,14 @@ void free_all(perm_handle h) {
 }
 
 // Parts of one tour that may grow on other walks at once (shared copies), and the
-// larger bound used once no tour of the run has finished for kStallNs.
+// larger bound used once no tour of the run has finished for kStallNs.  GB300, ms per
+// complete run at 5 / 2 / 0.7 / 0.3 ms: square n = 512, 4096 x 256 215 / 210 / 208 / 208;
+// cubic n = 512, 8192 x 128 173 / 168 / 166 / 165; square n = 256, 1000 x 64 32 / 28 / 26 / 25;
+// cubic n = 945, 2142 x 4 86 / 38 / 33 / 33; square n = 1725, 422 x 4 250 / 205 / 184 / 470.
 constexpr int kAutoWalks = 32;          // walks per CTA of the automatic layout
 constexpr int kDefaultShareCap = 4;
 constexpr int kBoostShareCap = 1024;
-constexpr long long kStallNs = 5000000;
+constexpr long long kStallNs = 700000;
 
 int scale_exp_host(int d, int n) { return d == 2 ? (11 * n) >> 3 : (9 * n) >> 2; }
 
@@ -365,7 +368,7 @@ int create_impl(perm_handle *out, const perm_config *cfg, const ForcedLayout *fo
         if (rc == PERM_OK) rc = dalloc(h, &h->outst, (size_t)h->xrows);
         if (rc == PERM_OK) rc = to_code(cudaMemsetAsync(h->outst, 0xFF, sizeof(unsigned int) * h->xrows, h->stream));
         if (rc == PERM_OK) rc = dalloc(h, &h->tmaxn, (size_t)h->xrows);
-        if (rc == PERM_OK) rc = dalloc(h, &h->hungry, 1);
+        if (rc == PERM_OK) rc = dalloc(h, &h->hungry, 3);
     }
     if (rc == PERM_OK) rc = to_code(cudaStreamSynchronize(h->stream));
     if (rc != PERM_OK) {
@@ -425,7 +428,7 @@ static RunDev make_params(perm_handle h) {
     P.stall_ns = kStallNs;
     P.dq_log2cap = h->dq_log2cap; P.dq_cell_bytes = h->dq_cell_bytes; P.dq_cells = h->dq_cells;
     P.dq_head = h->dq_head; P.dq_tail = h->dq_tail; P.dq_ready = h->dq_ready; P.dq_free = h->dq_free;
-    P.outst = h->outst; P.tmaxn = h->tmaxn; P.hungry = h->hungry;
+    P.outst = h->outst; P.tmaxn = h->tmaxn; P.hungry = h->hungry; P.queued = h->hungry ? h->hungry + 1 : nullptr; P.dq_used = h->hungry ? h->hungry + 2 : nullptr;
     P.status = h->status;
     P.cut = h->cut;
     P.cut_copies = h->cut_copies;
@@ -565,7 +568,7 @@ int perm_reset(perm_handle h) {
         if (e == cudaSuccess) e = cudaMemsetAsync(h->dq_tail, 0, sizeof(unsigned long long), h->stream);
         if (e == cudaSuccess) e = cudaMemsetAsync(h->dq_ready, 0, sizeof(unsigned int) * cap, h->stream);
         if (e == cudaSuccess) e = cudaMemsetAsync(h->dq_free, 0, sizeof(unsigned int) * cap, h->stream);
-        if (e == cudaSuccess) e = cudaMemsetAsync(h->hungry, 0, sizeof(int), h->stream);
+        if (e == cudaSuccess) e = cudaMemsetAsync(h->hungry, 0, 3 * sizeof(int), h->stream);
         if (e == cudaSuccess) e = cudaMemsetAsync(h->outst, 0xFF, sizeof(unsigned int) * h->xrows, h->stream);
         if (e == cudaSuccess) e = cudaMemsetAsync(h->tmaxn, 0, sizeof(unsigned int) * h->xrows, h->stream);
     }

@@ -361,6 +361,7 @@ __device__ __forceinline__ void grow_run(const RunDev &P, unsigned char *smem, c
         const long long t0 = global_ns();
         unsigned long long last_fin = *(volatile unsigned long long *)P.finished;
         long long t_change = t0;
+        bool boosted = false;
         if (lane == 0) *(volatile int *)&head->cap = P.share;
         for (long long it = 0;; ++it) {
             const long long c_it = clock64();
@@ -407,7 +408,12 @@ __device__ __forceinline__ void grow_run(const RunDev &P, unsigned char *smem, c
                 // tours spread over every idle walk from then on
                 const long long now = global_ns();
                 if (fin_now != last_fin) { last_fin = fin_now; t_change = now; }
-                else if (now - t_change > P.stall_ns) *(volatile int *)&head->cap = P.share_boost;
+                // and so does a run's end: no tour is left to start, and at most one in eight of
+                // the run's tours is not finished, so the table has samples at the lengths that
+                // the parts reach, and spreading makes no larger trees
+                const bool tail = (long long)Ms >= limit && (long long)fin_now >= limit - limit / 8;
+                if (now - t_change > P.stall_ns) boosted = true;
+                *(volatile int *)&head->cap = boosted || tail ? P.share_boost : P.share;
                 const int st_now = (now - t_change > P.stall_ns) ? 1 : 0;
                 if (st_now != *(volatile int *)&head->stalled) {
                     *(volatile int *)&head->stalled = st_now;
@@ -530,62 +536,82 @@ __device__ __forceinline__ void grow_run(const RunDev &P, unsigned char *smem, c
         // Its first lane decides and writes the cell's header; the whole warp copies the
         // sites 0..bdp with the slot that an in-order rebuild would give each, so the
         // taker places them without probing.
-        // (looked at every eighth iteration)
+        // (looked at every eighth iteration; the warp's donors reserve their cells together:
+        // a few round trips to L2 and one fence whatever their number)
         if (snapshot && P.share && __shfl_sync(kFull, *(volatile int *)&head->want_don, 0) > 0) {
-            // at most P.share parts of one tour grow at once (a soft cap: the parts of a
-            // tour stay few, so each still sees its siblings' samples)
+            // at most `cap` parts of one tour grow at once (a soft cap: the parts of a tour
+            // stay few, so each still sees its siblings' samples)
+            const bool part = did != 0u || donated;       // the tour has parts elsewhere already
+            uint32_t bm = 0u;
+            double bw = 0.0;
             bool can = first && state == kNode && top - bot >= 2;
-            if (can && !(did == 0u && !donated))
-                can = *(volatile unsigned int *)(P.outst + own) < (unsigned)*(volatile int *)&head->cap;
-            unsigned dm = __ballot_sync(kFull, can);
-            while (dm) {
-                const int src = __ffs(dm) - 1;
-                dm &= dm - 1u;
-                int cell = -1, bdp = 0;
-                uint32_t round = 0u;
-                if (lane == src) {
-                    const int bi = bot & (K - 1);
-                    const uint32_t bm = bot < sbase ? __ldcg(gmeta + bot) : smeta[bi];
-                    const double bw = bot < sbase ? __ldcg(gwt + bot) : sw[bi];
-                    bdp = (int)(bm & 0xFFFFu);
-                    if (P.n_max - bdp >= kMinShareGap && atomicSub(&head->want_don, 1) > 0) {
-                        unsigned long long pos = 0ull;
-                        bool got = false;
-                        for (int attempt = 0; attempt < 8; ++attempt) {
-                            const unsigned long long t0 = *(volatile unsigned long long *)P.dq_tail;
-                            const uint32_t c0 = (uint32_t)t0 & dq_mask;
-                            if (*(volatile unsigned int *)(P.dq_free + c0) != (uint32_t)(t0 >> P.dq_log2cap)) break;
-                            if (atomicCAS(P.dq_tail, t0, t0 + 1ull) == t0) { pos = t0; got = true; break; }
-                        }
-                        if (got) {
-                            if (did == 0u && !donated) P.outst[own] = 2u;
-                            else atomicAdd(P.outst + own, 1u);
-                            cell = (int)((uint32_t)pos & dq_mask);
-                            round = (uint32_t)(pos >> P.dq_log2cap);
-                            unsigned char *cb = P.dq_cells + (size_t)cell * (size_t)P.dq_cell_bytes;
-                            *reinterpret_cast<uint4 *>(cb) = make_uint4((uint32_t)own, seq, tour, (uint32_t)bdp);
-                            *reinterpret_cast<uint2 *>(cb + 16) = make_uint2(bm, 0u);
-                            *reinterpret_cast<double *>(cb + 24) = bw;
-                        } else {
-                            atomicAdd(&head->want_don, 1);
-                        }
+            if (can) {
+                const int bi = bot & (K - 1);
+                bm = bot < sbase ? __ldcg(gmeta + bot) : smeta[bi];
+                bw = bot < sbase ? __ldcg(gwt + bot) : sw[bi];
+                can = P.n_max - (int)(bm & 0xFFFFu) >= kMinShareGap;
+                if (can && part) can = *(volatile unsigned int *)(P.outst + own) < (unsigned)*(volatile int *)&head->cap;
+            }
+            const unsigned dm = __ballot_sync(kFull, can);
+            if (dm) {
+                const int cnt = __popc(dm), rk = __popc(dm & lt_mask);
+                int k = 0;
+                unsigned long long t0 = 0ull;
+                if (lane == 0) {
+                    // this CTA's quota first, then room in the ring (a count, as on the takers'
+                    // side), then the next cells: no retries
+                    const int quota = atomicSub(&head->want_don, cnt);
+                    k = quota < 0 ? 0 : (quota < cnt ? quota : cnt);
+                    if (k > 0) {
+                        const int room = (1 << P.dq_log2cap) - atomicAdd(P.dq_used, k);
+                        const int fit = room < 0 ? 0 : (room < k ? room : k);
+                        if (fit < k) atomicSub(P.dq_used, k - fit);
+                        k = fit;
+                        if (k > 0) t0 = atomicAdd(P.dq_tail, (unsigned long long)k);
                     }
+                    if (k < cnt) atomicAdd(&head->want_don, cnt - k);
                 }
-                cell = __shfl_sync(kFull, cell, src);
-                if (cell < 0) continue;
-                bdp = __shfl_sync(kFull, bdp, src);
+                k = __shfl_sync(kFull, k, 0);
+                t0 = __shfl_sync(kFull, t0, 0);
+                const unsigned long long pos = t0 + (unsigned long long)rk;
+                const uint32_t cell = (uint32_t)pos & dq_mask, round = (uint32_t)(pos >> P.dq_log2cap);
+                const bool gives = can && rk < k;
                 unsigned char *cb = P.dq_cells + (size_t)cell * (size_t)P.dq_cell_bytes;
-                unsigned char *sb = warp_base + wbytes * (size_t)(src / G);
-                copy_sites_to_cell<Key>(reinterpret_cast<const Key *>(sb), reinterpret_cast<const uint16_t *>(sb + hash_b),
-                                        bdp, reinterpret_cast<Key *>(cb + 32),
-                                        reinterpret_cast<uint16_t *>(cb + 32 + cell_key_bytes), lane);
-                __threadfence();
-                __syncwarp();
-                if (lane == src) *(volatile unsigned int *)(P.dq_ready + cell) = round + 1u;
-                if (lead == src) {
-                    if (did == 0u) donated = true;
-                    bot += 1;
-                    if (sbase < bot) sbase = bot;
+                if (gives) {
+                    // (the taker of the cell's last round may still be copying it)
+                    bool ok = false;
+                    for (int spin = 0; spin < kCellSpin; ++spin) {
+                        if (*(volatile unsigned int *)(P.dq_free + cell) == round) { ok = true; break; }
+                        __nanosleep(32);
+                    }
+                    if (!ok) set_status(P.status, PERM_ETIMEOUT);
+                    __threadfence();
+                    if (part) atomicAdd(P.outst + own, 1u);
+                    else P.outst[own] = 2u;
+                    *reinterpret_cast<uint4 *>(cb) = make_uint4((uint32_t)own, seq, tour, bm & 0xFFFFu);
+                    *reinterpret_cast<uint2 *>(cb + 16) = make_uint2(bm, 0u);
+                    *reinterpret_cast<double *>(cb + 24) = bw;
+                }
+                const unsigned gm = __ballot_sync(kFull, gives);
+                for (unsigned cm = gm; cm; cm &= cm - 1u) {
+                    const int src = __ffs(cm) - 1;
+                    unsigned char *db = P.dq_cells + (size_t)__shfl_sync(kFull, cell, src) * (size_t)P.dq_cell_bytes;
+                    unsigned char *sb = warp_base + wbytes * (size_t)(src / G);
+                    copy_sites_to_cell<Key>(reinterpret_cast<const Key *>(sb),
+                                            reinterpret_cast<const uint16_t *>(sb + hash_b),
+                                            (int)(__shfl_sync(kFull, bm, src) & 0xFFFFu), reinterpret_cast<Key *>(db + 32),
+                                            reinterpret_cast<uint16_t *>(db + 32 + cell_key_bytes), lane);
+                }
+                if (gm) {
+                    __threadfence();
+                    __syncwarp();
+                    if (gives) *(volatile unsigned int *)(P.dq_ready + cell) = round + 1u;
+                    if (lane == 0) atomicAdd(P.queued, __popc(gm));
+                    if (gm >> lead & 1u) {
+                        if (did == 0u) donated = true;
+                        bot += 1;
+                        if (sbase < bot) sbase = bot;
+                    }
                 }
             }
         }
@@ -694,9 +720,11 @@ __device__ __forceinline__ void grow_run(const RunDev &P, unsigned char *smem, c
             }
             fresh_need = true;
         }
+        // (rows and tickets are global: of old needs they are looked at every 32nd iteration)
+        const bool deep = P.alg == PERM_ALG1 || (iter & 31u) == 0u || __any_sync(kFull, state == kNeed && fresh_need);
         fresh_need = false;
         const bool blocked = state == kNeed && xbusy;
-        if (__any_sync(kFull, blocked)) {
+        if (deep && __any_sync(kFull, blocked)) {
             unsigned r0 = 0u, r1 = 0u;
             if (blocked && first) {
                 r0 = *(volatile unsigned int *)(P.outst + myrow);
@@ -709,7 +737,7 @@ __device__ __forceinline__ void grow_run(const RunDev &P, unsigned char *smem, c
                 else if (r1 == kRowFree) { myrow ^= 1; xbusy = false; }
             }
         }
-        const bool want_t = state == kNeed && !xbusy && !exhausted;
+        const bool want_t = deep && state == kNeed && !xbusy && !exhausted;
         const unsigned need = __ballot_sync(kFull, want_t && first);
         if (need) {
             if (P.alg == PERM_ALG2) {
@@ -828,15 +856,15 @@ __device__ __forceinline__ void grow_run(const RunDev &P, unsigned char *smem, c
             if (hm && __shfl_sync(kFull, *(volatile int *)&head->queued, 0) > 0) {
                 const int leader = __ffs(hm) - 1;
                 unsigned long long base = 0ull, take = 0ull;
-                if (lane == leader) {
-                    for (int attempt = 0; attempt < 8; ++attempt) {
-                        const unsigned long long h0 = *(volatile unsigned long long *)P.dq_head;
-                        const unsigned long long t0 = *(volatile unsigned long long *)P.dq_tail;
-                        if (t0 <= h0) break;
-                        unsigned long long k = t0 - h0;
-                        k = k < (unsigned long long)__popc(hm) ? k : (unsigned long long)__popc(hm);
-                        if (atomicCAS(P.dq_head, h0, h0 + k) == h0) { base = h0; take = k; break; }
-                    }
+                if (lane == leader && *(volatile int *)P.queued > 0) {
+                    // take from the count of published cells first, what was there; then the
+                    // next cells are this warp's (no retries: with a compare-and-swap on the
+                    // head, a thousand idle warps took 3.5 copies per microsecond together)
+                    const int k = __popc(hm), left = atomicSub(P.queued, k);
+                    const int got = left < 0 ? 0 : (left < k ? left : k);
+                    if (got < k) atomicAdd(P.queued, k - got);
+                    if (got > 0) base = atomicAdd(P.dq_head, (unsigned long long)got);
+                    take = (unsigned long long)got;
                 }
                 base = __shfl_sync(kFull, base, leader);
                 take = __shfl_sync(kFull, take, leader);
@@ -915,7 +943,10 @@ __device__ __forceinline__ void grow_run(const RunDev &P, unsigned char *smem, c
                 // every lane has read the cells: they may be written again
                 __threadfence();
                 __syncwarp();
-                if (claiming && first) *(volatile unsigned int *)(P.dq_free + cell) = round + 1u;
+                if (claiming && first) {
+                    *(volatile unsigned int *)(P.dq_free + cell) = round + 1u;
+                    atomicSub(P.dq_used, 1);
+                }
             }
             const int hcount = __popc(__ballot_sync(kFull, first && state == kNeed && (waiting || xbusy || exhausted)));
             if (hcount != my_hungry) {

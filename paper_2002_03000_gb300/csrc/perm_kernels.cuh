@@ -75,6 +75,8 @@ struct RunDev {
     unsigned int *outst;           // per tour-sum row: live parts of its tour (kRowFree: row unused)
     unsigned int *tmaxn;           // per tour-sum row: deepest length over the parts of its tour
     int *hungry;                   // walks waiting for work
+    int *queued;                   // donation cells written and not yet claimed
+    int *dq_used;                  // donation cells reserved and not yet given back
     int *status;
     // optional sampled trace
     perm_trace_record *trace;

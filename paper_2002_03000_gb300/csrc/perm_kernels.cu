@@ -153,13 +153,15 @@ struct Cutoffs {
 // snapshot (a double-precision division takes as long as a node).
 struct Tours {
     unsigned long long M;
+    double Md;                 // M rounded to double
     float Mf;                  // tours_float(M)
     double inv1, inv3, inv5;   // 1/M rounded to double, and 3 and 5 times that
 };
 __device__ __forceinline__ void set_tours(Tours &t, unsigned long long M) {
     t.M = M;
     t.Mf = tours_float(M);
-    t.inv1 = __drcp_rn(__ull2double_rn(M));
+    t.Md = __ull2double_rn(M);
+    t.inv1 = __drcp_rn(t.Md);
     t.inv3 = __dmul_rn(3.0, t.inv1);
     t.inv5 = __dmul_rn(5.0, t.inv1);
 }
@@ -186,19 +188,18 @@ __device__ __noinline__ Decision decide_node_exact(int a, double W, double Wsum,
 
 // The decision at a node with a >= 1 free neighbours (Sec. 2): r, the copies, the
 // children's weight.  Wsum: sum of the weights recorded at length n before this
-// node; refine: round the survivor's quotient by M correctly (one more step of the
+// node, sum: Wsum + W; refine: round the survivor's quotient by M correctly (one more step of the
 // division).  valid: the lane has a node to decide (the others' results are not used);
 // force_exact: decide on the double-precision r.  Shared by the persistent kernel
 // and the snapshot-state kernel; every lane of a walk's group takes the same decision.
 // One straight line with selects but for the exact path: a branch costs a lone warp
 // 25 cycles or more, a double-precision instruction 64 whatever its active lanes.
 template <int D>
-__device__ __forceinline__ Decision decide_node(int n, int a, double W, double Wsum, const Tours &t, bool refine,
-                                                uint32_t w0, const double *aoc, bool valid, bool force_exact) {
+__device__ __forceinline__ Decision decide_node(int n, int a, double W, double Wsum, double sum, const Tours &t,
+                                                bool refine, uint32_t w0, const double *aoc, bool valid, bool force_exact) {
     Decision o;
     o.exact = false;
     bool odd = false, amb = false, surv = false;
-    const double sum = __dadd_rn(Wsum, W);
     const float x = ratio_estimate(W, Wsum, t.Mf, odd);
     o.r = n == 0 ? 1.0 : widen(x);
     const int dE = scale_row<D>(n) + (D == 2 ? 1 : 2);
@@ -214,8 +215,10 @@ __device__ __forceinline__ Decision decide_node(int n, int a, double W, double W
     double base = W, fac = row[c];
     if (refine) {
         // q = sum (1/M), then q + (sum - q M)/M: the quotient to half a unit
-        const double Md = __ull2double_rn(t.M), q = __dmul_rn(sum, t.inv1);
-        base = surv ? __fma_rn(__fma_rn(-q, Md, sum), t.inv1, q) : W;
+        // (before the decision is known: its four dependent operations run beside it)
+        const double q = __dmul_rn(sum, t.inv1);
+        const double avg = __fma_rn(__fma_rn(-q, t.Md, sum), t.inv1, q);
+        base = surv ? avg : W;
         fac = surv ? row[0] : fac;
     } else {
         const double f0 = a == 3 ? t.inv3 : (a == 5 ? t.inv5 : t.inv1);
@@ -517,6 +520,10 @@ __device__ __forceinline__ void grow_run(const RunDev &P, unsigned char *smem, c
     double *acc = Wrow;        // the row this lane adds a node's weight to (lane 0: W_n, lane 1: the tour's sums)
 
     const bool extras = P.Rn != nullptr || P.cut != nullptr;
+    // fresh form: this walk alone reads and writes the table row of its tours (Algorithm 1:
+    // one row per sequence, one walk per sequence at a time; else a run of one walk, whose
+    // tickets it alone takes, so that M is its own tour's number)
+    const bool own_rows = !snapshot && (P.alg == PERM_ALG1 || P.slots == 1);
     const long long t_start = global_ns();
     for (uint32_t iter = 0u;; ++iter) {
         if ((iter & 7u) == 0u) {
@@ -1001,21 +1008,27 @@ __device__ __forceinline__ void grow_run(const RunDev &P, unsigned char *smem, c
             // lane each (fresh form: the W_n one returns the sum before it)
             if (snapshot) {
                 red_add(acc + n, W, isn && j < 2);
+            } else if (own_rows) {
+                // no other walk touches the row: a plain load (of the whole group) and store
+                // (of its first lane) through L1, not an atomic's round trip to L2 (1000
+                // cycles of a lone walk's 3300 a node)
+                Wsum = Wrow[n];
+                red_add(acc + n, W, isn && j == 1);
             } else {
                 double before = 0.0;
                 unsigned long long Mt = 0ull;
                 if (isn && first) {
                     before = atomicAdd(&Wrow[n], W);
-                    if (P.alg == PERM_ALG2) Mt = *(volatile unsigned long long *)P.tickets;
+                    Mt = *(volatile unsigned long long *)P.tickets;
                 }
                 red_add(acc + n, W, isn && j == 1);
                 Wsum = __shfl_sync(kFull, before, lead);
-                if (P.alg == PERM_ALG2) {
-                    Mt = __shfl_sync(kFull, Mt, lead);
-                    if ((long long)Mt > limit) Mt = (unsigned long long)limit;
-                    Mn = Mt > Mn ? Mt : Mn;
-                }
+                Mt = __shfl_sync(kFull, Mt, lead);
+                if ((long long)Mt > limit) Mt = (unsigned long long)limit;
+                Mn = Mt > Mn ? Mt : Mn;
             }
+            const double sum = __dadd_rn(Wsum, W);
+            if (!snapshot && own_rows && isn && first) Wrow[n] = sum;
             red_inc(Srow + n, isn && j == 2);
             maxn = (isn && n > maxn) ? n : maxn;
             // a full bucket without the key, a used-up block of random words, a new M: one
@@ -1047,7 +1060,7 @@ __device__ __forceinline__ void grow_run(const RunDev &P, unsigned char *smem, c
             // the node's random words, from the lane that holds its block
             const int wl = lead + (int)((ord - pbase) & (uint32_t)(G - 1));
             const uint32_t w0 = __shfl_sync(kFull, pw0, wl), w1 = __shfl_sync(kFull, pw1, wl);
-            Decision o = decide_node<D>(n, a1, W, Wsum, tours, !snapshot, w0, aoc, decides && !cutoffs, false);
+            Decision o = decide_node<D>(n, a1, W, Wsum, sum, tours, !snapshot, w0, aoc, decides && !cutoffs, false);
             if (extras) {
                 if (cutoffs && n > 0) o = decide_cutoffs<D>(n, a1, W, w0, aoc, cuts);
                 if (P.Rn != nullptr) {
@@ -1440,7 +1453,7 @@ __global__ void __launch_bounds__(32) debug_step_kernel(int n_max, int log2h, in
     const bool decides = grows_on && a > 0;
     Tours t;
     set_tours(t, M);
-    const Decision o = decide_node<D>(good ? n : 0, a > 0 ? a : 1, W, Wsum, t, true, w.x, aoc, decides,
+    const Decision o = decide_node<D>(good ? n : 0, a > 0 ? a : 1, W, Wsum, __dadd_rn(Wsum, W), t, true, w.x, aoc, decides,
                                       decides && force_exact != 0);
     if (!good || j != 0) return;
     const int c = decides ? o.c : 0;

@@ -234,9 +234,9 @@ __device__ __forceinline__ Decision decide_node(int n, int a, double W, double W
     return o;
 }
 
-// Original PERM's decision (Sec. 2, cut-offs T_n, t_n) at a node past the empty walk:
-// copies above T_n, survival with probability 1/q (weight times q) below t_n, one
-// copy between them.
+// Original PERM's decision (Sec. 2, cut-offs T_n, t_n): copies above T_n, survival with
+// probability 1/q (weight times q) below t_n, one copy between them and at the empty
+// walk.
 template <int D>
 __device__ __forceinline__ Decision decide_cutoffs(int n, int a, double W, uint32_t w0, const double *aoc,
                                                    const Cutoffs &cuts) {
@@ -244,7 +244,7 @@ __device__ __forceinline__ Decision decide_cutoffs(int n, int a, double W, uint3
     const double *row = aoc + 48 * scale_row<D>(n) + 8 * (a - 1);
     const double2 tc = __ldg(cuts.cut + n);
     o.exact = false;
-    const bool above = W > tc.x, below = W < tc.y;
+    const bool above = W > tc.x && n > 0, below = W < tc.y && n > 0;      // the empty walk: one copy
     o.c = above ? (cuts.copies < a ? cuts.copies : a) : (below && !((unsigned long long)w0 < cuts.K) ? 0 : 1);
     o.r = above ? (double)cuts.copies : (below ? cuts.inv_q : 1.0);
     o.child_w = __dmul_rn(below && !above ? __dmul_rn(W, cuts.q) : W, row[above ? o.c : 0]);
@@ -519,14 +519,19 @@ __device__ __forceinline__ void grow_run(const RunDev &P, unsigned char *smem, c
     double *Rrow = P.Rn;
     double *acc = Wrow;        // the row this lane adds a node's weight to (lane 0: W_n, lane 1: the tour's sums)
 
-    const bool extras = P.Rn != nullptr || P.cut != nullptr;
+    const bool extras = P.Rn != nullptr || P.trace != nullptr;
     // fresh form: this walk alone reads and writes the table row of its tours (Algorithm 1:
     // one row per sequence, one walk per sequence at a time; else a run of one walk, whose
     // tickets it alone takes, so that M is its own tour's number)
     const bool own_rows = !snapshot && (P.alg == PERM_ALG1 || P.slots == 1);
     const long long t_start = global_ns();
     for (uint32_t iter = 0u;; ++iter) {
-        if ((iter & 7u) == 0u) {
+        // ---------------- everything but the nodes ----------------
+        // Walks that ended their tour are looked after at once, the rest every eighth
+        // iteration: one vote and one branch on the node's way.
+        const bool eighth = (iter & 7u) == 0u;
+        if (eighth || __any_sync(kFull, state == kFlush || (state == kNeed && fresh_need))) {
+        __syncwarp();                           // the walks' regions as the last node left them
         if ((iter & 255u) == 0u) {
             const bool late = global_ns() - t_start > P.max_ns;
             if (__any_sync(kFull, late)) {
@@ -543,9 +548,9 @@ __device__ __forceinline__ void grow_run(const RunDev &P, unsigned char *smem, c
         // Its first lane decides and writes the cell's header; the whole warp copies the
         // sites 0..bdp with the slot that an in-order rebuild would give each, so the
         // taker places them without probing.
-        // (looked at every eighth iteration; the warp's donors reserve their cells together:
+        // (the warp's donors reserve their cells together:
         // a few round trips to L2 and one fence whatever their number)
-        if (snapshot && P.share && __shfl_sync(kFull, *(volatile int *)&head->want_don, 0) > 0) {
+        if (snapshot && P.share && eighth && __shfl_sync(kFull, *(volatile int *)&head->want_don, 0) > 0) {
             // at most `cap` parts of one tour grow at once (a soft cap: the parts of a tour
             // stay few, so each still sees its siblings' samples)
             const bool part = did != 0u || donated;       // the tour has parts elsewhere already
@@ -622,12 +627,6 @@ __device__ __forceinline__ void grow_run(const RunDev &P, unsigned char *smem, c
                 }
             }
         }
-        }
-        // ---------------- walks that ended their tour, or have none ----------------
-        // (looked after at once when a tour has ended; a walk that then found nothing to
-        // grow looks again every eighth iteration: the reads and atomics take several
-        // round trips to L2, which the warp's other walks wait for)
-        if (__any_sync(kFull, state == kFlush || (state == kNeed && (fresh_need || (iter & 7u) == 0u)))) {
         // ---------------- end of a tour (part): per-tour sums into Q (whole warp) ----------------
         if (__any_sync(kFull, state == kFlush)) {
             const bool fl = state == kFlush, whole = did == 0u && !donated;
@@ -727,7 +726,11 @@ __device__ __forceinline__ void grow_run(const RunDev &P, unsigned char *smem, c
             }
             fresh_need = true;
         }
-        // (rows and tickets are global: of old needs they are looked at every 32nd iteration)
+        // ---------------- walks with no tour: tickets, shared copies, leaving ----------------
+        // (a walk that found nothing to grow looks again every eighth iteration, and at
+        // rows and tickets, which are global, every 32nd: the reads and atomics take several
+        // round trips to L2, which the warp's other walks wait for)
+        if (__any_sync(kFull, state == kNeed)) {
         const bool deep = P.alg == PERM_ALG1 || (iter & 31u) == 0u || __any_sync(kFull, state == kNeed && fresh_need);
         fresh_need = false;
         const bool blocked = state == kNeed && xbusy;
@@ -969,14 +972,25 @@ __device__ __forceinline__ void grow_run(const RunDev &P, unsigned char *smem, c
             if (state == kNeed && exhausted && ((go & 1) || (!xbusy && (go & 2)))) state = kDone;
         }
         }
+        // the tours started, as the walks' nodes see them until the next look
+        if (snapshot) {
+            const unsigned long long Ms = __shfl_sync(kFull, *(volatile unsigned long long *)&head->Ms, 0);
+            const unsigned long long Mn = Ms > g + 1ull ? Ms : g + 1ull;
+            if (Mn != tours.M) set_tours(tours, Mn);
+        } else if (g + 1ull != tours.M && own_rows) {
+            set_tours(tours, g + 1ull);
+        }
         if (!__any_sync(kFull, state == kNode || state == kUnwindState)) {
             // nothing to grow: the warp backs off, or leaves
             if (!__any_sync(kFull, state != kDone)) break;
             __nanosleep(idle_ns);
             idle_ns = idle_ns < 4000u ? 2u * idle_ns : 4000u;
             fresh_need = true;
+            iter |= 7u;                         // (so that the next look is a full one)
             ++my_iters;
             continue;
+        }
+        idle_ns = 500u;
         }
         ++my_iters;
 
@@ -986,17 +1000,13 @@ __device__ __forceinline__ void grow_run(const RunDev &P, unsigned char *smem, c
         // and a branch on it.
         {
             __syncwarp();                       // the walks' hashes as the last iteration left them
-            // (two loads of the whole warp right after the barrier, one instruction each: the
-            // lanes of a group read the same value while the refresher writes)
-            unsigned long long Mn = g + 1ull;
+            const bool isn = state == kNode, grows_on = isn && n < P.n_max;
+            // the sum of the weights recorded at this length before the node (a load of the
+            // whole warp right after the barrier: one instruction, so the lanes of a group read
+            // the same value while the refresher writes)
             double Wsum = 0.0;
-            const bool isn = state == kNode;
-            if (snapshot) {
-                const unsigned long long Ms = *(volatile unsigned long long *)&head->Ms;
-                Wsum = *(volatile double *)&Wsnap[n];
-                Mn = Ms > Mn ? Ms : Mn;
-            }
-            const bool grows_on = isn && n < P.n_max;
+            if (snapshot) Wsum = *(volatile double *)&Wsnap[n];
+            else if (own_rows) Wsum = Wrow[n];
             // a_+ (Sec. 1): lane j of the group probes neighbour j
             const bool probes = grows_on && j < 2 * D;
             const Key nkey = cur + dkey;
@@ -1005,38 +1015,31 @@ __device__ __forceinline__ void grow_run(const RunDev &P, unsigned char *smem, c
             int place;
             look_bucket(hash, bucket, nkey, hit, full, place);
             // the node's weight goes into the tables with reductions that return nothing, one
-            // lane each (fresh form: the W_n one returns the sum before it)
-            if (snapshot) {
-                red_add(acc + n, W, isn && j < 2);
-            } else if (own_rows) {
-                // no other walk touches the row: a plain load (of the whole group) and store
-                // (of its first lane) through L1, not an atomic's round trip to L2 (1000
-                // cycles of a lone walk's 3300 a node)
-                Wsum = Wrow[n];
-                red_add(acc + n, W, isn && j == 1);
-            } else {
+            // lane each.  Fresh form: a row of the walk's own takes a load (of the whole group)
+            // and a store (of its first lane) through L1; on a shared one the add returns the
+            // sum before it, a round trip to L2
+            if (!snapshot && !own_rows) {
                 double before = 0.0;
                 unsigned long long Mt = 0ull;
                 if (isn && first) {
                     before = atomicAdd(&Wrow[n], W);
                     Mt = *(volatile unsigned long long *)P.tickets;
                 }
-                red_add(acc + n, W, isn && j == 1);
                 Wsum = __shfl_sync(kFull, before, lead);
                 Mt = __shfl_sync(kFull, Mt, lead);
                 if ((long long)Mt > limit) Mt = (unsigned long long)limit;
-                Mn = Mt > Mn ? Mt : Mn;
+                Mt = Mt > g + 1ull ? Mt : g + 1ull;
+                if (isn && Mt != tours.M) set_tours(tours, Mt);
             }
+            red_add(acc + n, W, isn && (snapshot ? j < 2 : j == 1));
+            red_inc(Srow + n, isn && j == 2);
             const double sum = __dadd_rn(Wsum, W);
             if (!snapshot && own_rows && isn && first) Wrow[n] = sum;
-            red_inc(Srow + n, isn && j == 2);
-            maxn = (isn && n > maxn) ? n : maxn;
-            // a full bucket without the key, a used-up block of random words, a new M: one
-            // vote for the three
+            // a full bucket without the key, a used-up block of random words: one vote for both
             bool more = probes && full && !hit;
-            if (__any_sync(kFull, isn && (more || ord - pbase >= (uint32_t)G || Mn != tours.M))) {
-                if (isn && Mn != tours.M) set_tours(tours, Mn);
-                if (__any_sync(kFull, isn && ord - pbase >= (uint32_t)G)) {
+            const bool refill = isn && ord - pbase >= (uint32_t)G;
+            if (__any_sync(kFull, more || refill)) {
+                if (__any_sync(kFull, refill)) {
                     pbase = ord;
                     if (isn && ord >= 0xFFFFFFF0u) set_status(P.status, PERM_EOVERFLOW);
                     const Philox4 w = philox4x32_10(ord + (uint32_t)j, did, tour, seq, P.key0, P.key1);
@@ -1060,29 +1063,28 @@ __device__ __forceinline__ void grow_run(const RunDev &P, unsigned char *smem, c
             // the node's random words, from the lane that holds its block
             const int wl = lead + (int)((ord - pbase) & (uint32_t)(G - 1));
             const uint32_t w0 = __shfl_sync(kFull, pw0, wl), w1 = __shfl_sync(kFull, pw1, wl);
-            Decision o = decide_node<D>(n, a1, W, Wsum, sum, tours, !snapshot, w0, aoc, decides && !cutoffs, false);
-            if (extras) {
-                if (cutoffs && n > 0) o = decide_cutoffs<D>(n, a1, W, w0, aoc, cuts);
-                if (P.Rn != nullptr) {
-                    // the observable of Sec. 1, eq. 5: W |omega_n|^2 (exact integer square)
-                    int cx, cy, cz;
-                    KeyCodec<D, Key>::decode(cur, cx, cy, cz);
-                    const long long r2 = (long long)cx * cx + (long long)cy * cy + (long long)cz * cz;
-                    red_add(Rrow + n, __dmul_rn(W, (double)r2), isn && j == 3);
-                }
-            }
-            const int c = decides ? o.c : 0;
-            if (o.exact && decides) my_exact += 1ull;
-            // the first child's step, its key and its place in the hash, from the lane that probed it
-            uint32_t list = lists[fm], xw = w1;
-            choose_step(0, a1, list, xw);
-            const int dir0 = (int)(list & 7u);
+            // the first child's step (a draw from the free list), its key and its place in the
+            // hash, from the lane that probed it
+            const uint32_t list = lists[fm];
+            const unsigned long long prod = (unsigned long long)w1 * (uint32_t)a1;
+            const int dir0 = (int)((list >> (3 * (int)(prod >> 32))) & 7u);
             const Key ckey = __shfl_sync(kFull, nkey, lead + dir0);
             const int cslot = __shfl_sync(kFull, nslot, lead + dir0);
-            if (c > 1)
-                for (int i = 1; i < c; ++i) choose_step(i, a, list, xw);
-            const uint32_t dirs = list;
+            Decision o;
+            if (cutoffs) o = decide_cutoffs<D>(n, a1, W, w0, aoc, cuts);
+            else o = decide_node<D>(n, a1, W, Wsum, sum, tours, !snapshot, w0, aoc, decides, false);
+            const int c = decides ? o.c : 0;
+            if (o.exact && decides) my_exact += 1ull;
+            const bool extend = c > 0, leaf = isn && c == 0;
 
+            if (extras) {
+            if (P.Rn != nullptr) {
+                // the observable of Sec. 1, eq. 5: W |omega_n|^2 (exact integer square)
+                int cx, cy, cz;
+                KeyCodec<D, Key>::decode(cur, cx, cy, cz);
+                const long long r2 = (long long)cx * cx + (long long)cy * cy + (long long)cz * cz;
+                red_add(Rrow + n, __dmul_rn(W, (double)r2), isn && j == 3);
+            }
             const unsigned long long ordinal = ((unsigned long long)did << 32) | ord;
             if (P.trace != nullptr && isn && first && (ordinal % (unsigned long long)P.trace_every) == 0ull &&
                 ((unsigned long long)tour % (unsigned long long)P.trace_tour_every) == 0ull) {
@@ -1092,6 +1094,8 @@ __device__ __forceinline__ void grow_run(const RunDev &P, unsigned char *smem, c
                     rec->n = n; rec->a_plus = a; rec->free_mask = fm; rec->c = c;
                     rec->outcome = !grows_on ? kLeafNmax : (a == 0 ? kTrapped : (c == 0 ? kPruned : kChildren));
                     rec->exact = decides && o.exact ? 1 : 0;
+                    uint32_t dirs = list, xw = w1;
+                    for (int i = 0; i < c; ++i) choose_step(i, a, dirs, xw);
                     for (int i = 0; i < 6; ++i)
                         rec->dirs[i] = (i < c) ? (int)((dirs >> (3 * i)) & 7u) : -1;
                     rec->seq = seq; rec->tour = tour;
@@ -1106,10 +1110,14 @@ __device__ __forceinline__ void grow_run(const RunDev &P, unsigned char *smem, c
                     }
                 }
             }
+            }
 
             if (c > 1) {
-                // copies 1..c-1 wait in one record (depth, count, steps, weight)
+                // copies 1..c-1 wait in one record (depth, count, steps, weight): the first
+                // draw's exchange, then the others'
                 const unsigned gmask = ((1u << G) - 1u) << lead;
+                uint32_t dirs = list, xw = w1;
+                for (int i = 0; i < c; ++i) choose_step(i, a, dirs, xw);
                 my_copies += (unsigned long long)(c - 1);
                 if (top - sbase == K) {
                     // ring full: the oldest kChunk records go to global memory
@@ -1136,7 +1144,6 @@ __device__ __forceinline__ void grow_run(const RunDev &P, unsigned char *smem, c
                 }
             }
             ord += isn ? 1u : 0u;
-            const bool extend = c > 0, leaf = isn && c == 0;
             cur = extend ? ckey : cur;
             W = extend ? o.child_w : W;
             const int n_leaf = n;
@@ -1152,6 +1159,7 @@ __device__ __forceinline__ void grow_run(const RunDev &P, unsigned char *smem, c
             if (leaf || state == kUnwindState) {
                 const unsigned gmask = ((1u << G) - 1u) << lead;
                 if (leaf) {
+                    maxn = n_leaf > maxn ? n_leaf : maxn;
                     if (top == sbase && sbase > bot) {
                         // ring empty: bring back up to kChunk records, the group's lanes side by side
                         const int lo = sbase - kChunk > bot ? sbase - kChunk : bot;
@@ -1222,7 +1230,6 @@ __device__ __forceinline__ void grow_run(const RunDev &P, unsigned char *smem, c
                     }
                 }
             }
-            __syncwarp();
         }
     }
     if (P.share && lane == 0 && my_hungry != 0) atomicAdd(P.hungry, -my_hungry);

@@ -210,7 +210,7 @@ int perm_batch_create_persistent(perm_batch_handle *out, const perm_config *cfgs
         for (int r = 0; rc == PERM_OK && r < R; ++r) rc = perm::member_reset(b->runs[r]);
         if (rc == PERM_OK && perm::launch_batch(B, grid, threads, smem, b->origin) != cudaSuccess) rc = PERM_EDEVICE;
         for (int r = 0; rc == PERM_OK && r < R; ++r)
-            if (perm::launch_finalize(P[r].tickets, P[r].tour_limit, b->origin) != cudaSuccess) rc = PERM_EDEVICE;
+            if (perm::launch_finalize(P[r], b->origin) != cudaSuccess) rc = PERM_EDEVICE;
         cudaGraph_t g = nullptr;
         const cudaError_t ec = cudaStreamEndCapture(b->origin, &g);
         if (rc == PERM_OK && ec != cudaSuccess) rc = PERM_EDEVICE;
@@ -285,7 +285,7 @@ int perm_batch_continue(perm_batch_handle b, const int64_t *extra_tours_per_seq)
         B.max_ns = b->max_ns;
         if (perm::launch_batch(B, b->grid, b->threads, b->smem, b->origin) != cudaSuccess) return PERM_EDEVICE;
         for (int r = 0; r < b->R; ++r)
-            if (perm::launch_finalize(P[r].tickets, P[r].tour_limit, b->origin) != cudaSuccess) return PERM_EDEVICE;
+            if (perm::launch_finalize(P[r], b->origin) != cudaSuccess) return PERM_EDEVICE;
         if (cudaStreamSynchronize(b->origin) != cudaSuccess) return PERM_EDEVICE;
     }
     for (perm_handle h : b->runs) {

@@ -39,6 +39,7 @@ struct perm_run_s {
     unsigned long long *Sn = nullptr, *tickets = nullptr, *seq_M = nullptr;
     unsigned long long *steps = nullptr, *max_stack = nullptr, *copies = nullptr, *refreshes = nullptr, *trace_count = nullptr;
     unsigned long long *iterations = nullptr, *finished = nullptr, *exact_steps = nullptr;
+    long long *admit = nullptr;    // admission of new tours (two counts)
     uint32_t *gstk_meta = nullptr;
     int *status = nullptr;
     // shared copies
@@ -84,7 +85,7 @@ int dalloc(perm_handle h, T **p, size_t count) {
 
 void free_all(perm_handle h) {
     void *ptrs[] = {h->Wn, h->Qn, h->Rn, h->X, h->gstk_w, h->Sn, h->tickets, h->seq_M, h->steps,
-                    h->max_stack, h->copies, h->refreshes, h->iterations, h->finished, h->exact_steps,
+                    h->max_stack, h->copies, h->refreshes, h->iterations, h->finished, h->exact_steps, h->admit,
                     h->trace_count, h->gstk_meta, h->status, h->trace,
                     h->trace_coords, h->dq_cells, h->dq_head, h->dq_tail, h->dq_ready, h->dq_free, h->outst,
                     h->tmaxn, h->hungry, h->cut, h->arena};
@@ -347,6 +348,7 @@ int create_impl(perm_handle *out, const perm_config *cfg, const ForcedLayout *fo
     if (rc == PERM_OK) rc = dalloc(h, &h->iterations, 1);
     if (rc == PERM_OK) rc = dalloc(h, &h->finished, 1);
     if (rc == PERM_OK) rc = dalloc(h, &h->exact_steps, 1);
+    if (rc == PERM_OK) rc = dalloc(h, &h->admit, 2);
     if (rc == PERM_OK) rc = dalloc(h, &h->trace_count, 1);
     if (rc == PERM_OK) rc = dalloc(h, &h->status, 1);
     // shared copies: a ring of cells, each one waiting copy record plus the keys of the
@@ -421,6 +423,7 @@ static RunDev make_params(perm_handle h) {
     P.steps = h->steps; P.max_stack = h->max_stack; P.copies = h->copies; P.refreshes = h->refreshes; P.iterations = h->iterations;
     P.exact_steps = h->exact_steps;
     P.finished = h->finished;
+    P.admit = h->admit;
     P.ramp_c0 = h->cfg.ramp_c0 < 0 ? -1 : (long long)h->cfg.ramp_c0;
     P.ramp_gamma_q16 = (unsigned long long)(h->cfg.ramp_gamma * 65536.0);
     P.share = h->share ? h->share_cap : 0;
@@ -487,7 +490,7 @@ int perm_run(perm_handle h, int64_t tours_per_seq) {
     e = perm::launch_grow(P, h->thresh, h->key64, h->ctas, h->stream);
     if (e != cudaSuccess) return to_code(e);
     if (h->cfg.alg == PERM_ALG2) {
-        e = perm::launch_finalize(h->tickets, h->tour_limit, h->stream);
+        e = perm::launch_finalize(P, h->stream);
         if (e != cudaSuccess) return to_code(e);
     }
     return PERM_OK;
@@ -557,6 +560,7 @@ int perm_reset(perm_handle h) {
     if (e == cudaSuccess) e = cudaMemsetAsync(h->refreshes, 0, sizeof(unsigned long long), h->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(h->iterations, 0, sizeof(unsigned long long), h->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(h->finished, 0, sizeof(unsigned long long), h->stream);
+    if (e == cudaSuccess) e = cudaMemsetAsync(h->admit, 0, 2 * sizeof(long long), h->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(h->exact_steps, 0, sizeof(unsigned long long), h->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(h->max_stack, 0, sizeof(unsigned long long), h->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(h->status, 0, sizeof(int), h->stream);
@@ -954,6 +958,11 @@ int perm_load(perm_handle *out, const char *path) {
                                   h->exact_steps, h->tickets};
     for (int i = 0; e == cudaSuccess && i < 8; ++i)
         e = cudaMemcpyAsync(dev[i], &vals[i], 8, cudaMemcpyHostToDevice, h->stream);
+    if (e == cudaSuccess && hd.cfg.alg == PERM_ALG2) {
+        // every saved tour has finished: the admission count as a launch leaves it
+        h->tour_limit = hd.tour_limit;
+        e = perm::launch_finalize(make_params(h), h->stream);
+    }
     if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
     if (e != cudaSuccess) { perm_destroy(h); return to_code(e); }
     h->tour_limit = hd.tour_limit;

@@ -49,7 +49,7 @@ namespace perm {
 namespace {
 
 constexpr int kUnwindSites = 16;   // hash deletions per walk per iteration
-constexpr int kPoolExtra = 4;      // extra tour tickets fetched per warp (snapshot)
+constexpr int kPoolExtra = 2;      // extra tour tickets fetched per warp (snapshot): M counts them as started
 constexpr int kChunk = 8;          // stack records moved per spill or fill (ring >= 2 kChunk)
 constexpr int kReloadBatch = 8;    // snapshot entries a refresher lane loads before storing them
 constexpr unsigned kRowFree = 0xFFFFFFFFu;   // outst: the walk's tour-sum row is unused
@@ -168,22 +168,35 @@ __device__ __forceinline__ void set_tours(Tours &t, unsigned long long M) {
 
 struct Decision {
     int c;               // copies (0: pruned)
-    double r;            // r as the decision used it (single-precision estimate or exact)
-    double child_w;
     bool exact;          // the decision was taken on r in double precision
+    float x;             // the estimate of r, and r itself where it was evaluated
+    double r;            // (cut-offs: in both forms what the cut-off stands for)
+    double child_w;
 };
+// r as the decision used it.
+__device__ __forceinline__ double decision_r(const Decision &o, int n, bool cutoffs) {
+    return o.exact || cutoffs ? o.r : (n == 0 ? 1.0 : widen(o.x));
+}
 
-// r exactly as defined and the decision on it (out of line: one node in 10^4 or fewer).
-__device__ __noinline__ Decision decide_node_exact(int a, double W, double Wsum, unsigned long long M, uint32_t w0,
-                                                   double a_sc) {
+// r exactly as defined and the decision on it.  avg: the running average (Wsum + W)/M,
+// correctly rounded.
+__device__ __forceinline__ Decision decide_on_average(int a, double W, double avg, uint32_t w0, double a_sc) {
     Decision o;
     bool surv = false;
     o.exact = true;
-    o.r = ratio_exact(W, Wsum, M);
+    o.x = 0.0f;
+    o.r = 1.0;
+    if (!(avg == W && W > 0.0)) o.r = __ddiv_rn(W, avg);         // (W/W = 1: no division)
     o.c = decide_exact(o.r, a, w0, surv);
     if (surv) o.child_w = __dmul_rn(__dmul_rn(W, __ddiv_rn(1.0, o.r)), a_sc);
-    else o.child_w = __dmul_rn(__ddiv_rn(W, (double)(o.c > 0 ? o.c : 1)), a_sc);
+    else o.child_w = o.c > 1 ? __dmul_rn(__ddiv_rn(W, (double)o.c), a_sc) : __dmul_rn(W, a_sc);
     return o;
+}
+// Snapshot form: one node in 10^4 or fewer, out of line (inline it costs the other nodes
+// 5 %, by their registers).
+__device__ __noinline__ Decision decide_node_exact(int a, double W, double sum, unsigned long long M, uint32_t w0,
+                                                   double a_sc) {
+    return decide_on_average(a, W, __ddiv_rn(sum, __ull2double_rn(M)), w0, a_sc);
 }
 
 // The decision at a node with a >= 1 free neighbours (Sec. 2): r, the copies, the
@@ -201,7 +214,8 @@ __device__ __forceinline__ Decision decide_node(int n, int a, double W, double W
     o.exact = false;
     bool odd = false, amb = false, surv = false;
     const float x = ratio_estimate(W, Wsum, t.Mf, odd);
-    o.r = n == 0 ? 1.0 : widen(x);
+    o.x = x;
+    o.r = 0.0;
     const int dE = scale_row<D>(n) + (D == 2 ? 1 : 2);
     const double *row = aoc + 48 * (dE - (D == 2 ? 1 : 2)) + 8 * (a - 1);
     int c = decide_estimate(x, a, w0, surv, amb);
@@ -214,14 +228,14 @@ __device__ __forceinline__ Decision decide_node(int n, int a, double W, double W
     // is far from the subnormals); the weight is within 2^-51 of the quotient
     double base = W, fac = row[c];
     if (refine) {
-        // q = sum (1/M), then q + (sum - q M)/M: the quotient to half a unit
-        // (before the decision is known: its four dependent operations run beside it)
-        const double q = __dmul_rn(sum, t.inv1);
-        const double avg = __fma_rn(__fma_rn(-q, t.Md, sum), t.inv1, q);
-        base = surv ? avg : W;
-        fac = surv ? row[0] : fac;
+        if (surv) {
+            // q = sum (1/M), then q + (sum - q M)/M: the quotient to half a unit
+            const double q = __dmul_rn(sum, t.inv1);
+            base = __fma_rn(__fma_rn(-q, t.Md, sum), t.inv1, q);
+            fac = row[0];
+        }
     } else {
-        const double f0 = a == 3 ? t.inv3 : (a == 5 ? t.inv5 : t.inv1);
+        const double f0 = a == 3 ? t.inv3 : (D == 3 && a == 5 ? t.inv5 : t.inv1);
         const int sh = (a == 2 ? 1 : (a == 4 ? 2 : 0)) - dE;
         const double fs = __hiloint2double(__double2hiint(f0) + (sh << 20), __double2loint(f0));
         base = surv ? sum : W;
@@ -230,7 +244,19 @@ __device__ __forceinline__ Decision decide_node(int n, int a, double W, double W
     o.child_w = __dmul_rn(base, fac);
     o.c = c;
     // the estimate cannot settle a comparison: r exactly as defined
-    if (exact) o = decide_node_exact(a, W, Wsum, t.M, w0, row[0]);
+    if (exact && refine) {
+        // fresh form (of a lone sequence the lengths n <= 3 come here at every tour: every
+        // weight is the same and r = 1 exactly).  The average by one step of the division
+        // from the correctly rounded 1/M (M below 2^32, the sum far from the range's ends),
+        // else by the division itself
+        const double q = __dmul_rn(sum, t.inv1);
+        double avg = __fma_rn(__fma_rn(-q, t.Md, sum), t.inv1, q);
+        const int es = __double2hiint(sum) >> 20;
+        if (odd || es < 128 || es > 1920) avg = __ddiv_rn(sum, t.Md);
+        o = decide_on_average(a, W, avg, w0, row[0]);
+    } else if (exact) {
+        o = decide_node_exact(a, W, sum, t.M, w0, row[0]);
+    }
     return o;
 }
 
@@ -244,6 +270,7 @@ __device__ __forceinline__ Decision decide_cutoffs(int n, int a, double W, uint3
     const double *row = aoc + 48 * scale_row<D>(n) + 8 * (a - 1);
     const double2 tc = __ldg(cuts.cut + n);
     o.exact = false;
+    o.x = 0.0f;
     const bool above = W > tc.x && n > 0, below = W < tc.y && n > 0;      // the empty walk: one copy
     o.c = above ? (cuts.copies < a ? cuts.copies : a) : (below && !((unsigned long long)w0 < cuts.K) ? 0 : 1);
     o.r = above ? (double)cuts.copies : (below ? cuts.inv_q : 1.0);
@@ -309,6 +336,36 @@ constexpr int kStalledBit = 4;
 // that the walks' hashes, site lists and stacks are reached by shared-memory
 // instructions rather than generic ones (a generic load that lands in shared
 // memory waits longer, and in the long-scoreboard queue).
+// Admission (Algorithm 2): tours in flight stay at most c0 + gamma * finished, i.e.
+// tickets at most c0 + f + gamma f.  admit[0] counts the admitted tours not yet taken
+// (c0 apart), admit[1] is the f + gamma f that went into it.  A warp takes what it
+// wants from the count and gives back what was not there; one that comes short brings
+// the count up to date with f.  `again`: the warp asks for walks that waited already,
+// so the count may be short: it looks before it takes (a thousand idle warps taking and
+// giving back would hide the few admitted tours from each other).  No retries: with a
+// compare-and-swap on the tickets a thousand warps got 3 grants per microsecond
+// together, and short tours waited for them (square n = 16, 4096 sequences, 40 tours
+// each: 27 ms, now 3.4).
+__device__ unsigned long long admitted(const RunDev &P, unsigned long long want, bool again) {
+    unsigned long long *left = reinterpret_cast<unsigned long long *>(P.admit);
+    for (int attempt = 0; attempt < 2; ++attempt) {
+        const long long k = (long long)want;
+        if (!again || (long long)*(volatile unsigned long long *)left + P.ramp_c0 > 0) {
+            const long long had = (long long)atomicAdd(left, 0ull - want) + P.ramp_c0;
+            const long long got = had < 0 ? 0 : (had < k ? had : k);
+            if (got < k) atomicAdd(left, (unsigned long long)(k - got));
+            if (got > 0) return (unsigned long long)got;
+        }
+        if (attempt > 0) break;
+        const unsigned long long f = *(volatile unsigned long long *)P.finished;
+        const unsigned long long now = f + ((f * P.ramp_gamma_q16) >> 16);
+        const unsigned long long was = atomicMax(left + 1, now);
+        if (now <= was) break;
+        atomicAdd(left, now - was);
+    }
+    return 0ull;
+}
+
 template <int D> constexpr int kGroupLanes = D == 2 ? 4 : 8;   // lanes that hold one walk
 
 template <int D, typename Key, int MODE, bool SHARED>
@@ -350,10 +407,13 @@ __device__ __forceinline__ void grow_run(const RunDev &P, unsigned char *smem, c
     fill_constants(aoc, D, threadIdx.x, blockDim.x);
     const long long limit = P.tour_limit;
     if (snapshot) {
-        unsigned long long Ms = *(volatile unsigned long long *)P.tickets;
-        if ((long long)Ms > limit) Ms = (unsigned long long)limit;
         for (int k = threadIdx.x; k < L; k += blockDim.x) Wsnap[k] = *(volatile double *)(P.Wn + k);
-        if (threadIdx.x == 0) head->Ms = Ms;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            unsigned long long Ms = *(volatile unsigned long long *)P.tickets;     // after the sums, as below
+            if ((long long)Ms > limit) Ms = (unsigned long long)limit;
+            head->Ms = Ms;
+        }
     }
     __syncthreads();
 
@@ -374,8 +434,7 @@ __device__ __forceinline__ void grow_run(const RunDev &P, unsigned char *smem, c
                 if (lane == 0) atomicAdd(P.refreshes, (unsigned long long)it);
                 break;
             }
-            unsigned long long Ms = *(volatile unsigned long long *)P.tickets;
-            if ((long long)Ms > limit) Ms = (unsigned long long)limit;
+            unsigned long long Ms = 0ull;
             for (int k0 = 0; k0 < L; k0 += 32 * kReloadBatch) {
                 double v[kReloadBatch];
 #pragma unroll
@@ -383,13 +442,25 @@ __device__ __forceinline__ void grow_run(const RunDev &P, unsigned char *smem, c
                     const int k = k0 + j * 32 + lane;
                     v[j] = k < L ? ld_relaxed(P.Wn + k) : 0.0;
                 }
+                if (k0 == 0) {
+                    // M read after the sums of the shortest lengths and published before them, so
+                    // that M counts every tour whose weights a node finds in them: with M older
+                    // than the sums r falls below 1 at n = 1, where every tour has the same
+                    // weight, and prunes some (the only way that c_2 can get an error at all)
+                    __threadfence();
+                    Ms = *(volatile unsigned long long *)P.tickets;
+                    if ((long long)Ms > limit) Ms = (unsigned long long)limit;
+                    Ms = __shfl_sync(kFull, Ms, 0);
+                    if (lane == 0) *(volatile unsigned long long *)&head->Ms = Ms;
+                    __threadfence_block();
+                    __syncwarp();
+                }
 #pragma unroll
                 for (int j = 0; j < kReloadBatch; ++j) {
                     const int k = k0 + j * 32 + lane;
                     if (k < L) *(volatile double *)&Wsnap[k] = v[j];
                 }
             }
-            if (lane == 0) *(volatile unsigned long long *)&head->Ms = Ms;
             if (P.share && lane == 0) {
                 // idle walks not yet served by a queued copy, split over the CTAs
                 const long long hg = *(volatile int *)P.hungry;
@@ -505,14 +576,13 @@ __device__ __forceinline__ void grow_run(const RunDev &P, unsigned char *smem, c
     bool exhausted = (bl != nullptr && bl->helper) || sidx >= P.tour_slots;
     int my_hungry = 0;         // this warp's share of P.hungry
     unsigned idle_ns = 500u;   // back-off of a warp with nothing to grow
-    int frow = 0, fmaxn = 0;   // tour-sum row to flush at a part's end, and its depth
-    bool do_flush = false, shared_flush = false;
     const uint32_t dq_mask = (1u << P.dq_log2cap) - 1u;
     // a donation cell: 32-byte header, the keys of sites 0..n_max, then their slots
     const size_t cell_key_bytes = align16(((size_t)P.n_max + 1) * sizeof(Key));
     unsigned long long my_iters = 0ull;
     Tours tours;               // tours started as this walk's nodes see them
     set_tours(tours, 1ull);
+    uint32_t ms_low = 0u;      // the low word of the snapshot's M as last taken
     bool fresh_need = true;    // the walk has ended its tour since it last looked for work
     double *Wrow = P.Wn;
     unsigned long long *Srow = P.Sn;
@@ -524,6 +594,30 @@ __device__ __forceinline__ void grow_run(const RunDev &P, unsigned char *smem, c
     // one row per sequence, one walk per sequence at a time; else a run of one walk, whose
     // tickets it alone takes, so that M is its own tour's number)
     const bool own_rows = !snapshot && (P.alg == PERM_ALG1 || P.slots == 1);
+    // start tour g at the empty walk (Sec. 1: W(empty) = 1); the walk's hash is empty, so
+    // the origin takes the first place of its home bucket
+    auto start_tour = [&]() {
+        if (P.alg == PERM_ALG1) {
+            seq = (uint32_t)cur_seq;
+            tour = (uint32_t)g;
+        } else if ((g >> 32) == 0ull) {            // (a 64-bit division takes three times as long)
+            tour = (uint32_t)g / (uint32_t)P.n_seq;
+            seq = (uint32_t)g - tour * (uint32_t)P.n_seq;
+        } else {
+            seq = (uint32_t)(g % (unsigned long long)P.n_seq);
+            tour = (uint32_t)(g / (unsigned long long)P.n_seq);
+        }
+        n = 0; cur = origin; maxn = 0; W = 1.0; ord = 0u; pbase = (uint32_t)-G;
+        top = 0; sbase = 0; bot = 0;
+        own = myrow; did = 0u; donated = false;
+        acc = first ? Wrow : P.X + (size_t)own * L;
+        if (first) {
+            const uint32_t s0 = hash_home(origin, log2b) * (uint32_t)Buckets<Key>::kKeys;
+            hash[s0] = origin;
+            sites[0] = (uint16_t)s0;
+        }
+        state = kNode;
+    };
     const long long t_start = global_ns();
     for (uint32_t iter = 0u;; ++iter) {
         // ---------------- everything but the nodes ----------------
@@ -630,13 +724,53 @@ __device__ __forceinline__ void grow_run(const RunDev &P, unsigned char *smem, c
         // ---------------- end of a tour (part): per-tour sums into Q (whole warp) ----------------
         if (__any_sync(kFull, state == kFlush)) {
             const bool fl = state == kFlush, whole = did == 0u && !donated;
-            // empty the ended walks' hashes, the whole warp one walk at a time: every
-            // bucket, or, of a short walk, its sites' slots
+            bool last = fl;                     // with this part the tour has ended
+            int row_max = maxn;                 // the row's deepest length
+            if (__any_sync(kFull, fl && !whole)) {
+                // parts of a tour grew on several walks: this part's sums must be in the row
+                // before the count of its parts says so (a tour that stayed on its walk needs
+                // the warp's own order only), and the last part to end flushes the row
+                __threadfence();
+                __syncwarp();
+                unsigned om = 0u, left = 0u;
+                if (fl && !whole && first) {
+                    om = atomicMax(P.tmaxn + own, (unsigned)maxn);
+                    __threadfence();
+                    left = atomicSub(P.outst + own, 1u);
+                    __threadfence();
+                }
+                __syncwarp();
+                om = __shfl_sync(kFull, om, lead);
+                left = __shfl_sync(kFull, left, lead);
+                bool other_row = false;
+                if (fl && !whole) {
+                    last = left == 1u;
+                    row_max = (int)(om > (unsigned)maxn ? om : (unsigned)maxn);
+                    // the row stays with the parts still growing: the next tour takes the
+                    // walk's other row, if that one is free
+                    other_row = !last && did == 0u;
+                    if (other_row) myrow ^= rows_per_walk - 1;
+                }
+                unsigned row_use = kRowFree;
+                if (other_row && first) row_use = *(volatile unsigned int *)(P.outst + myrow);
+                row_use = __shfl_sync(kFull, row_use, lead);
+                if (other_row) xbusy = row_use != kRowFree;
+            }
+            // the whole warp, one ended walk at a time: the row's sums squared into Q, the
+            // hash emptied (every bucket, or, of a short walk, its sites' slots)
             unsigned em = __ballot_sync(kFull, fl && first);
             while (em) {
                 const int src = __ffs(em) - 1;
                 em &= em - 1u;
                 const int hi = __shfl_sync(kFull, un_hi, src);
+                const int s_row = __shfl_sync(kFull, own, src);
+                const int s_max = __shfl_sync(kFull, last ? row_max : -1, src);
+                const int s_seq = P.alg == PERM_ALG1 ? __shfl_sync(kFull, cur_seq, src) : 0;
+                double *Xr = P.X + (size_t)s_row * L, *Qr = P.Qn + (size_t)s_seq * L;
+                // eight loads in flight per lane, the first of them while the hash is emptied
+                double x[8];
+#pragma unroll
+                for (int u = 0; u < 8; ++u) x[u] = u * 32 + lane <= s_max ? __ldcg(Xr + u * 32 + lane) : 0.0;
                 unsigned char *hb = warp_base + wbytes * (size_t)(src / G);
                 const int vecs = (int)(hash_b / 16);
                 if (vecs <= 2 * (hi + 1)) {
@@ -645,86 +779,58 @@ __device__ __forceinline__ void grow_run(const RunDev &P, unsigned char *smem, c
                     const uint16_t *st = reinterpret_cast<const uint16_t *>(hb + hash_b);
                     for (int i = lane; i <= hi; i += 32) reinterpret_cast<Key *>(hb)[st[i]] = (Key)0;
                 }
-            }
-            if (fl) my_steps += ord;
-            // the sums of a tour whose parts grew on several walks: this part's must be in
-            // the row before the count of its parts says so (a tour that stayed on this
-            // walk needs the warp's own order only)
-            if (__any_sync(kFull, fl && !whole)) __threadfence();
-            __syncwarp();
-            unsigned om = 0u, left = 0u;
-            if (fl && !whole && first) {
-                // parts of the tour grew elsewhere: the last part to end flushes
-                om = atomicMax(P.tmaxn + own, (unsigned)maxn);
-                __threadfence();
-                left = atomicSub(P.outst + own, 1u);
-                __threadfence();
-            }
-            __syncwarp();
-            om = __shfl_sync(kFull, om, lead);
-            left = __shfl_sync(kFull, left, lead);
-            bool other_row = false;
-            if (fl) {
-                frow = own;
-                shared_flush = !whole;
-                do_flush = whole || left == 1u;
-                fmaxn = whole ? maxn : (int)(om > (unsigned)maxn ? om : (unsigned)maxn);
-                // the row stays with the parts still growing: the next tour takes the
-                // walk's other row, if that one is free
-                other_row = !do_flush && did == 0u;
-                if (other_row) myrow ^= rows_per_walk - 1;
-            }
-            unsigned row_use = kRowFree;
-            if (other_row && first) row_use = *(volatile unsigned int *)(P.outst + myrow);
-            row_use = __shfl_sync(kFull, row_use, lead);
-            if (other_row) xbusy = row_use != kRowFree;
-            unsigned flm = __ballot_sync(kFull, fl && do_flush && first);
-            while (flm) {
-                const int src = __ffs(flm) - 1;
-                flm &= flm - 1u;
-                const int s_slot = __shfl_sync(kFull, frow, src);
-                const int s_maxn = __shfl_sync(kFull, fmaxn, src);
-                const int s_seq = __shfl_sync(kFull, cur_seq, src);
-                double *Xr = P.X + (size_t)s_slot * L;
-                double *Qr = (P.alg == PERM_ALG1) ? P.Qn + (size_t)(s_seq < 0 ? 0 : s_seq) * L : P.Qn;
-                // eight loads in flight per lane, then the squares go straight to Q_n
-                for (int k0 = 0; k0 <= s_maxn; k0 += 32 * 8) {
-                    double x[8];
+                for (int k0 = 0; k0 <= s_max;) {
 #pragma unroll
                     for (int u = 0; u < 8; ++u) {
+                        if (k0 + u * 32 > s_max) break;
                         const int k = k0 + u * 32 + lane;
-                        x[u] = (k <= s_maxn) ? __ldcg(Xr + k) : 0.0;
+                        const bool take = __double_as_longlong(x[u]) != 0ll;     // (an integer test: no -0.0 here)
+                        red_add(Qr + k, __dmul_rn(x[u], x[u]), take);
+                        if (take) __stcg(Xr + k, 0.0);
                     }
+                    k0 += 32 * 8;
+                    if (k0 > s_max) break;
 #pragma unroll
-                    for (int u = 0; u < 8; ++u) {
-                        const int k = k0 + u * 32 + lane;
-                        if (__double_as_longlong(x[u]) != 0ll) {     // (an integer test: no -0.0 here)
-                            atomicAdd(&Qr[k], __dmul_rn(x[u], x[u]));
-                            __stcg(Xr + k, 0.0);
-                        }
-                    }
+                    for (int u = 0; u < 8; ++u)
+                        x[u] = k0 + u * 32 + lane <= s_max ? __ldcg(Xr + k0 + u * 32 + lane) : 0.0;
                 }
             }
             __syncwarp();
             if (fl) {
-                if (do_flush) {
-                    if (first) {
-                        if (shared_flush) {
-                            P.tmaxn[frow] = 0u;
-                            __threadfence();       // (after the barrier above: the emptied row too)
-                            *(volatile unsigned int *)(P.outst + frow) = kRowFree;
-                        }
-                        atomicAdd(P.finished, 1ull);
+                my_steps += ord;
+                if (last && first) {
+                    if (!whole) {
+                        P.tmaxn[own] = 0u;
+                        __threadfence();           // (after the barrier above: the emptied row too)
+                        *(volatile unsigned int *)(P.outst + own) = kRowFree;
                     }
-                    if (P.alg == PERM_ALG1) {
-                        seq_t += 1;
-                        if (first) P.seq_M[cur_seq] = (unsigned long long)seq_t;
-                    }
+                    atomicAdd(P.finished, 1ull);
                 }
-                own = myrow; did = 0u; donated = false; do_flush = false;
+                if (P.alg == PERM_ALG1) {
+                    seq_t += 1;
+                    if (first) P.seq_M[cur_seq] = (unsigned long long)seq_t;
+                }
+                own = myrow; did = 0u; donated = false;
                 state = kNeed;
+                fresh_need = true;
             }
-            fresh_need = true;
+            // the next tours at once where they are known: the sequence's next one, or tickets
+            // that the warp holds
+            bool next = fl && !xbusy && !exhausted;
+            if (P.alg == PERM_ALG2) {
+                const unsigned nm = __ballot_sync(kFull, next && first);
+                const unsigned long long cnt = (unsigned long long)__popc(nm);
+                if (pool_hi - pool_lo >= cnt && (long long)(pool_lo + cnt) <= limit) {
+                    if (next) g = pool_lo + (unsigned long long)__popc(nm & lt_mask);
+                    pool_lo += cnt;
+                } else {
+                    next = false;
+                }
+            } else {
+                next = next && seq_t < P.seq_target;
+                if (next) g = (unsigned long long)seq_t;
+            }
+            if (next) start_tour();
         }
         // ---------------- walks with no tour: tickets, shared copies, leaving ----------------
         // (a walk that found nothing to grow looks again every eighth iteration, and at
@@ -759,31 +865,13 @@ __device__ __forceinline__ void grow_run(const RunDev &P, unsigned char *smem, c
                     // fetch tickets; admission keeps tours in flight at most
                     // c0 + gamma * finished (a partial grant is allowed)
                     const int leader = __ffs(need) - 1;
-                    const unsigned long long want = cnt - avail + (snapshot ? (unsigned long long)kPoolExtra : 0ull);
+                    const unsigned long long want = cnt - avail + (snapshot || own_rows ? (unsigned long long)kPoolExtra : 0ull);
+                    // (past the launch's last ticket a walk needs no admission to learn that)
                     if (lane == leader) {
-                        if (P.ramp_c0 < 0) {
-                            base = atomicAdd(P.tickets, want);
-                            take = want;
-                        } else {
-                            for (int attempt = 0; attempt < 64; ++attempt) {
-                                const unsigned long long t_now = *(volatile unsigned long long *)P.tickets;
-                                const unsigned long long f_now = *(volatile unsigned long long *)P.finished;
-                                unsigned long long k = want;
-                                if ((long long)t_now < limit) {
-                                    const unsigned long long allow = (unsigned long long)P.ramp_c0 +
-                                                                     ((f_now * P.ramp_gamma_q16) >> 16);
-                                    const unsigned long long infl = t_now - (f_now < t_now ? f_now : t_now);
-                                    k = allow > infl ? allow - infl : 0ull;
-                                    k = k < want ? k : want;
-                                }
-                                if (k == 0ull) break;
-                                if (atomicCAS(P.tickets, t_now, t_now + k) == t_now) {
-                                    base = t_now;
-                                    take = k;
-                                    break;
-                                }
-                            }
-                        }
+                        const bool over = snapshot ? *(volatile unsigned long long *)&head->Ms >= (unsigned long long)limit
+                                                   : *(volatile unsigned long long *)P.tickets >= (unsigned long long)limit;
+                        take = P.ramp_c0 < 0 || over ? want : admitted(P, want, waiting);
+                        base = over ? (unsigned long long)limit : (take > 0ull ? atomicAdd(P.tickets, take) : 0ull);
                     }
                     base = __shfl_sync(kFull, base, leader);
                     take = __shfl_sync(kFull, take, leader);
@@ -807,14 +895,6 @@ __device__ __forceinline__ void grow_run(const RunDev &P, unsigned char *smem, c
                         else state = kDone;
                         if (bl != nullptr && first && (atomicOr(bl->closed + P.run_index, 1) & 3) == 0)
                             atomicSub(bl->runs_open, 1);
-                    } else {
-                        if ((g >> 32) == 0ull) {           // (a 64-bit division takes several times as long)
-                            tour = (uint32_t)g / (uint32_t)P.n_seq;
-                            seq = (uint32_t)g - tour * (uint32_t)P.n_seq;
-                        } else {
-                            seq = (uint32_t)(g % (unsigned long long)P.n_seq);
-                            tour = (uint32_t)(g / (unsigned long long)P.n_seq);
-                        }
                     }
                 }
             } else {
@@ -835,27 +915,12 @@ __device__ __forceinline__ void grow_run(const RunDev &P, unsigned char *smem, c
                     }
                 }
                 if (state == kNeed && cur_seq >= 0 && seq_t < P.seq_target) {
-                    seq = (uint32_t)cur_seq;
-                    tour = (uint32_t)seq_t;
                     g = (unsigned long long)seq_t;
                 } else if (state == kNeed) {
                     cur_seq = -1;          // sequence finished: ask again next round
                 }
             }
-            if (state == kNeed && !waiting && !xbusy && !exhausted && (P.alg == PERM_ALG2 || cur_seq >= 0)) {
-                // start a tour at the empty walk (Sec. 1: W(empty) = 1); the walk's hash
-                // is empty, so the origin takes the first place of its home bucket
-                n = 0; cur = origin; maxn = 0; W = 1.0; ord = 0u; pbase = (uint32_t)-G;
-                top = 0; sbase = 0; bot = 0;
-                own = myrow; did = 0u; donated = false;
-                acc = first ? Wrow : P.X + (size_t)own * L;
-                if (first) {
-                    const uint32_t s0 = hash_home(origin, log2b) * (uint32_t)Buckets<Key>::kKeys;
-                    hash[s0] = origin;
-                    sites[0] = (uint16_t)s0;
-                }
-                state = kNode;
-            }
+            if (state == kNeed && !waiting && !xbusy && !exhausted && (P.alg == PERM_ALG2 || cur_seq >= 0)) start_tour();
         }
         if (P.share) {
             // ---------------- shared copies: idle walks take queued ones ----------------
@@ -972,14 +1037,7 @@ __device__ __forceinline__ void grow_run(const RunDev &P, unsigned char *smem, c
             if (state == kNeed && exhausted && ((go & 1) || (!xbusy && (go & 2)))) state = kDone;
         }
         }
-        // the tours started, as the walks' nodes see them until the next look
-        if (snapshot) {
-            const unsigned long long Ms = __shfl_sync(kFull, *(volatile unsigned long long *)&head->Ms, 0);
-            const unsigned long long Mn = Ms > g + 1ull ? Ms : g + 1ull;
-            if (Mn != tours.M) set_tours(tours, Mn);
-        } else if (g + 1ull != tours.M && own_rows) {
-            set_tours(tours, g + 1ull);
-        }
+        if (snapshot ? g + 1ull > tours.M : own_rows && g + 1ull != tours.M) set_tours(tours, g + 1ull);
         if (!__any_sync(kFull, state == kNode || state == kUnwindState)) {
             // nothing to grow: the warp backs off, or leaves
             if (!__any_sync(kFull, state != kDone)) break;
@@ -1005,8 +1063,13 @@ __device__ __forceinline__ void grow_run(const RunDev &P, unsigned char *smem, c
             // whole warp right after the barrier: one instruction, so the lanes of a group read
             // the same value while the refresher writes)
             double Wsum = 0.0;
-            if (snapshot) Wsum = *(volatile double *)&Wsnap[n];
-            else if (own_rows) Wsum = Wrow[n];
+            uint32_t m_low = ms_low;            // low word of the snapshot's M: whether it changed
+            if (snapshot) {
+                Wsum = *(volatile double *)&Wsnap[n];
+                m_low = *(volatile uint32_t *)&head->Ms;
+            } else if (own_rows) {
+                Wsum = Wrow[n];
+            }
             // a_+ (Sec. 1): lane j of the group probes neighbour j
             const bool probes = grows_on && j < 2 * D;
             const Key nkey = cur + dkey;
@@ -1035,10 +1098,17 @@ __device__ __forceinline__ void grow_run(const RunDev &P, unsigned char *smem, c
             red_inc(Srow + n, isn && j == 2);
             const double sum = __dadd_rn(Wsum, W);
             if (!snapshot && own_rows && isn && first) Wrow[n] = sum;
-            // a full bucket without the key, a used-up block of random words: one vote for both
+            // a full bucket without the key, a used-up block of random words, a new M: one vote
+            // for the three
             bool more = probes && full && !hit;
             const bool refill = isn && ord - pbase >= (uint32_t)G;
-            if (__any_sync(kFull, more || refill)) {
+            if (__any_sync(kFull, more || refill || m_low != ms_low)) {
+                if (snapshot) {
+                    ms_low = __shfl_sync(kFull, m_low, 0);
+                    const unsigned long long Ms = __shfl_sync(kFull, *(volatile unsigned long long *)&head->Ms, 0);
+                    const unsigned long long Mn = Ms > g + 1ull ? Ms : g + 1ull;
+                    if (Mn != tours.M) set_tours(tours, Mn);
+                }
                 if (__any_sync(kFull, refill)) {
                     pbase = ord;
                     if (isn && ord >= 0xFFFFFFF0u) set_status(P.status, PERM_EOVERFLOW);
@@ -1100,7 +1170,7 @@ __device__ __forceinline__ void grow_run(const RunDev &P, unsigned char *smem, c
                         rec->dirs[i] = (i < c) ? (int)((dirs >> (3 * i)) & 7u) : -1;
                     rec->seq = seq; rec->tour = tour;
                     rec->ordinal = ordinal; rec->M = tours.M;
-                    rec->W = W; rec->Wsum = Wsum; rec->r = o.r; rec->child_w = c > 0 ? o.child_w : 0.0;
+                    rec->W = W; rec->Wsum = Wsum; rec->r = decision_r(o, n, cutoffs); rec->child_w = c > 0 ? o.child_w : 0.0;
                     int32_t *cc = P.trace_coords + (size_t)idx * L * D;
                     for (int k = 0; k <= n; ++k) {
                         int x, y, z;
@@ -1117,31 +1187,36 @@ __device__ __forceinline__ void grow_run(const RunDev &P, unsigned char *smem, c
                 // draw's exchange, then the others'
                 const unsigned gmask = ((1u << G) - 1u) << lead;
                 uint32_t dirs = list, xw = w1;
-                for (int i = 0; i < c; ++i) choose_step(i, a, dirs, xw);
+                choose_step(0, a, dirs, xw);
+                choose_step(1, a, dirs, xw);
+                for (int i = 2; i < c; ++i) choose_step(i, a, dirs, xw);
                 my_copies += (unsigned long long)(c - 1);
-                if (top - sbase == K) {
-                    // ring full: the oldest kChunk records go to global memory
-#pragma unroll
-                    for (int i = 0; i < kChunk; i += G) {
-                        const int idx = sbase + i + j;
-                        gmeta[idx] = smeta[idx & (K - 1)];
-                        gwt[idx] = sw[idx & (K - 1)];
+                if (top - sbase == K || top >= P.n_max) {
+                    // ring full: the oldest kChunk records go to global memory (a walk has at
+                    // most n_max records: their depths increase)
+                    if (top >= P.n_max) {
+                        set_status(P.status, PERM_EOVERFLOW);
+                        top = P.n_max - 1;
                     }
-                    sbase += kChunk;
+                    if (top - sbase == K) {
+#pragma unroll
+                        for (int i = 0; i < kChunk; i += G) {
+                            const int idx = sbase + i + j;
+                            gmeta[idx] = smeta[idx & (K - 1)];
+                            gwt[idx] = sw[idx & (K - 1)];
+                        }
+                        sbase += kChunk;
+                    }
                     __syncwarp(gmask);
                 }
-                if (top >= P.n_max) {
-                    set_status(P.status, PERM_EOVERFLOW);
-                } else {
-                    if (first) {
-                        const uint32_t rest = (dirs >> 3) & ((1u << (3 * (c - 1))) - 1u);
-                        const int ti = top & (K - 1);
-                        smeta[ti] = (uint32_t)n | ((uint32_t)(c - 1) << 16) | (rest << 19);
-                        sw[ti] = o.child_w;
-                    }
-                    ++top;
-                    my_max_stack = top - bot > my_max_stack ? top - bot : my_max_stack;
+                if (first) {
+                    const uint32_t rest = (dirs >> 3) & ((1u << (3 * (c - 1))) - 1u);
+                    const int ti = top & (K - 1);
+                    smeta[ti] = (uint32_t)n | ((uint32_t)(c - 1) << 16) | (rest << 19);
+                    sw[ti] = o.child_w;
                 }
+                ++top;
+                my_max_stack = top - bot > my_max_stack ? top - bot : my_max_stack;
             }
             ord += isn ? 1u : 0u;
             cur = extend ? ckey : cur;
@@ -1158,76 +1233,77 @@ __device__ __forceinline__ void grow_run(const RunDev &P, unsigned char *smem, c
             // group's lanes side by side; then the walk resumes.
             if (leaf || state == kUnwindState) {
                 const unsigned gmask = ((1u << G) - 1u) << lead;
+                if (leaf && top == sbase && sbase > bot) {
+                    // ring empty: bring back up to kChunk records, the group's lanes side by side
+                    const int lo = sbase - kChunk > bot ? sbase - kChunk : bot;
+                    for (int idx = lo + j; idx < sbase; idx += G) {
+                        smeta[idx & (K - 1)] = __ldcg(gmeta + idx);
+                        sw[idx & (K - 1)] = __ldcg(gwt + idx);
+                    }
+                    sbase = lo;
+                    __syncwarp(gmask);
+                }
+                // one straight line from here for a group that pops a record, one that ends
+                // its tour and one still deleting (selects; a branch costs more)
+                const bool pops = leaf && top != bot;
+                const int ti = (top - 1) & (K - 1);
+                const uint32_t meta = smeta[ti], rest = meta >> 19;
+                const double rec_w = sw[ti];
+                const int cnt = (int)((meta >> 16) & 7u);
                 if (leaf) {
                     maxn = n_leaf > maxn ? n_leaf : maxn;
-                    if (top == sbase && sbase > bot) {
-                        // ring empty: bring back up to kChunk records, the group's lanes side by side
-                        const int lo = sbase - kChunk > bot ? sbase - kChunk : bot;
-                        for (int idx = lo + j; idx < sbase; idx += G) {
-                            smeta[idx & (K - 1)] = __ldcg(gmeta + idx);
-                            sw[idx & (K - 1)] = __ldcg(gwt + idx);
-                        }
-                        sbase = lo;
-                        __syncwarp(gmask);
-                    }
                     un_hi = n_leaf < P.n_max - 1 ? n_leaf : P.n_max - 1;
-                    state = kFlush;
-                    if (top != bot) {
-                        const int ti = (top - 1) & (K - 1);
-                        const uint32_t meta = smeta[ti];
-                        const int dp = (int)(meta & 0xFFFFu);
-                        const int cnt = (int)((meta >> 16) & 7u);
-                        const uint32_t rest = meta >> 19;
-                        pend_dir = (int)(rest & 7u);
-                        pend_w = sw[ti];
-                        pend_depth = dp;
-                        __syncwarp(gmask);      // every lane has read the record
-                        if (cnt <= 1) --top;
-                        else if (first) smeta[ti] = (uint32_t)dp | ((uint32_t)(cnt - 1) << 16) | ((rest >> 3) << 19);
-                        un_lo = dp + 1;
-                        state = kUnwindState;
-                    }
+                    state = pops ? kUnwindState : kFlush;
                 }
-                if (state == kUnwindState) {
-                    const Key rkey = hash[sites[pend_depth]] + step_key<D, Key>(pend_dir);
-                    constexpr int kUnwind = kUnwindSites / G;
-                    int sl[kUnwind];
+                if (pops) {
+                    pend_dir = (int)(rest & 7u);
+                    pend_w = rec_w;
+                    pend_depth = (int)(meta & 0xFFFFu);
+                    un_lo = pend_depth + 1;
+                    top -= cnt <= 1 ? 1 : 0;
+                }
+                __syncwarp(gmask);              // every lane has read the record
+                if (pops && cnt > 1 && first)
+                    smeta[ti] = (meta & 0xFFFFu) | ((uint32_t)(cnt - 1) << 16) | ((rest >> 3) << 19);
+                const bool back = state == kUnwindState;
+                const Key rkey = hash[sites[back ? pend_depth : 0]] + step_key<D, Key>(pend_dir);
+                constexpr int kUnwind = kUnwindSites / G;
+                int sl[kUnwind];
 #pragma unroll
-                    for (int i = 0; i < kUnwind; ++i) {
-                        const int k = un_hi - j - i * G;
-                        sl[i] = k >= un_lo ? (int)sites[k] : -1;
-                    }
+                for (int i = 0; i < kUnwind; ++i) {
+                    const int k = un_hi - j - i * G;
+                    sl[i] = back && k >= un_lo ? (int)sites[k] : -1;
+                }
 #pragma unroll
-                    for (int i = 0; i < kUnwind; ++i)
-                        if (sl[i] >= 0) hash[sl[i]] = (Key)0;
-                    un_hi -= kUnwindSites;
-                    __syncwarp(gmask);
-                    if (un_hi < un_lo) {
-                        n = pend_depth + 1;
-                        cur = rkey;
-                        W = pend_w;
-                        state = kNode;
-                        if (n < P.n_max) {
-                            // the new end-point's place (every lane of the group looks at the same
-                            // buckets): the first bucket of its sequence that is not full
-                            const uint32_t bmask = (1u << log2b) - 1u;
-                            uint32_t b = hash_home(rkey, log2b);
-                            look_bucket(hash, b, rkey, hit, full, place);
-                            for (uint32_t it = 0u; full && it < bmask; ++it) {
-                                b = (b + it + 1u) & bmask;
-                                look_bucket(hash, b, rkey, hit, full, place);
-                            }
-                            __syncwarp(gmask);
-                            if (full) {
-                                set_status(P.status, PERM_EOVERFLOW);
-                                state = kDone;
-                            } else if (first) {
-                                const uint32_t rs = b * (uint32_t)Buckets<Key>::kKeys + (uint32_t)place;
-                                hash[rs] = rkey;
-                                sites[n] = (uint16_t)rs;
-                            }
-                        }
+                for (int i = 0; i < kUnwind; ++i)
+                    if (sl[i] >= 0) hash[sl[i]] = (Key)0;
+                un_hi -= back ? kUnwindSites : 0;
+                __syncwarp(gmask);
+                // the new end-point's place (every lane of the group looks at the same buckets):
+                // the first bucket of its sequence that is not full
+                const bool resumes = back && un_hi < un_lo;
+                const bool places = resumes && pend_depth + 1 < P.n_max;
+                uint32_t rb = hash_home(rkey, log2b);
+                if (SHARED || places) look_bucket(hash, rb, rkey, hit, full, place);
+                if (places && full) {
+                    const uint32_t bmask = (1u << log2b) - 1u;
+                    for (uint32_t it = 0u; full && it < bmask; ++it) {
+                        rb = (rb + it + 1u) & bmask;
+                        look_bucket(hash, rb, rkey, hit, full, place);
                     }
+                    if (full) set_status(P.status, PERM_EOVERFLOW);
+                }
+                __syncwarp(gmask);              // every lane has looked
+                if (resumes) {
+                    n = pend_depth + 1;
+                    cur = rkey;
+                    W = pend_w;
+                    state = places && full ? kDone : kNode;
+                }
+                if (places && first && !full) {
+                    const uint32_t rs = rb * (uint32_t)Buckets<Key>::kKeys + (uint32_t)place;
+                    hash[rs] = rkey;
+                    sites[n] = (uint16_t)rs;
                 }
             }
         }
@@ -1473,7 +1549,7 @@ __global__ void __launch_bounds__(32) debug_step_kernel(int n_max, int log2h, in
     oi[3] = c;
     for (int i = 0; i < 6; ++i) oi[4 + i] = (i < c) ? (int)((dirs >> (3 * i)) & 7u) : -1;
     oi[10] = decides && o.exact ? 1 : 0;
-    out_r[b] = o.r;
+    out_r[b] = decision_r(o, n, false);
     out_w[b] = c > 0 ? o.child_w : 0.0;
 }
 
@@ -1484,9 +1560,13 @@ __global__ void philox_kernel(int B, const uint32_t *ctr, uint32_t k0, uint32_t 
     out[4 * b] = w.x; out[4 * b + 1] = w.y; out[4 * b + 2] = w.z; out[4 * b + 3] = w.w;
 }
 
-__global__ void finalize_kernel(unsigned long long *tickets, long long limit) {
+__global__ void finalize_kernel(unsigned long long *tickets, long long limit, long long *admit, unsigned long long gamma_q16) {
     if (threadIdx.x == 0 && blockIdx.x == 0) {
         if ((long long)*tickets > limit) *tickets = (unsigned long long)limit;
+        // every tour has finished: what the admission rule leaves beyond them
+        const long long extra = (long long)(((unsigned long long)limit * gamma_q16) >> 16);
+        admit[0] = extra;
+        admit[1] = limit + extra;
     }
 }
 
@@ -1586,8 +1666,8 @@ cudaError_t launch_grow(const RunDev &P, int thresh_mode, bool key64, int ctas, 
                                     : launch_one<3, uint32_t, kFresh>(P, ctas, stream);
 }
 
-cudaError_t launch_finalize(unsigned long long *tickets, long long limit, cudaStream_t stream) {
-    finalize_kernel<<<1, 32, 0, stream>>>(tickets, limit);
+cudaError_t launch_finalize(const RunDev &P, cudaStream_t stream) {
+    finalize_kernel<<<1, 32, 0, stream>>>(P.tickets, P.tour_limit, P.admit, P.ramp_gamma_q16);
     return cudaGetLastError();
 }
 

@@ -60,6 +60,8 @@ struct RunDev {
     unsigned long long *finished;  // Alg. 2: tours finished (admission of new tours)
     long long ramp_c0;             // admission: in flight <= c0 + gamma * finished
     unsigned long long ramp_gamma_q16;
+    long long *admit;              // [0] admitted tours not yet taken, ramp_c0 apart; [1] the admission
+                                   // (finished + gamma * finished) that went into it
     // shared copies (snapshot form of Alg. 2): a walk with no tour to start
     // takes a waiting copy from the bottom of another walk's stack
     int share;                     // 0: off; else the most parts of one tour growing at once
@@ -128,7 +130,8 @@ constexpr int kMaxWalkWarps = 8;
 
 cudaError_t launch_grow(const RunDev &P, int thresh_mode, bool key64, int ctas,
                         cudaStream_t stream);
-cudaError_t launch_finalize(unsigned long long *tickets, long long limit, cudaStream_t stream);
+// After a launch: the ticket counter clamped to M, the admission count of the next one.
+cudaError_t launch_finalize(const RunDev &P, cudaStream_t stream);
 cudaError_t set_smem_limits();
 
 cudaError_t launch_debug_step(int d, int n_max, int B, const int32_t *coords, const int32_t *len,

@@ -41,7 +41,7 @@ def bytes_per_step(d, f):
     return base + 32.0 * f
 
 
-KERNEL_SOURCES = ("perm_kernels.cu", "perm_kernels.cuh", "perm_device.cuh")
+KERNEL_SOURCES = ("perm_grow.cuh", "perm_kernels.cu", "perm_kernels.cuh", "perm_device.cuh")
 
 
 def code_tokens(text):

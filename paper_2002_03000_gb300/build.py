@@ -1,6 +1,6 @@
 """Build libperm.so (the C-ABI library of include/perm.h) for sm_103a, in-tree.
 
-Two translation units are compiled in parallel with nvcc and linked into
+The translation units are compiled in parallel with nvcc and linked into
 paper_2002_03000_gb300/_build/libperm.so.  No torch, no cmake.
 """
 import os
@@ -12,8 +12,9 @@ ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 OUT_DIR = os.path.join(HERE, "_build")
 LIB = os.path.join(OUT_DIR, "libperm.so")
-SOURCES = ["perm_kernels.cu", "perm_capi.cu", "perm_noalloc.cu", "perm_batch.cu"]
-HEADERS = ["perm_device.cuh", "perm_kernels.cuh"]
+SOURCES = ["perm_kernels.cu", "perm_grow_square.cu", "perm_grow_cubic.cu", "perm_grow_cubic_long.cu",
+            "perm_capi.cu", "perm_noalloc.cu", "perm_batch.cu"]
+HEADERS = ["perm_device.cuh", "perm_kernels.cuh", "perm_grow.cuh"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "--fmad=false", "-Xcompiler", "-fPIC",
          "-I", os.path.join(ROOT, "include"), "-I", CSRC]

@@ -49,6 +49,12 @@ struct perm_batch_s {
 
 namespace {
 
+bool all_plain(const std::vector<perm::RunDev> &P) {
+    for (const perm::RunDev &p : P)
+        if (!perm::plain_run(p)) return false;
+    return true;
+}
+
 void batch_free(perm_batch_handle b) {
     if (!b) return;
     if (b->origin) cudaStreamSynchronize(b->origin);
@@ -203,6 +209,7 @@ int perm_batch_create_persistent(perm_batch_handle *out, const perm_config *cfgs
     B.closed = b->d_ctl + 2 * R;
     B.runs_open = b->d_ctl + 3 * R;
     B.max_ns = (long long)(max_s * 1e9);
+    B.plain = all_plain(P);
     // capture: reset every run, the batch kernel, clamp each run's tour counter
     if (rc == PERM_OK && cudaStreamBeginCapture(b->origin, cudaStreamCaptureModeThreadLocal) != cudaSuccess)
         rc = PERM_EDEVICE;
@@ -283,6 +290,7 @@ int perm_batch_continue(perm_batch_handle b, const int64_t *extra_tours_per_seq)
         B.closed = b->d_ctl + 2 * b->R;
         B.runs_open = b->d_ctl + 3 * b->R;
         B.max_ns = b->max_ns;
+        B.plain = all_plain(P);
         if (perm::launch_batch(B, b->grid, b->threads, b->smem, b->origin) != cudaSuccess) return PERM_EDEVICE;
         for (int r = 0; r < b->R; ++r)
             if (perm::launch_finalize(P[r], b->origin) != cudaSuccess) return PERM_EDEVICE;

@@ -102,6 +102,14 @@ constexpr int kDefaultShareCap = 4;
 constexpr int kBoostShareCap = 1024;
 constexpr long long kStallNs = 700000;
 
+// A length's cut-offs as the kernel compares them, by their bit patterns: no NaN (which no
+// weight is above or below) and no -0.0.
+double2 clean_cutoffs(double hi, double lo) {
+    if (std::isnan(hi)) hi = INFINITY;
+    if (std::isnan(lo)) lo = 0.0;
+    return make_double2(hi == 0.0 ? 0.0 : hi, lo == 0.0 ? 0.0 : lo);
+}
+
 int scale_exp_host(int d, int n) { return d == 2 ? (11 * n) >> 3 : (9 * n) >> 2; }
 
 int max_n_for(int d, bool key64) {
@@ -461,7 +469,7 @@ int perm_set_cutoffs(perm_handle h, const double *T_hi, const double *t_lo, int 
         return PERM_EINVAL;
     const size_t L = (size_t)h->cfg.n_max + 1;
     std::vector<double2> host(L);
-    for (size_t k = 0; k < L; ++k) host[k] = make_double2(T_hi[k], t_lo[k]);
+    for (size_t k = 0; k < L; ++k) host[k] = clean_cutoffs(T_hi[k], t_lo[k]);
     if (!h->cut) {
         const int rc = dalloc(h, &h->cut, L);
         if (rc != PERM_OK) return rc;
@@ -946,7 +954,12 @@ int perm_load(perm_handle *out, const char *path) {
     if (e == cudaSuccess && hd.has_cut) {
         rc = dalloc(h, &h->cut, L);
         if (rc != PERM_OK) { perm_destroy(h); return rc; }
-        e = put(h->cut, L * sizeof(double2));
+        std::vector<double2> cut(L);
+        std::memcpy(cut.data(), p, L * sizeof(double2));
+        for (double2 &c : cut) c = clean_cutoffs(c.x, c.y);
+        p += L * sizeof(double2);
+        e = cudaMemcpyAsync(h->cut, cut.data(), L * sizeof(double2), cudaMemcpyHostToDevice, h->stream);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
         h->cut_copies = hd.cut_copies;
         h->cut_q = hd.cut_q;
     }

@@ -96,9 +96,13 @@ struct BatchDev {
     int *active;          // per run: CTAs on it now
     int *granted;         // per run: tour-growing walks handed to CTAs
     int *runs_open;       // runs with tours to start and walks to grant
+    bool plain;           // no run has cut-offs, observables or a trace
     int *closed;          // per run: bit 0 tickets exhausted, bit 1 walks all granted
     long long max_ns;     // wall-clock bound of the launch
 };
+
+// A run without cut-offs, observables or a trace, its walks in shared memory.
+bool plain_run(const RunDev &P);
 
 // Largest dynamic shared memory a batch CTA can have (and allow it).
 cudaError_t batch_smem_budget(size_t *dynamic_max);
@@ -128,6 +132,13 @@ size_t walk_bytes(bool key64, int n_max, int log2h, int stack_cache);
 int walks_per_warp_max(int d);
 constexpr int kMaxWalkWarps = 8;
 
+// One lattice and key width each (perm_grow_*.cu), and their shared memory limits.
+cudaError_t launch_square(const RunDev &P, int thresh_mode, int ctas, cudaStream_t stream);
+cudaError_t launch_cubic(const RunDev &P, int thresh_mode, int ctas, cudaStream_t stream);
+cudaError_t launch_cubic_long(const RunDev &P, int thresh_mode, int ctas, cudaStream_t stream);
+cudaError_t allow_square();
+cudaError_t allow_cubic();
+cudaError_t allow_cubic_long();
 cudaError_t launch_grow(const RunDev &P, int thresh_mode, bool key64, int ctas,
                         cudaStream_t stream);
 // After a launch: the ticket counter clamped to M, the admission count of the next one.

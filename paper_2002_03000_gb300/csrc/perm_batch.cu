@@ -45,6 +45,7 @@ struct perm_batch_s {
     size_t smem = 0;
     long long max_ns = 0;
     std::vector<perm::RunDev> P0;   // the descriptors a replay grows (from empty tables)
+    bool failed = false;            // a run of the last launch failed: it may have left tour sums behind
 };
 
 namespace {
@@ -237,6 +238,15 @@ int perm_batch_create_persistent(perm_batch_handle *out, const perm_config *cfgs
 
 int perm_batch_run(perm_batch_handle b) {
     if (!b || !b->exec) return PERM_EINVAL;
+    if (b->failed) {
+        for (perm_handle h : b->runs) {
+            const int rc = perm::member_clear_sums(h);
+            if (rc != PERM_OK) return rc;
+        }
+        for (cudaStream_t s : b->streams)
+            if (cudaStreamSynchronize(s) != cudaSuccess) return PERM_EDEVICE;
+        b->failed = false;
+    }
     // a replay grows every run from empty tables by its creation-time tours, also
     // after perm_batch_continue moved the descriptors and tour counts on
     if (b->persistent && cudaMemcpyAsync(b->d_runs, b->P0.data(), sizeof(perm::RunDev) * b->R,
@@ -252,8 +262,10 @@ int perm_batch_run(perm_batch_handle b) {
     for (perm_handle h : b->runs) {
         perm_stats_t st;
         const int rc = perm_stats(h, &st);
-        if (rc != PERM_OK) return rc;
-        if (st.status != PERM_OK) return st.status;
+        if (rc != PERM_OK || st.status != PERM_OK) {
+            b->failed = true;
+            return rc != PERM_OK ? rc : st.status;
+        }
     }
     return PERM_OK;
 }
@@ -299,8 +311,10 @@ int perm_batch_continue(perm_batch_handle b, const int64_t *extra_tours_per_seq)
     for (perm_handle h : b->runs) {
         perm_stats_t st;
         const int rc = perm_stats(h, &st);
-        if (rc != PERM_OK) return rc;
-        if (st.status != PERM_OK) return st.status;
+        if (rc != PERM_OK || st.status != PERM_OK) {
+            b->failed = true;
+            return rc != PERM_OK ? rc : st.status;
+        }
     }
     return PERM_OK;
 }

@@ -34,7 +34,11 @@ struct perm_run_s {
     int ntab = 1;
     int xrows = 0;                 // tour-sum rows: one per walk, two with shared copies
     int tour_slots = 0;            // walks that start tours; the other slots are helpers
-    // device buffers
+    // what a reset zeroes, in one buffer: the counters (a 256-byte line each: the kernels' walks
+    // meet on several of them), the tables and the rings' stamps
+    unsigned char *block = nullptr;
+    size_t zero_bytes = 0;
+    // device buffers (those of the block point into it)
     double *Wn = nullptr, *Qn = nullptr, *X = nullptr, *gstk_w = nullptr, *Rn = nullptr;
     unsigned long long *Sn = nullptr, *tickets = nullptr, *seq_M = nullptr;
     unsigned long long *steps = nullptr, *max_stack = nullptr, *copies = nullptr, *refreshes = nullptr, *trace_count = nullptr;
@@ -49,7 +53,7 @@ struct perm_run_s {
     unsigned char *dq_cells = nullptr;
     unsigned long long *dq_head = nullptr, *dq_tail = nullptr;
     unsigned int *dq_ready = nullptr, *dq_free = nullptr, *outst = nullptr, *tmaxn = nullptr;
-    int *hungry = nullptr;         // [0] walks waiting for work, [1] cells waiting for a walk, [2] cells in use
+    int *hungry = nullptr, *queued = nullptr, *dq_used = nullptr;
     double2 *cut = nullptr;        // original PERM's cut-offs (nullptr: flatPERM)
     int cut_copies = 1;
     double cut_q = 1.0;
@@ -65,6 +69,12 @@ struct perm_run_s {
 };
 
 namespace {
+
+// The counters of a handle's block, a line each.
+constexpr size_t kLine = 256;
+constexpr size_t kOneCopy = 1 << 20;   // tables up to this size come back in one copy
+enum Counter { kTickets, kSteps, kMaxStack, kCopies, kRefreshes, kIterations, kFinished, kExact, kStatus, kAdmit, kHead, kTail,
+               kHungry, kQueued, kUsed, kCounters };
 
 int to_code(cudaError_t e) {
     if (e == cudaSuccess) return PERM_OK;
@@ -84,11 +94,8 @@ int dalloc(perm_handle h, T **p, size_t count) {
 }
 
 void free_all(perm_handle h) {
-    void *ptrs[] = {h->Wn, h->Qn, h->Rn, h->X, h->gstk_w, h->Sn, h->tickets, h->seq_M, h->steps,
-                    h->max_stack, h->copies, h->refreshes, h->iterations, h->finished, h->exact_steps, h->admit,
-                    h->trace_count, h->gstk_meta, h->status, h->trace,
-                    h->trace_coords, h->dq_cells, h->dq_head, h->dq_tail, h->dq_ready, h->dq_free, h->outst,
-                    h->tmaxn, h->hungry, h->cut, h->arena};
+    void *ptrs[] = {h->block, h->X, h->gstk_w, h->gstk_meta, h->trace_count, h->trace, h->trace_coords, h->dq_cells,
+                    h->outst, h->cut, h->arena};
     for (void *p : ptrs) if (p) cudaFree(p);
 }
 
@@ -336,49 +343,72 @@ int create_impl(perm_handle *out, const perm_config *cfg, const ForcedLayout *fo
     const size_t L = (size_t)n_max + 1;
     h->ntab = (cfg->alg == PERM_ALG1) ? n_seq : 1;
     int rc = PERM_OK;
-    if (rc == PERM_OK) rc = dalloc(h, &h->Wn, L * h->ntab);
-    if (rc == PERM_OK) rc = dalloc(h, &h->Qn, L * h->ntab);
-    if (rc == PERM_OK) rc = dalloc(h, &h->Sn, L * h->ntab);
-    if (rc == PERM_OK && cfg->observables) rc = dalloc(h, &h->Rn, L * h->ntab);
-    if (rc == PERM_OK) rc = dalloc(h, &h->tickets, 1);
-    if (rc == PERM_OK) rc = dalloc(h, &h->seq_M, (size_t)n_seq);
     h->share = cfg->share_copies >= 0 && cfg->alg == PERM_ALG2 && h->thresh == perm::kSnapshot;
     h->xrows = h->slots * (h->share ? 2 : 1);
+    // shared copies: a ring of cells, each one waiting copy record plus the keys of the
+    // walk up to its branch point (header, the keys of sites 0..n_max, their hash slots)
+    h->share_cap = cfg->share_copies > 0 ? cfg->share_copies : kDefaultShareCap;
+    size_t cells = 0;
+    if (h->share) {
+        int lc = 6;
+        while ((1 << lc) < h->slots && lc < 12) ++lc;
+        h->dq_log2cap = lc;
+        h->dq_cell_bytes = (int)(32 + ((((size_t)n_max + 1) * (key64 ? 8 : 4) + 15) & ~(size_t)15) +
+                                 ((((size_t)n_max + 1) * 2 + 15) & ~(size_t)15));
+        cells = (size_t)1 << lc;
+    }
+    // the block a reset zeroes
+    const size_t cnt = L * (size_t)h->ntab;
+    size_t off = 0;
+    auto place = [&](size_t bytes) {
+        const size_t at = off;
+        off += (bytes + kLine - 1) / kLine * kLine;
+        return at;
+    };
+    const size_t o_counters = place(kCounters * kLine), o_W = place(cnt * 8), o_Q = place(cnt * 8), o_S = place(cnt * 8);
+    const size_t o_R = cfg->observables ? place(cnt * 8) : 0, o_M = place((size_t)n_seq * 8);
+    const size_t o_ready = place(cells * 4), o_free = place(cells * 4), o_tmax = place(h->share ? (size_t)h->xrows * 4 : 0);
+    h->zero_bytes = off;
+    rc = dalloc(h, &h->block, off);
+    if (rc == PERM_OK) {
+        unsigned char *B = h->block;
+        auto counter = [&](int i) { return reinterpret_cast<unsigned long long *>(B + o_counters + (size_t)i * kLine); };
+        h->Wn = reinterpret_cast<double *>(B + o_W);
+        h->Qn = reinterpret_cast<double *>(B + o_Q);
+        h->Sn = reinterpret_cast<unsigned long long *>(B + o_S);
+        if (cfg->observables) h->Rn = reinterpret_cast<double *>(B + o_R);
+        h->seq_M = reinterpret_cast<unsigned long long *>(B + o_M);
+        h->tickets = counter(kTickets);
+        h->steps = counter(kSteps);
+        h->max_stack = counter(kMaxStack);
+        h->copies = counter(kCopies);
+        h->refreshes = counter(kRefreshes);
+        h->iterations = counter(kIterations);
+        h->finished = counter(kFinished);
+        h->exact_steps = counter(kExact);
+        h->status = reinterpret_cast<int *>(counter(kStatus));
+        h->admit = reinterpret_cast<long long *>(counter(kAdmit));
+        if (h->share) {
+            h->dq_head = counter(kHead);
+            h->dq_tail = counter(kTail);
+            h->hungry = reinterpret_cast<int *>(counter(kHungry));
+            h->queued = reinterpret_cast<int *>(counter(kQueued));
+            h->dq_used = reinterpret_cast<int *>(counter(kUsed));
+            h->dq_ready = reinterpret_cast<unsigned int *>(B + o_ready);
+            h->dq_free = reinterpret_cast<unsigned int *>(B + o_free);
+            h->tmaxn = reinterpret_cast<unsigned int *>(B + o_tmax);
+        }
+    }
     if (rc == PERM_OK) rc = dalloc(h, &h->X, L * (size_t)h->xrows);
     if (rc == PERM_OK) rc = dalloc(h, &h->gstk_meta, (size_t)n_max * h->slots);
     if (rc == PERM_OK) rc = dalloc(h, &h->gstk_w, (size_t)n_max * h->slots);
     if (rc == PERM_OK && h->arena_mode != perm::kArenaNone)
         rc = dalloc(h, &h->arena, (size_t)h->arena_cta_bytes * (size_t)h->ctas);
-    if (rc == PERM_OK) rc = dalloc(h, &h->steps, 1);
-    if (rc == PERM_OK) rc = dalloc(h, &h->max_stack, 1);
-    if (rc == PERM_OK) rc = dalloc(h, &h->copies, 1);
-    if (rc == PERM_OK) rc = dalloc(h, &h->refreshes, 1);
-    if (rc == PERM_OK) rc = dalloc(h, &h->iterations, 1);
-    if (rc == PERM_OK) rc = dalloc(h, &h->finished, 1);
-    if (rc == PERM_OK) rc = dalloc(h, &h->exact_steps, 1);
-    if (rc == PERM_OK) rc = dalloc(h, &h->admit, 2);
     if (rc == PERM_OK) rc = dalloc(h, &h->trace_count, 1);
-    if (rc == PERM_OK) rc = dalloc(h, &h->status, 1);
-    // shared copies: a ring of cells, each one waiting copy record plus the keys of the
-    // walk up to its branch point
-    h->share_cap = cfg->share_copies > 0 ? cfg->share_copies : kDefaultShareCap;
     if (rc == PERM_OK && h->share) {
-        int lc = 6;
-        while ((1 << lc) < h->slots && lc < 12) ++lc;
-        h->dq_log2cap = lc;
-        // header, the keys of sites 0..n_max, their hash slots (u16)
-        h->dq_cell_bytes = (int)(32 + ((((size_t)n_max + 1) * (key64 ? 8 : 4) + 15) & ~(size_t)15) +
-                                 ((((size_t)n_max + 1) * 2 + 15) & ~(size_t)15));
-        const size_t cap = (size_t)1 << lc;
-        rc = dalloc(h, &h->dq_cells, cap * (size_t)h->dq_cell_bytes);
-        if (rc == PERM_OK) rc = dalloc(h, &h->dq_ready, cap);
-        if (rc == PERM_OK) rc = dalloc(h, &h->dq_free, cap);
-        if (rc == PERM_OK) rc = dalloc(h, &h->dq_head, 1);
-        if (rc == PERM_OK) rc = dalloc(h, &h->dq_tail, 1);
+        rc = dalloc(h, &h->dq_cells, cells * (size_t)h->dq_cell_bytes);
         if (rc == PERM_OK) rc = dalloc(h, &h->outst, (size_t)h->xrows);
         if (rc == PERM_OK) rc = to_code(cudaMemsetAsync(h->outst, 0xFF, sizeof(unsigned int) * h->xrows, h->stream));
-        if (rc == PERM_OK) rc = dalloc(h, &h->tmaxn, (size_t)h->xrows);
-        if (rc == PERM_OK) rc = dalloc(h, &h->hungry, 3);
     }
     if (rc == PERM_OK) rc = to_code(cudaStreamSynchronize(h->stream));
     if (rc != PERM_OK) {
@@ -439,7 +469,7 @@ static RunDev make_params(perm_handle h) {
     P.stall_ns = kStallNs;
     P.dq_log2cap = h->dq_log2cap; P.dq_cell_bytes = h->dq_cell_bytes; P.dq_cells = h->dq_cells;
     P.dq_head = h->dq_head; P.dq_tail = h->dq_tail; P.dq_ready = h->dq_ready; P.dq_free = h->dq_free;
-    P.outst = h->outst; P.tmaxn = h->tmaxn; P.hungry = h->hungry; P.queued = h->hungry ? h->hungry + 1 : nullptr; P.dq_used = h->hungry ? h->hungry + 2 : nullptr;
+    P.outst = h->outst; P.tmaxn = h->tmaxn; P.hungry = h->hungry; P.queued = h->queued; P.dq_used = h->dq_used;
     P.status = h->status;
     P.cut = h->cut;
     P.cut_copies = h->cut_copies;
@@ -512,11 +542,11 @@ static cudaError_t copy_out(perm_handle h, void *dst, const void *src, size_t by
     return e;
 }
 
+// Wait for the stream; the run's status (one copy: it orders after the run and reports
+// its failure).
 static int sync_status(perm_handle h) {
-    cudaError_t e = cudaStreamSynchronize(h->stream);
-    if (e != cudaSuccess) return to_code(e);
     int st = 0;
-    e = copy_out(h, &st, h->status, sizeof(int));
+    const cudaError_t e = copy_out(h, &st, h->status, sizeof(int));
     if (e != cudaSuccess) return to_code(e);
     h->last_status = st;
     return st;
@@ -530,16 +560,36 @@ int perm_run_sync(perm_handle h, int64_t tours_per_seq) {
 
 int perm_tables(perm_handle h, double *W_n, double *S_n, double *Q_n, int64_t *M) {
     if (!h) return PERM_EINVAL;
-    int st = sync_status(h);
-    if (st < 0 && st != PERM_EOVERFLOW && st != PERM_ETIMEOUT) return st;
     const size_t L = (size_t)h->cfg.n_max + 1, cnt = L * h->ntab;
+    const unsigned char *from = h->block;
+    const size_t o_W = (size_t)(reinterpret_cast<unsigned char *>(h->Wn) - from), o_Q = (size_t)(reinterpret_cast<unsigned char *>(h->Qn) - from),
+                 o_S = (size_t)(reinterpret_cast<unsigned char *>(h->Sn) - from), upto = o_S + cnt * 8;
     cudaError_t e = cudaSuccess;
-    if (W_n) e = copy_out(h, W_n, h->Wn, cnt * sizeof(double));
-    if (e == cudaSuccess && Q_n) e = copy_out(h, Q_n, h->Qn, cnt * sizeof(double));
-    if (e == cudaSuccess && S_n) {
-        std::vector<unsigned long long> s(cnt);
-        e = copy_out(h, s.data(), h->Sn, cnt * sizeof(unsigned long long));
-        for (size_t i = 0; i < cnt; ++i) S_n[i] = (double)s[i];
+    int st;
+    if (upto <= kOneCopy) {
+        // the counters and the tables in one copy (each costs about 10 us of host time)
+        std::vector<unsigned char> buf(upto);
+        e = copy_out(h, buf.data(), from, upto);
+        if (e != cudaSuccess) return to_code(e);
+        std::memcpy(&st, buf.data() + kStatus * kLine, sizeof(int));
+        h->last_status = st;
+        if (st < 0 && st != PERM_EOVERFLOW && st != PERM_ETIMEOUT) return st;
+        if (W_n) std::memcpy(W_n, buf.data() + o_W, cnt * 8);
+        if (Q_n) std::memcpy(Q_n, buf.data() + o_Q, cnt * 8);
+        if (S_n) {
+            const unsigned long long *s = reinterpret_cast<const unsigned long long *>(buf.data() + o_S);
+            for (size_t i = 0; i < cnt; ++i) S_n[i] = (double)s[i];
+        }
+    } else {
+        st = sync_status(h);
+        if (st < 0 && st != PERM_EOVERFLOW && st != PERM_ETIMEOUT) return st;
+        if (W_n) e = copy_out(h, W_n, h->Wn, cnt * sizeof(double));
+        if (e == cudaSuccess && Q_n) e = copy_out(h, Q_n, h->Qn, cnt * sizeof(double));
+        if (e == cudaSuccess && S_n) {
+            std::vector<unsigned long long> s(cnt);
+            e = copy_out(h, s.data(), h->Sn, cnt * sizeof(unsigned long long));
+            for (size_t i = 0; i < cnt; ++i) S_n[i] = (double)s[i];
+        }
     }
     if (e == cudaSuccess && M) {
         if (h->cfg.alg == PERM_ALG2) {
@@ -556,34 +606,12 @@ int perm_tables(perm_handle h, double *W_n, double *S_n, double *Q_n, int64_t *M
 
 int perm_reset(perm_handle h) {
     if (!h) return PERM_EINVAL;
-    const size_t L = (size_t)h->cfg.n_max + 1, cnt = L * h->ntab;
-    cudaError_t e = cudaMemsetAsync(h->Wn, 0, cnt * sizeof(double), h->stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(h->Qn, 0, cnt * sizeof(double), h->stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(h->Sn, 0, cnt * sizeof(unsigned long long), h->stream);
-    if (e == cudaSuccess && h->Rn) e = cudaMemsetAsync(h->Rn, 0, cnt * sizeof(double), h->stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(h->tickets, 0, sizeof(unsigned long long), h->stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(h->seq_M, 0, sizeof(unsigned long long) * h->cfg.n_seq, h->stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(h->steps, 0, sizeof(unsigned long long), h->stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(h->copies, 0, sizeof(unsigned long long), h->stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(h->refreshes, 0, sizeof(unsigned long long), h->stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(h->iterations, 0, sizeof(unsigned long long), h->stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(h->finished, 0, sizeof(unsigned long long), h->stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(h->admit, 0, 2 * sizeof(long long), h->stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(h->exact_steps, 0, sizeof(unsigned long long), h->stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(h->max_stack, 0, sizeof(unsigned long long), h->stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(h->status, 0, sizeof(int), h->stream);
+    const size_t L = (size_t)h->cfg.n_max + 1;
+    cudaError_t e = cudaMemsetAsync(h->block, 0, h->zero_bytes, h->stream);
     if (e == cudaSuccess && h->last_status != PERM_OK)   // a stopped run may leave tour sums behind
         e = cudaMemsetAsync(h->X, 0, L * (size_t)h->xrows * sizeof(double), h->stream);
-    if (e == cudaSuccess && h->share) {
-        const size_t cap = (size_t)1 << h->dq_log2cap;
-        e = cudaMemsetAsync(h->dq_head, 0, sizeof(unsigned long long), h->stream);
-        if (e == cudaSuccess) e = cudaMemsetAsync(h->dq_tail, 0, sizeof(unsigned long long), h->stream);
-        if (e == cudaSuccess) e = cudaMemsetAsync(h->dq_ready, 0, sizeof(unsigned int) * cap, h->stream);
-        if (e == cudaSuccess) e = cudaMemsetAsync(h->dq_free, 0, sizeof(unsigned int) * cap, h->stream);
-        if (e == cudaSuccess) e = cudaMemsetAsync(h->hungry, 0, 3 * sizeof(int), h->stream);
-        if (e == cudaSuccess) e = cudaMemsetAsync(h->outst, 0xFF, sizeof(unsigned int) * h->xrows, h->stream);
-        if (e == cudaSuccess) e = cudaMemsetAsync(h->tmaxn, 0, sizeof(unsigned int) * h->xrows, h->stream);
-    }
+    if (e == cudaSuccess && h->share)
+        e = cudaMemsetAsync(h->outst, 0xFF, sizeof(unsigned int) * h->xrows, h->stream);
     if (e != cudaSuccess) return to_code(e);
     h->tour_limit = 0;
     h->seq_target = 0;
@@ -687,17 +715,20 @@ int perm_observable_r2(perm_handle h, double *mean_r2, double *R_n) {
 
 int perm_stats(perm_handle h, perm_stats_t *out) {
     if (!h || !out) return PERM_EINVAL;
-    int st = sync_status(h);
+    unsigned char buf[kCounters * kLine];
+    const cudaError_t e = copy_out(h, buf, h->block, sizeof(buf));
+    if (e != cudaSuccess) return to_code(e);
+    int st = 0;
+    std::memcpy(&st, buf + kStatus * kLine, sizeof(int));
+    h->last_status = st;
     if (st < 0 && st != PERM_EOVERFLOW && st != PERM_ETIMEOUT) return st;
-    unsigned long long steps = 0, ms = 0, cp = 0, rf = 0, it = 0, fin = 0, shr = 0, ex = 0;
-    if (copy_out(h, &steps, h->steps, 8) != cudaSuccess) return PERM_EDEVICE;
-    if (copy_out(h, &cp, h->copies, 8) != cudaSuccess) return PERM_EDEVICE;
-    if (copy_out(h, &rf, h->refreshes, 8) != cudaSuccess) return PERM_EDEVICE;
-    if (copy_out(h, &it, h->iterations, 8) != cudaSuccess) return PERM_EDEVICE;
-    if (copy_out(h, &ms, h->max_stack, 8) != cudaSuccess) return PERM_EDEVICE;
-    if (copy_out(h, &fin, h->finished, 8) != cudaSuccess) return PERM_EDEVICE;
-    if (copy_out(h, &ex, h->exact_steps, 8) != cudaSuccess) return PERM_EDEVICE;
-    if (h->share && copy_out(h, &shr, h->dq_tail, 8) != cudaSuccess) return PERM_EDEVICE;
+    auto value = [&](int i) {
+        unsigned long long v;
+        std::memcpy(&v, buf + (size_t)i * kLine, 8);
+        return v;
+    };
+    const unsigned long long steps = value(kSteps), ms = value(kMaxStack), cp = value(kCopies), rf = value(kRefreshes),
+                             it = value(kIterations), fin = value(kFinished), ex = value(kExact), shr = value(kTail);
     out->steps = (int64_t)steps;
     out->tours = h->cfg.alg == PERM_ALG2 ? h->tour_limit : h->seq_target * h->cfg.n_seq;
     out->max_stack = (int64_t)ms;
@@ -815,9 +846,9 @@ int member_extend(perm_handle h, int64_t extra_tours_per_seq, int run_index, Run
     return PERM_OK;
 }
 
-int member_reset(perm_handle h) {
-    int rc = perm_reset(h);
-    if (rc != PERM_OK) return rc;
+int member_reset(perm_handle h) { return perm_reset(h); }
+
+int member_clear_sums(perm_handle h) {
     const size_t L = (size_t)h->cfg.n_max + 1;
     return to_code(cudaMemsetAsync(h->X, 0, L * (size_t)h->xrows * sizeof(double), h->stream));
 }

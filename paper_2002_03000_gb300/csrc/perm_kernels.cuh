@@ -118,8 +118,10 @@ cudaError_t launch_batch(const BatchDev &B, int ctas, int threads, size_t smem, 
 int member_create(perm_handle *out, const perm_config *cfg, int ctas, size_t smem_budget);
 int member_params(perm_handle h, int64_t tours_per_seq, int run_index, RunDev *P, size_t *smem,
                   int *worker_warps);
-// Empty tables and tour sums (every row, also after a failed run), on the run's stream.
+// Empty tables, on the run's stream; and the tour sums (which a completed run leaves at
+// zero, so that only a failed one needs it).
 int member_reset(perm_handle h);
+int member_clear_sums(perm_handle h);
 // The descriptor after extra_tours_per_seq more tours per sequence on top of the
 // run's current tables (cumulative, as perm_run).
 int member_extend(perm_handle h, int64_t extra_tours_per_seq, int run_index, RunDev *P);

@@ -262,20 +262,30 @@ __device__ __forceinline__ double widen(float f) {
 // x enters capped at 16, past every a_+ + 1.  Selects, no branches: a warp's walks
 // take different sides, and a branch costs a lone warp 25 cycles or more.  (The same
 // decision by ceilings and thresholds on w0 took 144 cycles of a lone warp, this
-// one 60.)
-// Returns c (0: pruned); `surv` marks a survivor of pruning.
+// one 60.)  Everything but the cap a_+ is formed before the probes have settled a_+.
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ int decide_estimate(float x, int a, uint32_t w0, bool &surv, bool &amb) {
+struct Guess {
+    float x;             // the estimate of r
+    int c;               // floor of the sum, not yet capped at a_+ (r < 1: 1 survives, 0 is pruned)
+    int k;               // the integer next to the sum
+    bool up, near_k;     // r >= 1; the sum lies within the margin of k
+    bool open;           // no branch of r settled, or no estimate
+};
+__device__ __forceinline__ Guess guess(double W, double Wsum, float Mf, uint32_t w0) {
+    Guess g;
+    bool odd = false;
     const float uf = __fmul_rn(__uint2float_rn(w0), 0x1p-32f), vf = __fmul_rn(__uint2float_rn(~w0), 0x1p-32f);
-    const float xc = fminf(x, 16.0f), lim = (float)a;
-    const bool up = xc >= 1.0f;
-    const float y = __fadd_rn(xc, up ? uf : vf);
-    const float k = __fsub_rn(__fadd_rn(y, 12582912.0f), 12582912.0f);        // y to the nearest integer
+    g.x = ratio_estimate(W, Wsum, Mf, odd);
+    const float xc = fminf(g.x, 16.0f);
+    g.up = xc >= 1.0f;
+    const float y = __fadd_rn(xc, g.up ? uf : vf);
+    const float kf = __fsub_rn(__fadd_rn(y, 12582912.0f), 12582912.0f);       // y to the nearest integer
     const float tol = __fmaf_rn(xc, 0x1p-20f, 0x1p-23f);
-    amb = fabsf(__fsub_rn(xc, 1.0f)) < 0x1p-19f || (fabsf(__fsub_rn(y, k)) <= tol && k <= lim);
-    const int c = (int)fminf(k > y ? __fsub_rn(k, 1.0f) : k, lim);
-    surv = !up && c > 0;
-    return c;
+    g.k = (int)kf;
+    g.c = kf > y ? g.k - 1 : g.k;
+    g.near_k = fabsf(__fsub_rn(y, kf)) <= tol;
+    g.open = odd || fabsf(__fsub_rn(xc, 1.0f)) < 0x1p-19f;
+    return g;
 }
 
 // The same decision on the double-precision r, with the comparisons taken on

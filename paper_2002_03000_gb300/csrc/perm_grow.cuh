@@ -207,27 +207,25 @@ __device__ __noinline__ Decision decide_node_exact(int a, double W, double sum, 
 }
 
 // The decision at a node with a >= 1 free neighbours (Sec. 2): r, the copies, the
-// children's weight.  Wsum: sum of the weights recorded at length n before this
-// node, sum: Wsum + W; refine: round the survivor's quotient by M correctly (one more step of the
+// children's weight.  sum: the weights recorded at length n up to this node, gs: what
+// the estimate of r says; refine: round the survivor's quotient by M correctly (one more step of the
 // division).  valid: the lane has a node to decide (the others' results are not used);
 // force_exact: decide on the double-precision r.  Shared by the persistent kernel
 // and the snapshot-state kernel; every lane of a walk's group takes the same decision.
 // One straight line with selects but for the exact path: a branch costs a lone warp
 // 25 cycles or more, a double-precision instruction 64 whatever its active lanes.
 template <int D>
-__device__ __forceinline__ Decision decide_node(int n, int a, double W, double Wsum, double sum, const Tours &t,
+__device__ __forceinline__ Decision decide_node(int n, int a, double W, double sum, const Guess &gs, const Tours &t,
                                                 bool refine, uint32_t w0, const double *aoc, bool valid, bool force_exact) {
     Decision o;
     o.exact = false;
-    bool odd = false, amb = false, surv = false;
-    const float x = ratio_estimate(W, Wsum, t.Mf, odd);
-    o.x = x;
+    o.x = gs.x;
     o.r = 0.0;
     const int dE = scale_row<D>(n) + (D == 2 ? 1 : 2);
     const double *row = aoc + 48 * (dE - (D == 2 ? 1 : 2)) + 8 * (a - 1);
-    int c = decide_estimate(x, a, w0, surv, amb);
-    if (n == 0) { c = 1; surv = false; }                 // r = 1 at the empty walk
-    const bool exact = valid && n != 0 && (amb || odd || force_exact);
+    const bool surv = !gs.up && gs.c > 0 && n != 0;
+    const int c = n == 0 ? 1 : (gs.c < a ? gs.c : a);    // r = 1 at the empty walk
+    const bool exact = valid && n != 0 && (gs.open || (gs.near_k && gs.k <= a) || force_exact);
     // a survivor carries W/r = [W_n]^sample = (Wsum + W)/M, a child of an enrichment
     // (W/c) a_+ 2^-dE: one double-precision product for both, on the critical path
     // alone.  The survivor's factor (1/M) a_+ 2^-dE (a node past the empty walk has
@@ -259,7 +257,7 @@ __device__ __forceinline__ Decision decide_node(int n, int a, double W, double W
         const double q = __dmul_rn(sum, t.inv1);
         double avg = __fma_rn(__fma_rn(-q, t.Md, sum), t.inv1, q);
         const int es = __double2hiint(sum) >> 20;
-        if (odd || es < 128 || es > 1920) avg = __ddiv_rn(sum, t.Md);
+        if (t.Mf < 0.0f || es < 128 || es > 1920) avg = __ddiv_rn(sum, t.Md);
         o = decide_on_average(a, W, avg, w0, row[0]);
     } else if (exact) {
         o = decide_node_exact(a, W, sum, t.M, w0, row[0]);
@@ -1145,9 +1143,12 @@ __device__ __forceinline__ void grow_run(const RunDev &P, unsigned char *smem, c
             const int fm = (int)((__ballot_sync(kFull, free_j) >> lead) & ((1u << G) - 1u));
             const int a = __popc(fm), a1 = a > 0 ? a : 1;
             const bool decides = grows_on && a > 0;
-            // the node's random words, from the lane that holds its block
+            // the node's random words, from the lane that holds its block, and what the estimate
+            // of r says
             const int wl = lead + (int)((ord - pbase) & (uint32_t)(G - 1));
             const uint32_t w0 = __shfl_sync(kFull, pw0, wl), w1 = __shfl_sync(kFull, pw1, wl);
+            Guess gs;
+            if (!cutoffs) gs = guess(W, Wsum, tours.Mf, w0);
             // the first child's step (a draw from the free list), its key and its place in the
             // hash, from the lane that probed it
             const uint32_t list = lists[fm];
@@ -1157,7 +1158,7 @@ __device__ __forceinline__ void grow_run(const RunDev &P, unsigned char *smem, c
             const int cslot = __shfl_sync(kFull, nslot, lead + dir0);
             Decision o;
             if (cutoffs) o = decide_cutoffs<D>(n, a1, W, cut_n, w0, aoc, cuts);
-            else o = decide_node<D>(n, a1, W, Wsum, sum, tours, !snapshot, w0, aoc, decides, false);
+            else o = decide_node<D>(n, a1, W, sum, gs, tours, !snapshot, w0, aoc, decides, false);
             const int c = decides ? o.c : 0;
             if (o.exact && decides) my_exact += 1ull;
             const bool extend = c > 0, leaf = isn && c == 0;

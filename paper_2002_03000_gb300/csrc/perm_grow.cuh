@@ -25,7 +25,9 @@
 //
 // Threshold sources for Algorithm 2 (one shared table W, Fig. 1):
 //  - snapshot: every node adds its weight to the global table with a
-//    reduction that returns nothing; one extra warp per CTA reloads a
+//    reduction that returns nothing (S_n, the nodes of length n, is kept as its
+//    differences along n: +1 where a walk started or resumed, -1 past its leaf,
+//    one reduction a leaf); one extra warp per CTA reloads a
 //    shared-memory copy of W_n and M every refresh period.  The nodes read
 //    that copy (a stale but fixed threshold keeps the estimator unbiased:
 //    enrichment and pruning conserve the expected weight for any r).  Walks
@@ -51,7 +53,7 @@ namespace perm {
 
 namespace {
 
-constexpr int kUnwindSites = 16;   // hash deletions per walk per iteration
+constexpr int kUnwind = 4;         // hash deletions per lane per iteration (16 or 32 per walk)
 constexpr int kPoolExtra = 2;      // extra tour tickets fetched per warp (snapshot): M counts them as started
 constexpr int kChunk = 8;          // stack records moved per spill or fill (ring >= 2 kChunk)
 constexpr int kReloadBatch = 8;    // snapshot entries a refresher lane loads before storing them
@@ -292,9 +294,9 @@ __device__ __forceinline__ void red_add(double *p, double v, bool take) {
     asm volatile("{\n.reg .pred q;\nsetp.ne.s32 q, %2, 0;\n@q red.relaxed.gpu.global.add.f64 [%0], %1;\n}"
                  :: "l"(p), "d"(v), "r"((int)take) : "memory");
 }
-__device__ __forceinline__ void red_inc(unsigned long long *p, bool take) {
+__device__ __forceinline__ void red_count(unsigned long long *p, long long v, bool take) {
     asm volatile("{\n.reg .pred q;\nsetp.ne.s32 q, %2, 0;\n@q red.relaxed.gpu.global.add.u64 [%0], %1;\n}"
-                 :: "l"(p), "l"(1ull), "r"((int)take) : "memory");
+                 :: "l"(p), "l"(v), "r"((int)take) : "memory");
 }
 
 // The whole warp copies a donor's sites 0..bdp (key and hash slot) into a cell.
@@ -555,6 +557,7 @@ __device__ __forceinline__ void grow_run(const RunDev &P, unsigned char *smem, c
     // the walk's state: the same in every lane of its group
     int state = active ? kNeed : kDone;
     int n = 0, maxn = 0;
+    int seg = 0;               // length at which the walk started or last resumed
     Key cur = origin;          // key of the end-point
     double W = 1.0;
     uint32_t ord = 0u;         // nodes of this part so far; a node's 64-bit ordinal is did 2^32 + ord
@@ -628,6 +631,7 @@ __device__ __forceinline__ void grow_run(const RunDev &P, unsigned char *smem, c
             sites[0] = (uint16_t)s0;
         }
         state = kNode;
+        seg = 0;
     };
     const long long t_start = global_ns();
     for (uint32_t iter = 0u;; ++iter) {
@@ -1108,7 +1112,6 @@ __device__ __forceinline__ void grow_run(const RunDev &P, unsigned char *smem, c
                 if (isn && Mt != tours.M) set_tours<!cutoffs>(tours, Mt);
             }
             red_add(acc + n, W, isn && (snapshot ? j < 2 : j == 1));
-            red_inc(Srow + n, isn && j == 2);
             const double sum = __dadd_rn(Wsum, W);
             if (!snapshot && own_rows && isn && first) Wrow[n] = sum;
             // a full bucket without the key, a used-up block of random words, a new M: one vote
@@ -1270,6 +1273,10 @@ __device__ __forceinline__ void grow_run(const RunDev &P, unsigned char *smem, c
                     maxn = n_leaf > maxn ? n_leaf : maxn;
                     un_hi = n_leaf < P.n_max - 1 ? n_leaf : P.n_max - 1;
                     state = pops ? kUnwindState : kFlush;
+                    // one node of each length since the walk started or resumed (Srow:
+                    // differences along n)
+                    red_count(Srow + (j == 2 ? seg : n_leaf + 1), j == 2 ? 1 : -1,
+                              j == 2 || (j == 3 && n_leaf < P.n_max));
                 }
                 if (pops) {
                     pend_dir = (int)(rest & 7u);
@@ -1283,7 +1290,6 @@ __device__ __forceinline__ void grow_run(const RunDev &P, unsigned char *smem, c
                     smeta[ti] = (meta & 0xFFFFu) | ((uint32_t)(cnt - 1) << 16) | ((rest >> 3) << 19);
                 const bool back = state == kUnwindState;
                 const Key rkey = hash[sites[back ? pend_depth : 0]] + step_key<D, Key>(pend_dir);
-                constexpr int kUnwind = kUnwindSites / G;
                 int sl[kUnwind];
 #pragma unroll
                 for (int i = 0; i < kUnwind; ++i) {
@@ -1293,7 +1299,7 @@ __device__ __forceinline__ void grow_run(const RunDev &P, unsigned char *smem, c
 #pragma unroll
                 for (int i = 0; i < kUnwind; ++i)
                     if (sl[i] >= 0) hash[sl[i]] = (Key)0;
-                un_hi -= back ? kUnwindSites : 0;
+                un_hi -= back ? kUnwind * G : 0;
                 __syncwarp(gmask);
                 // the new end-point's place (every lane of the group looks at the same buckets):
                 // the first bucket of its sequence that is not full
@@ -1315,6 +1321,7 @@ __device__ __forceinline__ void grow_run(const RunDev &P, unsigned char *smem, c
                     cur = rkey;
                     W = pend_w;
                     state = places && full ? kDone : kNode;
+                    seg = n;
                 }
                 if (places && first && !full) {
                     const uint32_t rs = rb * (uint32_t)Buckets<Key>::kKeys + (uint32_t)place;
@@ -1329,6 +1336,7 @@ __device__ __forceinline__ void grow_run(const RunDev &P, unsigned char *smem, c
     // statistics (a walk cut short by an error counts its part so far), then tell the
     // refresher this warp is done
     if (state == kNode || state == kUnwindState) my_steps += ord;
+    red_count(Srow + (j == 2 ? seg : n), j == 2 ? 1 : -1, state == kNode && n > seg && (j == 2 || j == 3));
     unsigned long long tot = first ? my_steps : 0ull, cps = first ? my_copies : 0ull, exn = first ? my_exact : 0ull;
     int ms = my_max_stack;
 #pragma unroll

@@ -234,6 +234,25 @@ __global__ void finalize_kernel(unsigned long long *tickets, long long limit, lo
     }
 }
 
+// An inclusive sum of L entries in place, by one block: each thread a run of entries.
+__global__ void __launch_bounds__(1024) counts_kernel(unsigned long long *S, int L) {
+    __shared__ unsigned long long part[1024];
+    const int per = (L + (int)blockDim.x - 1) / (int)blockDim.x;
+    const int lo = min(L, (int)threadIdx.x * per), hi = min(L, lo + per);
+    unsigned long long sum = 0ull;
+    for (int i = lo; i < hi; ++i) sum += S[i];
+    part[threadIdx.x] = sum;
+    __syncthreads();
+    for (int off = 1; off < (int)blockDim.x; off <<= 1) {
+        const unsigned long long v = (int)threadIdx.x >= off ? part[threadIdx.x - off] : 0ull;
+        __syncthreads();
+        part[threadIdx.x] += v;
+        __syncthreads();
+    }
+    unsigned long long run = part[threadIdx.x] - sum;
+    for (int i = lo; i < hi; ++i) { run += S[i]; S[i] = run; }
+}
+
 }  // namespace
 
 bool plain_run(const RunDev &P) {
@@ -300,6 +319,11 @@ cudaError_t set_smem_limits() {
 cudaError_t launch_grow(const RunDev &P, int thresh_mode, bool key64, int ctas, cudaStream_t stream) {
     if (P.d == 2) return launch_square(P, thresh_mode, ctas, stream);
     return key64 ? launch_cubic_long(P, thresh_mode, ctas, stream) : launch_cubic(P, thresh_mode, ctas, stream);
+}
+
+cudaError_t launch_counts(unsigned long long *Sn, int L, cudaStream_t stream) {
+    counts_kernel<<<1, 1024, 0, stream>>>(Sn, L);
+    return cudaGetLastError();
 }
 
 cudaError_t launch_finalize(const RunDev &P, cudaStream_t stream) {

@@ -33,7 +33,7 @@ struct RunDev {
     long long max_ns;          // wall-clock bound of the launch (bounded waits)
     // global tables: Alg. 2 one row, Alg. 1 n_seq rows of n_max+1
     double *Wn;
-    unsigned long long *Sn;
+    unsigned long long *Sn;        // differences of the node counts S_n along n, row by row
     double *Qn;
     double *Rn;                    // optional (nullptr: off): sum of W |omega_n|^2 per length
     // original PERM (nullptr: flatPERM): per length (T_n, t_n) at the stored scale; a node
@@ -143,6 +143,8 @@ cudaError_t allow_cubic();
 cudaError_t allow_cubic_long();
 cudaError_t launch_grow(const RunDev &P, int thresh_mode, bool key64, int ctas,
                         cudaStream_t stream);
+// Differences along n to counts, in place (L entries).
+cudaError_t launch_counts(unsigned long long *Sn, int L, cudaStream_t stream);
 // After a launch: the ticket counter clamped to M, the admission count of the next one.
 cudaError_t launch_finalize(const RunDev &P, cudaStream_t stream);
 cudaError_t set_smem_limits();

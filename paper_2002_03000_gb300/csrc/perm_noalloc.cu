@@ -120,6 +120,8 @@ extern "C" int perm_run_static(const perm_config *cfg, int64_t tours_per_seq, do
         if ((long long)lanes * warps <= most) break;
     }
     slots = std::min(slots, (long long)num_sms * lanes * warps);
+    // twice the hash where the CTA's walks then still fit (as a handle's run)
+    if (head + perm::walk_bytes(key64, n_max, log2h + 1, K) * (size_t)(lanes * warps) <= optin && log2h < 16) ++log2h;
     const int ctas = (int)((slots + (long long)warps * lanes - 1) / ((long long)warps * lanes));
 
     unsigned char *p = static_cast<unsigned char *>(base);
@@ -164,6 +166,8 @@ extern "C" int perm_run_static(const perm_config *cfg, int64_t tours_per_seq, do
     P.trace_cap = 0; P.trace_every = 1; P.trace_tour_every = 1;
 
     e = perm::launch_grow(P, snap ? perm::kSnapshot : perm::kFresh, key64, ctas, st);
+    if (e != cudaSuccess) return PERM_EDEVICE;
+    e = perm::launch_counts(S_n, (int)L, st);
     if (e != cudaSuccess) return PERM_EDEVICE;
     e = perm::launch_finalize(P, st);
     if (e != cudaSuccess) return PERM_EDEVICE;

@@ -420,7 +420,12 @@ __device__ __forceinline__ void grow_run(const RunDev &P, unsigned char *smem, c
     fill_constants(aoc, D, threadIdx.x, blockDim.x);
     const long long limit = P.tour_limit;
     if (snapshot) {
-        for (int k = threadIdx.x; k < L; k += blockDim.x) Wsnap[k] = *(volatile double *)(P.Wn + k);
+        for (int k = threadIdx.x; k < L; k += blockDim.x) {
+            double v = *(volatile double *)(P.Wn + k);
+            for (int q = 1; q < P.parts; ++q)
+                v = __dadd_rn(v, *(volatile double *)(P.Wp + (size_t)(q - 1) * (size_t)P.part_stride + k));
+            Wsnap[k] = v;
+        }
         __syncthreads();
         if (threadIdx.x == 0) {
             unsigned long long Ms = *(volatile unsigned long long *)P.tickets;     // after the sums, as below
@@ -454,6 +459,17 @@ __device__ __forceinline__ void grow_run(const RunDev &P, unsigned char *smem, c
                 for (int j = 0; j < kReloadBatch; ++j) {
                     const int k = k0 + j * 32 + lane;
                     v[j] = k < L ? ld_relaxed(P.Wn + k) : 0.0;
+                }
+                for (int q = 1; q < P.parts; ++q) {
+                    const double *Wq = P.Wp + (size_t)(q - 1) * (size_t)P.part_stride;
+                    double u[kReloadBatch];
+#pragma unroll
+                    for (int j = 0; j < kReloadBatch; ++j) {
+                        const int k = k0 + j * 32 + lane;
+                        u[j] = k < L ? ld_relaxed(Wq + k) : 0.0;
+                    }
+#pragma unroll
+                    for (int j = 0; j < kReloadBatch; ++j) v[j] = __dadd_rn(v[j], u[j]);
                 }
                 if (k0 == 0) {
                     // M read after the sums of the shortest lengths and published before them, so
@@ -598,7 +614,11 @@ __device__ __forceinline__ void grow_run(const RunDev &P, unsigned char *smem, c
     set_tours<!cutoffs>(tours, 1ull);
     uint32_t ms_low = 0u;      // the low word of the snapshot's M as last taken
     bool fresh_need = true;    // the walk has ended its tour since it last looked for work
-    double *Wrow = P.Wn;
+    // this CTA's copies of the tables (parts: a table of a kilobyte sits in one slice of L2,
+    // which adds 2.9e9 doubles a second whoever sends them)
+    const int part = snapshot && P.parts > 1 ? (int)(blockIdx.x % (unsigned)P.parts) : 0;
+    double *Wrow = part > 0 ? P.Wp + (size_t)(part - 1) * (size_t)P.part_stride : P.Wn;
+    double *Qtab = part > 0 ? P.Qp + (size_t)(part - 1) * (size_t)P.part_stride : P.Qn;
     unsigned long long *Srow = P.Sn;
     double *Rrow = P.Rn;
     double *acc = Wrow;        // the row this lane adds a node's weight to (lane 0: W_n, lane 1: the tour's sums)
@@ -781,7 +801,7 @@ __device__ __forceinline__ void grow_run(const RunDev &P, unsigned char *smem, c
                 const int s_row = __shfl_sync(kFull, own, src);
                 const int s_max = __shfl_sync(kFull, last ? row_max : -1, src);
                 const int s_seq = P.alg == PERM_ALG1 ? __shfl_sync(kFull, cur_seq, src) : 0;
-                double *Xr = P.X + (size_t)s_row * L, *Qr = P.Qn + (size_t)s_seq * L;
+                double *Xr = P.X + (size_t)s_row * L, *Qr = Qtab + (size_t)s_seq * L;
                 // eight loads in flight per lane, the first of them while the hash is emptied
                 double x[8];
 #pragma unroll

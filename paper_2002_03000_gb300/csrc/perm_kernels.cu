@@ -224,13 +224,29 @@ __global__ void philox_kernel(int B, const uint32_t *ctr, uint32_t k0, uint32_t 
     out[4 * b] = w.x; out[4 * b + 1] = w.y; out[4 * b + 2] = w.z; out[4 * b + 3] = w.w;
 }
 
-__global__ void finalize_kernel(unsigned long long *tickets, long long limit, long long *admit, unsigned long long gamma_q16) {
-    if (threadIdx.x == 0 && blockIdx.x == 0) {
-        if ((long long)*tickets > limit) *tickets = (unsigned long long)limit;
+__global__ void finalize_kernel(const RunDev P) {
+    if (threadIdx.x == 0) {
+        const long long limit = P.tour_limit;
+        if ((long long)*P.tickets > limit) *P.tickets = (unsigned long long)limit;
         // every tour has finished: what the admission rule leaves beyond them
-        const long long extra = (long long)(((unsigned long long)limit * gamma_q16) >> 16);
-        admit[0] = extra;
-        admit[1] = limit + extra;
+        const long long extra = (long long)(((unsigned long long)limit * P.ramp_gamma_q16) >> 16);
+        P.admit[0] = extra;
+        P.admit[1] = limit + extra;
+    }
+    // the tables' further copies into the first
+    if (P.parts > 1) {
+        for (int k = threadIdx.x; k <= P.n_max; k += blockDim.x) {
+            double w = P.Wn[k], q = P.Qn[k];
+            for (int r = 0; r + 1 < P.parts; ++r) {
+                const size_t at = (size_t)r * (size_t)P.part_stride + (size_t)k;
+                w = __dadd_rn(w, P.Wp[at]);
+                q = __dadd_rn(q, P.Qp[at]);
+                P.Wp[at] = 0.0;
+                P.Qp[at] = 0.0;
+            }
+            P.Wn[k] = w;
+            P.Qn[k] = q;
+        }
     }
 }
 
@@ -327,7 +343,7 @@ cudaError_t launch_counts(unsigned long long *Sn, int L, cudaStream_t stream) {
 }
 
 cudaError_t launch_finalize(const RunDev &P, cudaStream_t stream) {
-    finalize_kernel<<<1, 32, 0, stream>>>(P.tickets, P.tour_limit, P.admit, P.ramp_gamma_q16);
+    finalize_kernel<<<1, P.parts > 1 ? 256 : 32, 0, stream>>>(P);
     return cudaGetLastError();
 }
 

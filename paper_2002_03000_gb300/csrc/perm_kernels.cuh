@@ -35,6 +35,12 @@ struct RunDev {
     double *Wn;
     unsigned long long *Sn;        // differences of the node counts S_n along n, row by row
     double *Qn;
+    // interacting sequences with few lengths: a CTA adds to one of `parts` copies of W_n and
+    // Q_n (its own rows above are the first, the rest lie here, part_stride entries apart);
+    // the refresher sums them, and launch_finalize folds them into the first
+    int parts;
+    long long part_stride;
+    double *Wp, *Qp;
     double *Rn;                    // optional (nullptr: off): sum of W |omega_n|^2 per length
     // original PERM (nullptr: flatPERM): per length (T_n, t_n) at the stored scale; a node
     // above T_n makes cut_copies copies, one below t_n survives iff its first random

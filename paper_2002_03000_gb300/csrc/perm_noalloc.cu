@@ -153,7 +153,7 @@ extern "C" int perm_run_static(const perm_config *cfg, int64_t tours_per_seq, do
     P.tour_limit = tours_per_seq * (long long)n_seq;
     P.refresh_ns = cfg->refresh_ns ? (cfg->refresh_ns > 1000000 ? 1000000 : cfg->refresh_ns) : 8000;
     P.max_ns = (long long)((cfg->max_seconds > 0.0 ? cfg->max_seconds : 600.0) * 1e9);
-    P.Wn = W_n; P.Sn = S_n; P.Qn = Q_n;
+    P.Wn = W_n; P.Sn = S_n; P.Qn = Q_n; P.parts = 1;
     P.tickets = cnt + 0; P.seq_M = nullptr;
     P.X = X; P.gstk_meta = gmeta; P.gstk_w = gw;
     P.steps = cnt + 1; P.max_stack = cnt + 2; P.copies = cnt + 3; P.refreshes = cnt + 4;

@@ -76,8 +76,9 @@ namespace {
 constexpr size_t kLine = 256;
 // Few lengths and many walks: the walks' additions to W_n and Q_n meet on a few lines.  With
 // tables of a kilobyte or two in one slice of L2 the steady rate was 1.7e9 steps/s at
-// n = 16, 2.4e9 at 64 and 2.9e9 at 128, against 5.0e9 at 256 (square, 8192 sequences).
-constexpr int kParts = 4, kPartsLengths = 200, kPartsWalks = 512;
+// n = 16, 2.4e9 at 64, 2.9e9 at 128 and 5.0e9 at 256; with four copies 3.6, 4.9, 5.2 and 5.3e9
+// (square, 8192 sequences; 8 or 16 copies the same; at n = 512 they gain nothing).
+constexpr int kParts = 4, kPartsLengths = 400, kPartsWalks = 512;
 constexpr size_t kPartStride = 544;      // doubles: 4352 bytes apart
 constexpr size_t kOneCopy = 1 << 20;   // tables up to this size come back in one copy
 enum Counter { kTickets, kSteps, kMaxStack, kCopies, kRefreshes, kIterations, kFinished, kExact, kStatus, kAdmit, kHead, kTail,

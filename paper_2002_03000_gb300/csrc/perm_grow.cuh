@@ -175,6 +175,17 @@ __device__ __forceinline__ void set_tours(Tours &t, unsigned long long M) {
     t.inv5 = __dmul_rn(5.0, t.inv1);
 }
 
+// The running average sum / M, correctly rounded: q = sum (1/M) and one step of the division
+// from the correctly rounded 1/M (M below 2^32, the sum far from the range's ends),
+// else the division itself.
+__device__ __forceinline__ double average(double sum, const Tours &t) {
+    const double q = __dmul_rn(sum, t.inv1);
+    double avg = __fma_rn(__fma_rn(-q, t.Md, sum), t.inv1, q);
+    const int es = __double2hiint(sum) >> 20;
+    if (t.Mf < 0.0f || es < 128 || es > 1920) avg = __ddiv_rn(sum, t.Md);
+    return avg;
+}
+
 struct Decision {
     int c;               // copies (0: pruned)
     bool exact;          // the decision was taken on r in double precision
@@ -194,8 +205,14 @@ __device__ __forceinline__ Decision decide_on_average(int a, double W, double av
     bool surv = false;
     o.exact = true;
     o.x = 0.0f;
-    o.r = 1.0;
-    if (!(avg == W && W > 0.0)) o.r = __ddiv_rn(W, avg);         // (W/W = 1: no division)
+    if (avg == W && W > 0.0) {
+        // r = 1 exactly (of a lone sequence at every n <= 3, where every weight is the same)
+        o.r = 1.0;
+        o.c = 1;
+        o.child_w = __dmul_rn(W, a_sc);
+        return o;
+    }
+    o.r = __ddiv_rn(W, avg);
     o.c = decide_exact(o.r, a, w0, surv);
     if (surv) o.child_w = __dmul_rn(__dmul_rn(W, __ddiv_rn(1.0, o.r)), a_sc);
     else o.child_w = o.c > 1 ? __dmul_rn(__ddiv_rn(W, (double)o.c), a_sc) : __dmul_rn(W, a_sc);
@@ -235,8 +252,9 @@ __device__ __forceinline__ Decision decide_node(int n, int a, double W, double s
     // is far from the subnormals); the weight is within 2^-51 of the quotient
     double base = W, fac = row[c];
     if (refine) {
+        // (under a branch: three dependent operations of 62 cycles, which ran no faster beside
+        // the probes)
         if (surv) {
-            // q = sum (1/M), then q + (sum - q M)/M: the quotient to half a unit
             const double q = __dmul_rn(sum, t.inv1);
             base = __fma_rn(__fma_rn(-q, t.Md, sum), t.inv1, q);
             fac = row[0];
@@ -252,15 +270,7 @@ __device__ __forceinline__ Decision decide_node(int n, int a, double W, double s
     o.c = c;
     // the estimate cannot settle a comparison: r exactly as defined
     if (exact && refine) {
-        // fresh form (of a lone sequence the lengths n <= 3 come here at every tour: every
-        // weight is the same and r = 1 exactly).  The average by one step of the division
-        // from the correctly rounded 1/M (M below 2^32, the sum far from the range's ends),
-        // else by the division itself
-        const double q = __dmul_rn(sum, t.inv1);
-        double avg = __fma_rn(__fma_rn(-q, t.Md, sum), t.inv1, q);
-        const int es = __double2hiint(sum) >> 20;
-        if (t.Mf < 0.0f || es < 128 || es > 1920) avg = __ddiv_rn(sum, t.Md);
-        o = decide_on_average(a, W, avg, w0, row[0]);
+        o = decide_on_average(a, W, average(sum, t), w0, row[0]);
     } else if (exact) {
         o = decide_node_exact(a, W, sum, t.M, w0, row[0]);
     }

@@ -200,7 +200,8 @@ __global__ void __launch_bounds__(32) debug_step_kernel(int n_max, int log2h, in
     const bool decides = grows_on && a > 0;
     Tours t;
     set_tours<true>(t, M);
-    const Decision o = decide_node<D>(good ? n : 0, a > 0 ? a : 1, W, __dadd_rn(Wsum, W), guess(W, Wsum, t.Mf, w.x), t,
+    const double sum = __dadd_rn(Wsum, W);
+    const Decision o = decide_node<D>(good ? n : 0, a > 0 ? a : 1, W, sum, guess(W, Wsum, t.Mf, w.x), t,
                                       true, w.x, aoc, decides, decides && force_exact != 0);
     if (!good || j != 0) return;
     const int c = decides ? o.c : 0;

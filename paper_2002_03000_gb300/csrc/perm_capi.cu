@@ -304,10 +304,22 @@ int create_impl(perm_handle *out, const perm_config *cfg, const ForcedLayout *fo
         lanes = (t + max_w - 1) / max_w;
         warps = (t + lanes - 1) / lanes;
     };
+    // automatic: at most 32 walks per SM, on the square lattice (8 walks a warp at most) 48
+    // or 40 where twice the hash then still fits, else 40 where they fit.  GB300, ms at 32 /
+    // 40 / 48 / 56 walks, 8192 sequences: n = 128, 64 tours continued 13.8 / 12.0 / 10.9 / 10.6,
+    // from empty tables 19.5 / 18.5 / 17.2 / 17.4; n = 256, 32 tours 14.9 / 13.4 / 13.4 (48
+    // without the larger hash) / 13.7 and 25.7 / 24.2 / 25.0 / 25.6; n = 512, 16 tours 20.5 /
+    // 20.0 / 21.3 (42) and 44.0 / 42.2 / 44.6
+    int auto_walks = kAutoWalks;
+    if (arena_mode == perm::kArenaNone && max_l * max_w > kAutoWalks) {
+        const size_t twice = log2h < 16 ? perm::walk_bytes(key64, n_max, log2h + 1, h->stack_cache) : budget;
+        if (head_b + twice * 48 <= budget) auto_walks = 48;
+        else if (head_b + twice * 40 <= budget || head_b + walk_b * 40 <= budget) auto_walks = 40;
+    }
     if (force) {
-        // every CTA of the batch grid may join this run: the most walks up to 32 (the
-        // automatic layout's bound) that fit the shared memory
-        for (int t = kAutoWalks; t >= 1 && !warps; --t) {
+        // every CTA of the batch grid may join this run: the most walks up to the automatic
+        // layout's bound that fit the shared memory
+        for (int t = auto_walks; t >= 1 && !warps; --t) {
             spread(t);
             if (smem_for(warps * lanes) > budget) warps = 0;
         }
@@ -317,8 +329,11 @@ int create_impl(perm_handle *out, const perm_config *cfg, const ForcedLayout *fo
     }
     for (; !force;) {
         const long long per_cta = (slots + h->num_sms - 1) / h->num_sms;
-        // automatic: at most 32 walks per SM.  More lengthen the start-up and buy little
-        const int cap = lpw ? max_w * std::min(lpw, max_l) : kAutoWalks;
+        const int cap = lpw ? max_w * std::min(lpw, max_l) : auto_walks;
+        if (!lpw && per_cta > cap) {
+            slots = (long long)h->num_sms * cap;
+            continue;
+        }
         if (per_cta <= cap) {
             if (lpw) {
                 lanes = (int)std::min<long long>(per_cta, std::min(lpw, max_l));

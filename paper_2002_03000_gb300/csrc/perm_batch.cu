@@ -198,7 +198,7 @@ int perm_batch_create_persistent(perm_batch_handle *out, const perm_config *cfgs
     if (rc == PERM_OK && (perm::batch_grid(threads, smem, &resident) != cudaSuccess || resident < grid))
         rc = PERM_EUNSUPPORTED;
     if (rc == PERM_OK && cudaMalloc((void **)&b->d_runs, sizeof(perm::RunDev) * R) != cudaSuccess) rc = PERM_ENOMEM;
-    if (rc == PERM_OK && cudaMalloc((void **)&b->d_ctl, sizeof(int) * (3 * (size_t)R + 1)) != cudaSuccess) rc = PERM_ENOMEM;
+    if (rc == PERM_OK && cudaMalloc((void **)&b->d_ctl, sizeof(int) * (3 * (size_t)R + 1 + (size_t)grid)) != cudaSuccess) rc = PERM_ENOMEM;
     if (rc == PERM_OK &&
         cudaMemcpy(b->d_runs, P.data(), sizeof(perm::RunDev) * R, cudaMemcpyHostToDevice) != cudaSuccess)
         rc = PERM_EDEVICE;
@@ -209,6 +209,8 @@ int perm_batch_create_persistent(perm_batch_handle *out, const perm_config *cfgs
     B.granted = b->d_ctl + R;
     B.closed = b->d_ctl + 2 * R;
     B.runs_open = b->d_ctl + 3 * R;
+    B.first = b->d_ctl + 3 * R + 1;
+    B.ctas = grid;
     B.max_ns = (long long)(max_s * 1e9);
     B.plain = all_plain(P);
     // capture: reset every run, the batch kernel, clamp each run's tour counter
@@ -301,6 +303,8 @@ int perm_batch_continue(perm_batch_handle b, const int64_t *extra_tours_per_seq)
         B.granted = b->d_ctl + b->R;
         B.closed = b->d_ctl + 2 * b->R;
         B.runs_open = b->d_ctl + 3 * b->R;
+        B.first = b->d_ctl + 3 * b->R + 1;
+        B.ctas = b->grid;
         B.max_ns = b->max_ns;
         B.plain = all_plain(P);
         if (perm::launch_batch(B, b->grid, b->threads, b->smem, b->origin) != cudaSuccess) return PERM_EDEVICE;

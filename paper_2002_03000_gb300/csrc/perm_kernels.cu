@@ -17,65 +17,78 @@ namespace {
 // no run open, a CTA joins an unfinished run (a stalled one first) as a helper
 // whose walks take waiting copies only.
 // ---------------------------------------------------------------------------
+// Takes walks of run r for this CTA (one walk per sequence over all CTAs); 0: none left.
+__device__ int grant_walks(const BatchDev &B, int r) {
+    const RunDev &Q = B.runs[r];
+    const int cap = Q.worker_warps * Q.S;
+    for (int attempt = 0; attempt < 64; ++attempt) {
+        const int g = *(volatile int *)(B.granted + r);
+        const int k = Q.n_seq - g < cap ? Q.n_seq - g : cap;
+        if (k <= 0) break;
+        if (atomicCAS(B.granted + r, g, g + k) == g) {
+            if (g + k >= Q.n_seq && (atomicOr(B.closed + r, 2) & 3) == 0) atomicSub(B.runs_open, 1);
+            return k;
+        }
+    }
+    return 0;
+}
+
 // Returns the run to join (walks: how many of the CTA's walks grow tours), -1
 // when no run can take the CTA now, -2 when every run has finished or failed.
 __device__ int pick_run(const BatchDev &B, int &walks, bool &helper) {
-    int best = -1, stall = -1;
-    double best_s = -1.0, stall_s = -1.0;
-    bool best_open = false, unfinished = false;
-    for (int r = 0; r < B.R; ++r) {
-        const RunDev &Q = B.runs[r];
-        if (*(volatile int *)Q.status != 0) continue;
-        const long long lim = Q.tour_limit;
-        const long long f = (long long)*(volatile unsigned long long *)Q.finished;
-        if (f >= lim) continue;
-        unfinished = true;
-        const long long t = (long long)*(volatile unsigned long long *)Q.tickets;
-        const int a = *(volatile int *)(B.active + r);
-        const int g = *(volatile int *)(B.granted + r);
-        const double len = (double)(Q.n_max + 1);
-        // a run stalled on a large tour is the batch's critical path: among runs
-        // that take helpers it comes first, up to the CTAs its parts can use
-        const int fl = *(volatile int *)(B.closed + r);
-        if ((fl & kStalledBit) && Q.share && a * Q.worker_warps * Q.S < Q.share_boost) {
-            const double sc = (double)(lim - f) * len / (double)(a + 1);
-            if (sc > stall_s) { stall = r; stall_s = sc; }
-        }
-        if (t < lim) {
-            if (g < Q.n_seq) {
-                const double sc = (double)(lim - t) * len / (double)(a + 1);
-                if (!best_open || sc > best_s) { best = r; best_s = sc; best_open = true; }
-            }
-        } else if (!best_open && Q.share) {
-            const double sc = (double)(lim - f) * len / (double)(a + 1);
-            if (sc > best_s) { best = r; best_s = sc; }
-        }
-    }
     walks = 0;
     helper = false;
-    if (stall >= 0 && !best_open) best = stall;
-    if (best < 0) return unfinished ? -1 : -2;
-    const RunDev &Q = B.runs[best];
-    const int cap = Q.worker_warps * Q.S;
-    if (best_open) {
-        // grant up to a CTA's worth of walks, never more than one per sequence
-        for (int attempt = 0; attempt < 64; ++attempt) {
-            const int g = *(volatile int *)(B.granted + best);
-            const int k = Q.n_seq - g < cap ? Q.n_seq - g : cap;
-            if (k <= 0) break;
-            if (atomicCAS(B.granted + best, g, g + k) == g) {
-                walks = k;
-                if (g + k >= Q.n_seq && (atomicOr(B.closed + best, 2) & 3) == 0) atomicSub(B.runs_open, 1);
-                break;
+    for (int attempt = 0; attempt < 4; ++attempt) {
+        int best = -1, stall = -1, seen = 0;
+        double best_s = -1.0, stall_s = -1.0, next_s = -1.0, best_w = 0.0;
+        bool best_open = false, unfinished = false;
+        for (int r = 0; r < B.R; ++r) {
+            const RunDev &Q = B.runs[r];
+            if (*(volatile int *)Q.status != 0) continue;
+            const long long lim = Q.tour_limit;
+            const long long f = (long long)*(volatile unsigned long long *)Q.finished;
+            if (f >= lim) continue;
+            unfinished = true;
+            const long long t = (long long)*(volatile unsigned long long *)Q.tickets;
+            const int a = *(volatile int *)(B.active + r);
+            const int g = *(volatile int *)(B.granted + r);
+            const double len = (double)(Q.n_max + 1);
+            // a run stalled on a large tour is the batch's critical path: among runs
+            // that take helpers it comes first, up to the CTAs its parts can use
+            const int fl = *(volatile int *)(B.closed + r);
+            if ((fl & kStalledBit) && Q.share && a * Q.worker_warps * Q.S < Q.share_boost) {
+                const double sc = (double)(lim - f) * len / (double)(a + 1);
+                if (sc > stall_s) { stall = r; stall_s = sc; }
             }
+            const bool open = t < lim;
+            if (open ? g >= Q.n_seq : (best_open || !Q.share)) continue;
+            const double w = (double)(open ? lim - t : lim - f) * len, sc = w / (double)(a + 1);
+            if (open && !best_open) { best_s = next_s = -1.0; best_open = true; }
+            if (sc > best_s) { next_s = best_s; best = r; best_s = sc; best_w = w; seen = a; }
+            else if (sc > next_s) next_s = sc;
         }
-        if (walks == 0) return -1;
-    } else {
-        walks = cap;                    // helper
-        helper = true;
+        if (stall >= 0 && !best_open) { best = stall; next_s = -1.0; }
+        if (best < 0) return unfinished ? -1 : -2;
+        // CTAs that look at the same moment see the same best run: one that finds others have
+        // joined it since looks again while another run now comes before it
+        const int now = atomicAdd(B.active + best, 1);
+        if (attempt < 3 && now > seen && best_w / (double)(now + 1) < next_s) {
+            atomicSub(B.active + best, 1);
+            continue;
+        }
+        if (best_open) {
+            walks = grant_walks(B, best);
+            if (walks == 0) {
+                atomicSub(B.active + best, 1);
+                return -1;
+            }
+        } else {
+            walks = B.runs[best].worker_warps * B.runs[best].S;
+            helper = true;
+        }
+        return best;
     }
-    atomicAdd(B.active + best, 1);
-    return best;
+    return -1;
 }
 
 template <int MODE, int FORM>
@@ -84,11 +97,21 @@ __global__ void __launch_bounds__(32 * 9, 1) batch_kernel(const BatchDev B) {
     __shared__ RunDev Ps;
     __shared__ int cur, walks, helping;
     const long long t0 = global_ns();
-    for (;;) {
+    for (bool at_start = true;; at_start = false) {
         if (threadIdx.x == 0) {
             int w = 0;
             bool hp = false;
-            int r = pick_run(B, w, hp);
+            int r = -1;
+            if (at_start) {
+                // (the launch's first runs were shared out by batch_init_kernel)
+                r = B.first[blockIdx.x];
+                if (r >= 0) {
+                    w = grant_walks(B, r);
+                    if (w > 0) atomicAdd(B.active + r, 1);
+                    else r = -1;
+                }
+            }
+            if (r < 0) r = pick_run(B, w, hp);
             helping = hp ? 1 : 0;
             if (r == -1 && global_ns() - t0 > B.max_ns) {
                 // the batch's time is up: every run not finished fails
@@ -127,22 +150,59 @@ __global__ void __launch_bounds__(32 * 9, 1) batch_kernel(const BatchDev B) {
 }
 
 // Scheduling counters of a batch launch: nothing granted, no CTA on a run; a run
-// with no tours left to start counts as closed.
+// with no tours left to start counts as closed.  And each CTA's first run: the CTAs go
+// one by one to the run with the most work per CTA already given (at most the CTAs that
+// hold one walk per sequence).  When every CTA chose for itself at the launch's start,
+// they all saw the same empty counts, filled the largest runs and left the others, with
+// their start-up, for later (24 runs of n = 64..256, 8 tours: 21.1 ms, so 15.5).
+// One block of 256 threads; past kSharedOut runs every CTA chooses for itself.
+constexpr int kSharedOut = 512;
 __global__ void batch_init_kernel(const BatchDev B) {
     __shared__ int open;
+    __shared__ float work[kSharedOut];     // 0: takes no CTA
+    __shared__ int given[kSharedOut], most[kSharedOut];
     if (threadIdx.x == 0) open = 0;
     __syncthreads();
     for (int r = threadIdx.x; r < B.R; r += blockDim.x) {
         // a run grows in this launch if it has tours left to start (a continued
         // batch leaves retired runs with none)
-        const bool grows = B.runs[r].tour_limit > (long long)*(volatile unsigned long long *)B.runs[r].tickets;
+        const RunDev &Q = B.runs[r];
+        const long long left = Q.tour_limit - (long long)*(volatile unsigned long long *)Q.tickets;
+        const bool grows = left > 0;
         B.active[r] = 0;
         B.granted[r] = 0;
         B.closed[r] = grows ? 0 : 3;
         if (grows) atomicAdd(&open, 1);
+        if (r < kSharedOut) {
+            const int cap = Q.worker_warps * Q.S;
+            work[r] = grows ? (float)left * (float)(Q.n_max + 1) : 0.0f;
+            given[r] = 0;
+            most[r] = (Q.n_seq + cap - 1) / cap;
+        }
     }
     __syncthreads();
     if (threadIdx.x == 0) *B.runs_open = open;
+    if (threadIdx.x >= 32) return;
+    const int lane = threadIdx.x, R = B.R <= kSharedOut ? B.R : 0;
+    for (int b = 0; b < B.ctas; ++b) {
+        float best_s = 0.0f;
+        int best = -1;
+        for (int r = lane; r < R; r += 32) {
+            const float sc = given[r] < most[r] ? work[r] / (float)(given[r] + 1) : 0.0f;
+            if (sc > best_s) { best_s = sc; best = r; }
+        }
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) {
+            const float os = __shfl_xor_sync(kFull, best_s, off);
+            const int ob = __shfl_xor_sync(kFull, best, off);
+            if (os > best_s || (os == best_s && ob > best)) { best_s = os; best = ob; }
+        }
+        if (lane == 0) {
+            B.first[b] = best;
+            if (best >= 0) given[best] += 1;
+        }
+        __syncwarp();
+    }
 }
 
 // ---------------------------------------------------------------------------

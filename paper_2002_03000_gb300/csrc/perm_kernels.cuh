@@ -102,6 +102,8 @@ struct BatchDev {
     int *active;          // per run: CTAs on it now
     int *granted;         // per run: tour-growing walks handed to CTAs
     int *runs_open;       // runs with tours to start and walks to grant
+    int *first;           // per CTA: the run it joins first (-1: none)
+    int ctas;             // of the launch
     bool plain;           // no run has cut-offs, observables or a trace
     int *closed;          // per run: bit 0 tickets exhausted, bit 1 walks all granted
     long long max_ns;     // wall-clock bound of the launch

@@ -13,7 +13,7 @@
 //     one.  Every lane of a group carries the walk's state; lane j of the group
 //     stands for direction j.
 //   - A walk's occupancy hash, its per-site slot list and its stack ring are
-//     contiguous.  The hash is made of 16-byte buckets.
+//     contiguous.  The hash is made of buckets of 4 keys.
 //   - Keys pack the lattice coordinates of a site; 0 is the empty slot.  The key of
 //     neighbour j is the site's key plus a constant of the direction.
 //   - Directions: j = 0..2d-1 -> axis j/2, sign + for even j (+x,-x,+y,-y,+z,-z).
@@ -104,19 +104,21 @@ __device__ __forceinline__ Key step_key(int j) {
 }
 
 // ---------------------------------------------------------------------------
-// The occupancy hash: 2^log2b buckets of 16 bytes (4 keys of 32 bits or 2 of 64),
+// The occupancy hash: 2^log2b buckets of 4 keys (16 bytes, or 32 with 64-bit keys),
 // probed triangularly from the key's home: the i-th bucket is home + i(i+1)/2 mod
 // 2^log2b, which visits every bucket once.  A key sits in the first bucket of its
 // sequence with room, in that bucket's first empty place.  Keys are deleted in
 // LIFO order only, so a bucket's keys always fill its first places, every bucket
 // that a key passed over is full while the key lives, and a probe may stop at the
-// first bucket that is not full.  One 16-byte load settles a probe unless the
-// bucket is full: at the load of at most 1/2 that a walk reaches at n_max, one
-// bucket of four in seven is full, against one slot in two with one key per probe.
+// first bucket that is not full.  One look at a bucket (a 16-byte load, or two that
+// are in flight together) settles a probe unless it is full: at the load of at most
+// 1/2 that a walk reaches at n_max, one bucket of four in seven is full, against one
+// slot in two with one key per probe.  64-bit keys went in twos before, one load a
+// look and more looks: cubic Algorithm 1 at n_max 4096 47.6 ms against 49.1, 1000
+// 21.5 against 22.6, 10000 (tables in L2) 94.9 against 97.0.
 // ---------------------------------------------------------------------------
 template <typename Key> struct Buckets {
-    static constexpr int kKeys = 16 / (int)sizeof(Key);
-    static constexpr int kLog2 = sizeof(Key) == 4 ? 2 : 1;
+    static constexpr int kKeys = 4, kLog2 = 2;
 };
 
 __device__ __forceinline__ uint32_t hash_home(uint32_t k, int log2b) {
@@ -136,10 +138,11 @@ __device__ __forceinline__ void look_bucket(const uint32_t *tab, uint32_t b, uin
 }
 __device__ __forceinline__ void look_bucket(const unsigned long long *tab, uint32_t b, unsigned long long k, bool &hit,
                                             bool &full, int &e) {
-    const ulonglong2 v = *reinterpret_cast<const ulonglong2 *>(tab + 2u * b);
-    hit = v.x == k || v.y == k;
-    full = v.y != 0ull;
-    e = v.x != 0ull;
+    const ulonglong2 v = *reinterpret_cast<const ulonglong2 *>(tab + 4u * b);
+    const ulonglong2 u = *reinterpret_cast<const ulonglong2 *>(tab + 4u * b + 2u);
+    hit = v.x == k || v.y == k || u.x == k || u.y == k;
+    full = u.y != 0ull;
+    e = (v.x != 0ull) + (v.y != 0ull) + (u.x != 0ull);
 }
 
 // Every lane of the warp probes for its own key in its own walk's table (want:

@@ -5,7 +5,7 @@
 // cubic one, so a warp holds up to 8 or 4 walks.  Every lane of a group carries the
 // walk's state; lane j probes neighbour j, deletes every 4th (8th) site of a
 // backtrack, and issues one of the node's table updates.  Per walk, shared memory
-// holds the occupancy hash (16-byte buckets, keys deleted in LIFO order on
+// holds the occupancy hash (buckets of 4 keys, keys deleted in LIFO order on
 // backtrack), the hash slot of every site, and the top of the stack of waiting
 // copies (the rest spills to global memory).  Each walk runs the tours handed to
 // it one after another; a tour is a depth-first traversal of the tree of copies

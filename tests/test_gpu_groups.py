@@ -14,6 +14,7 @@ import pytest
 
 import paper_2002_03000_gb300 as pg
 from oracle import oracle as orc
+from paper_2002_03000_gb300 import batch as pb
 from tests import inputs
 from tests.gpu_util import REL_W, Run, torch_cuda
 
@@ -126,3 +127,18 @@ def test_interacting_runs_keep_what_holds_for_any_schedule(d, n_max, N, tours, l
     assert S[0] == N * tours and S[1] == N * tours
     assert int(S.sum()) == st["steps"]
     assert math.isclose(math.exp(lc[1]), 2 * d, rel_tol=1e-12)
+
+
+@pytest.mark.parametrize("runs", [1, 512, 513])
+def test_persistent_batches_of_tiny_runs_complete(runs):
+    """One run; the most runs whose CTAs are shared out at the start; one more."""
+    torch_cuda()
+    cfgs = [pb.make_config(2 + i % 2, 4 + i % 3, 1 + i % 5, 9, run_id=i, max_seconds=60.0) for i in range(runs)]
+    with pb.Batch(cfgs, [2] * runs, persistent=True) as b:
+        b.run()
+        for r, cfg in enumerate(cfgs):
+            lc, S, rv = b.estimates(r)
+            st = b.stats(r)
+            assert st["status"] == 0 and st["tours_finished"] == 2 * cfg.n_seq
+            assert S[0] == S[1] == 2 * cfg.n_seq and int(S.sum()) == st["steps"]
+            assert math.isclose(math.exp(lc[1]), 2 * cfg.d, rel_tol=1e-12)

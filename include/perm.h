@@ -68,7 +68,8 @@ typedef struct {
     int threshold;     /* PERM_THRESH_SNAPSHOT or PERM_THRESH_FRESH (Alg. 2 only) */
     int slots;         /* concurrent walks on the GPU; 0 = min(N, device capacity) */
     int lanes_per_warp;/* walks per warp, 1..32, at most the 8 (d=2) or 4 (d=3) that a warp
-                          holds; 0 = automatic (the walks of an SM over up to 8 warps) */
+                          holds; 0 = automatic (the walks of an SM over up to 11
+                          warps, 8 with 64-bit keys) */
     int refresh_ns;    /* snapshot refresh period in ns, paced on the SM cycle counter; 0 = default (8000) */
     double max_seconds;/* wall-clock bound of one launch; past it the kernel stops and the
                           run reports PERM_ETIMEOUT; 0 = default (600) */

@@ -112,7 +112,10 @@ void free_all(perm_handle h) {
 // complete run at 5 / 2 / 0.7 / 0.3 ms: square n = 512, 4096 x 256 215 / 210 / 208 / 208;
 // cubic n = 512, 8192 x 128 173 / 168 / 166 / 165; square n = 256, 1000 x 64 32 / 28 / 26 / 25;
 // cubic n = 945, 2142 x 4 86 / 38 / 33 / 33; square n = 1725, 422 x 4 250 / 205 / 184 / 470.
-constexpr int kAutoWalks = 32;          // walks per CTA of the automatic layout
+constexpr int kAutoWalks = 32;          // walks per CTA of the automatic layout, in the arena
+constexpr int kBatchWalks = 48;         // and of a persistent batch's members: each has scratch for
+                                        // a grid of such CTAs (24 runs of n = 64..256: 0.66, 0.76
+                                        // and 0.99 GB, 15.1, 15.4 and 15.6 ms at 40, 48 and 88)
 constexpr int kDefaultShareCap = 4;
 constexpr int kBoostShareCap = 1024;
 constexpr long long kStallNs = 700000;
@@ -254,11 +257,11 @@ int create_impl(perm_handle *out, const perm_config *cfg, const ForcedLayout *fo
     h->own_stream = true;
 
     // layout: walks per warp (lanes), walk warps per CTA, CTAs.  A group of lanes grows
-    // one walk; the walks of an SM are spread over up to 8 warps, so that every
-    // scheduler has two walks' dependent chains to issue from.
+    // one walk; the walks of an SM are spread over up to 11 warps (8 with 64-bit
+    // keys), so that every scheduler has several walks' dependent chains to issue from.
     const bool snap = (h->thresh == perm::kSnapshot);
     const size_t budget = force ? force->smem_budget : prop.sharedMemPerBlockOptin;
-    const int max_l = perm::walks_per_warp_max(d), max_w = perm::kMaxWalkWarps;
+    const int max_l = perm::walks_per_warp_max(d), max_w = perm::walk_warps_max(key64);
     size_t walk_b = perm::walk_bytes(key64, n_max, log2h, h->stack_cache);
     // where the walks' hashes, site lists and stack rings live: shared memory, or a
     // global arena when asked for or when not one walk per CTA fits beside the head
@@ -277,8 +280,9 @@ int create_impl(perm_handle *out, const perm_config *cfg, const ForcedLayout *fo
         return head_b + walk_b * (size_t)walks;
     };
     if (!force && cfg->max_ctas == -1) {
-        // dense packing: the fewest CTAs (of up to 8 full warps) that hold one walk
-        // per sequence, so that runs sharing the device take few SMs each
+        // dense packing: the fewest CTAs that hold one walk per sequence, so that runs
+        // sharing the device take few SMs each (24 runs of n = 64..256 on streams: 33.8 ms at 4
+        // full warps a CTA, 25.4 at 8, 22.6 at 11)
         long long per_cta = 0;
         for (int t = max_w * max_l; t >= 1; --t)
             if (smem_for(t) <= budget) { per_cta = t; break; }
@@ -297,29 +301,34 @@ int create_impl(perm_handle *out, const perm_config *cfg, const ForcedLayout *fo
     long long helpers = cfg->helper_walks;
     if (helpers < 0) helpers = can_help && !lpw ? std::max(0LL, (long long)h->num_sms * 32 - tslots) : 0;
     long long slots = tslots + helpers;
-    const long long slots_wanted = slots;
     int warps = 0, lanes = 0;
-    // walks of a CTA over its warps: over as many of the 8 as there are walks
+    // walks of a CTA over its warps: over as many of them as there are walks
     auto spread = [&](int t) {
         lanes = (t + max_w - 1) / max_w;
         warps = (t + lanes - 1) / lanes;
     };
-    // automatic: at most 32 walks per SM, on the square lattice (8 walks a warp at most) 48
-    // or 40 where twice the hash then still fits, else 40 where they fit.  GB300, ms at 32 /
-    // 40 / 48 / 56 walks, 8192 sequences: n = 128, 64 tours continued 13.8 / 12.0 / 10.9 / 10.6,
-    // from empty tables 19.5 / 18.5 / 17.2 / 17.4; n = 256, 32 tours 14.9 / 13.4 / 13.4 (48
-    // without the larger hash) / 13.7 and 25.7 / 24.2 / 25.0 / 25.6; n = 512, 16 tours 20.5 /
-    // 20.0 / 21.3 (42) and 44.0 / 42.2 / 44.6
-    int auto_walks = kAutoWalks;
-    if (arena_mode == perm::kArenaNone && max_l * max_w > kAutoWalks) {
-        const size_t twice = log2h < 16 ? perm::walk_bytes(key64, n_max, log2h + 1, h->stack_cache) : budget;
-        if (head_b + twice * 48 <= budget) auto_walks = 48;
-        else if (head_b + twice * 40 <= budget || head_b + walk_b * 40 <= budget) auto_walks = 40;
+    // automatic: of the layouts that fill the shared memory, the one whose walks times
+    // warps are the most.  A warp's iteration takes hardly longer for more walks, and an
+    // SM's iterations take hardly longer for more warps.  GB300, 16384 sequences, ms:
+    // n = 400, 8 tours continued, 484 (11 warps x 4 walks) 12.0, 363 (11 x 3) 13.3, 320
+    // (8 x 5) 13.5, 294 (7 x 6) 14.2, 252 (6 x 7) 15.1, 200 (5 x 8) 16.5; n = 512, 400
+    // (10 x 4) 18.5, 363 18.6, 294 20.6, 242 (11 x 2) 20.8, 200 24.5; n = 128, 32 tours,
+    // where all fit, 11 x 4 / 5 / 6 / 7 / 8 11.1 / 9.7 / 8.8 / 8.2 / 7.8, from empty tables
+    // 17.3 / 16.5 / 15.8 / 15.6 / 15.4 (the walks go before twice the hash: n = 256, 16
+    // tours, 44 with it 12.4 and 23.0, 80 without 11.3 and 23.5)
+    int auto_walks = kAutoWalks, full_l = 0;
+    if (arena_mode == perm::kArenaNone) {
+        const long long room = (long long)((budget - head_b) / walk_b);
+        long long best = 0;
+        for (int l = 1; l <= max_l; ++l) {
+            const long long w = std::min<long long>(max_w, room / l);
+            if (w * w * l > best) { best = w * w * l; full_l = l; auto_walks = (int)(w * l); }
+        }
     }
     if (force) {
         // every CTA of the batch grid may join this run: the most walks up to the automatic
         // layout's bound that fit the shared memory
-        for (int t = auto_walks; t >= 1 && !warps; --t) {
+        for (int t = std::min(auto_walks, kBatchWalks); t >= 1 && !warps; --t) {
             spread(t);
             if (smem_for(warps * lanes) > budget) warps = 0;
         }
@@ -327,33 +336,27 @@ int create_impl(perm_handle *out, const perm_config *cfg, const ForcedLayout *fo
         if (!warps || slots > (1LL << 30)) { cudaStreamDestroy(h->stream); delete h; return PERM_EUNSUPPORTED; }
         h->num_sms = force->ctas;
     }
-    for (; !force;) {
-        const long long per_cta = (slots + h->num_sms - 1) / h->num_sms;
-        const int cap = lpw ? max_w * std::min(lpw, max_l) : auto_walks;
-        if (!lpw && per_cta > cap) {
-            slots = (long long)h->num_sms * cap;
-            continue;
-        }
-        if (per_cta <= cap) {
+    if (!force) {
+        // the walks that the SMs share, or the most of them that fit
+        long long t = std::min<long long>((slots + h->num_sms - 1) / h->num_sms,
+                                          lpw ? max_w * std::min(lpw, max_l) : auto_walks);
+        for (; t >= 1 && !warps; --t) {
             if (lpw) {
-                lanes = (int)std::min<long long>(per_cta, std::min(lpw, max_l));
-                warps = (int)((per_cta + lanes - 1) / lanes);
+                lanes = (int)std::min<long long>(t, std::min(lpw, max_l));
+                warps = (int)((t + lanes - 1) / lanes);
+            } else if (t == auto_walks && full_l) {
+                lanes = full_l;
+                warps = auto_walks / full_l;
             } else {
-                spread((int)per_cta);
+                spread((int)t);
             }
-            if (smem_for(warps * lanes) <= budget) break;
-            warps = 0;
+            if (smem_for(warps * lanes) > budget) warps = 0;
         }
-        if (slots <= 1) break;
-        slots = slots - (slots + 7) / 8;        // does not fit: fewer concurrent walks
     }
     if (!warps) { cudaStreamDestroy(h->stream); delete h; return PERM_EUNSUPPORTED; }
     const long long per_cta_eff = (long long)warps * lanes;
-    // with the layout fixed, use every SM (sequences beyond it wait at tour boundaries)
-    if (!force && slots < slots_wanted) {
-        const long long cap = (long long)h->num_sms * per_cta_eff;
-        slots = slots_wanted < cap ? slots_wanted : cap;
-    }
+    // (sequences beyond the layout wait at tour boundaries)
+    if (!force) slots = std::min(slots, (long long)h->num_sms * per_cta_eff);
     h->ctas = (int)((slots + per_cta_eff - 1) / per_cta_eff);
     // helpers are the walks beyond the tour walks (fewer when not all fit).  A batch
     // member is laid out for the whole grid and its walks are granted per sequence by

@@ -1393,7 +1393,7 @@ __device__ __forceinline__ void grow_run(const RunDev &P, unsigned char *smem, c
 
 // A launch's kernel.  (Walks in the arena: the two forms that are not plain serve them.)
 template <int D, typename Key, int MODE, int FORM>
-__global__ void __launch_bounds__(32 * 9, 1) grow_kernel(const __grid_constant__ RunDev P) {
+__global__ void __launch_bounds__(32 * (walk_warps_max(sizeof(Key) == 8) + 1), 1) grow_kernel(const __grid_constant__ RunDev P) {
     extern __shared__ __align__(16) unsigned char smem[];
     if (FORM == kPlain || P.arena_mode == kArenaNone)
         grow_run<D, Key, MODE, true, FORM>(P, smem, nullptr, P.worker_warps * P.S);

@@ -92,7 +92,7 @@ __device__ int pick_run(const BatchDev &B, int &walks, bool &helper) {
 }
 
 template <int MODE, int FORM>
-__global__ void __launch_bounds__(32 * 9, 1) batch_kernel(const BatchDev B) {
+__global__ void __launch_bounds__(32 * (walk_warps_max(false) + 1), 1) batch_kernel(const BatchDev B) {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ RunDev Ps;
     __shared__ int cur, walks, helping;

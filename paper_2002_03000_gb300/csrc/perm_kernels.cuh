@@ -137,10 +137,13 @@ int member_extend(perm_handle h, int64_t extra_tours_per_seq, int run_index, Run
 // Bytes of a CTA's head region, and of one walk's region.
 size_t cta_head_bytes(int n_max, bool snapshot);
 size_t walk_bytes(bool key64, int n_max, int log2h, int stack_cache);
-// Walks that a warp holds at most (a walk takes a group of its lanes), and walk
-// warps of a CTA.
+// Walks that a warp holds at most (a walk takes a group of its lanes), and walk warps of
+// a CTA: with the refresher 12 warps, the most that leave each the 168 registers that
+// the loop takes.  8 warps before: square n = 512, 4096 sequences continued 53.1 -> 50.0 ms,
+// cubic, 8192, 55.4 -> 47.8 ms (12 warps of 160 registers 56.7 and 54.2, 14 of 128 54.2
+// and 49.4).  With 64-bit keys at most 13 walks fit an SM, and more registers stay free.
 int walks_per_warp_max(int d);
-constexpr int kMaxWalkWarps = 8;
+constexpr int walk_warps_max(bool key64) { return key64 ? 8 : 11; }
 
 // One lattice and key width each (perm_grow_*.cu), and their shared memory limits.
 cudaError_t launch_square(const RunDev &P, int thresh_mode, int ctas, cudaStream_t stream);

@@ -97,7 +97,7 @@ extern "C" int perm_run_static(const perm_config *cfg, int64_t tours_per_seq, do
         return PERM_EDEVICE;
     const size_t optin = (size_t)smem_optin;
 
-    // layout: walks over up to 8 warps per CTA, as many as shared memory allows, one
+    // layout: walks over up to 11 warps per CTA (8 with 64-bit keys), as many as shared memory allows, one
     // CTA per SM
     const bool snap = (cfg->threshold == PERM_THRESH_SNAPSHOT);
     int log2h = 4;
@@ -105,8 +105,9 @@ extern "C" int perm_run_static(const perm_config *cfg, int64_t tours_per_seq, do
     const int K = 16;
     const size_t head = perm::cta_head_bytes(n_max, snap), walk = perm::walk_bytes(key64, n_max, log2h, K);
     if (head + walk > optin) return PERM_EUNSUPPORTED;
+    const int max_w = perm::walk_warps_max(key64);
     const long long most = std::min((long long)((optin - head) / walk),
-                                    (long long)perm::kMaxWalkWarps * perm::walks_per_warp_max(d));
+                                    (long long)max_w * perm::walks_per_warp_max(d));
 
     long long slots = cfg->slots ? cfg->slots : n_seq;
     if (slots > n_seq) slots = n_seq;
@@ -115,7 +116,7 @@ extern "C" int perm_run_static(const perm_config *cfg, int64_t tours_per_seq, do
     long long per_cta = (slots + num_sms - 1) / num_sms;
     int lanes = 1, warps = 1;
     for (;; --per_cta) {                        // whole warps of `lanes` walks, within shared memory
-        lanes = (int)((per_cta + perm::kMaxWalkWarps - 1) / perm::kMaxWalkWarps);
+        lanes = (int)((per_cta + max_w - 1) / max_w);
         warps = (int)((per_cta + lanes - 1) / lanes);
         if ((long long)lanes * warps <= most) break;
     }

@@ -52,6 +52,10 @@ LAYOUTS = [
     (3, 513, 40, 3, dict(threshold=SNAP, hash_scale=1)),        # 64-bit keys
     (2, 90, 40, 5, dict(threshold=SNAP, walk_memory=2)),        # walks in the arena
     (3, 600, 20, 3, dict(threshold=FRESH, walk_memory=2, hash_scale=2)),
+    (2, 40, 90, 4, dict(threshold=SNAP, max_ctas=1)),           # one full CTA: 88 walks, 44, 13
+    (3, 40, 50, 4, dict(threshold=FRESH, max_ctas=1)),
+    (3, 513, 30, 2, dict(threshold=SNAP, max_ctas=1, lanes_per_warp=2)),
+    (2, 300, 60, 2, dict(threshold=SNAP, max_ctas=-1)),
 ]
 
 

@@ -55,6 +55,7 @@ LAYOUTS = [
     (2, 40, 90, 4, dict(threshold=SNAP, max_ctas=1)),           # one full CTA: 88 walks, 44, 13
     (3, 40, 50, 4, dict(threshold=FRESH, max_ctas=1)),
     (3, 513, 30, 2, dict(threshold=SNAP, max_ctas=1, lanes_per_warp=2)),
+    (2, 63, 77, 6, dict(threshold=SNAP, ramp_c0=3)),            # an admission limit of the caller's
     (2, 300, 60, 2, dict(threshold=SNAP, max_ctas=-1)),
 ]
 
@@ -131,6 +132,24 @@ def test_interacting_runs_keep_what_holds_for_any_schedule(d, n_max, N, tours, l
     assert S[0] == N * tours and S[1] == N * tours
     assert int(S.sum()) == st["steps"]
     assert math.isclose(math.exp(lc[1]), 2 * d, rel_tol=1e-12)
+
+
+def test_flatperm_after_cutoffs_without_an_admission_limit():
+    """Cut-offs admit every tour at once; the limit holds again for flatPERM after them."""
+    torch_cuda()
+    d, n_max, N = 2, 100, 700
+    hi, lo = _cuts(d, n_max, 1.4)
+    with Run(d, n_max, N, 12) as run:
+        for k in (1, 2):
+            run.set_cutoffs(hi, lo, 2, 2.0)
+            run.run(2)
+            run.set_cutoffs(None, None)
+            run.run(3)
+            lc, S, rv = run.estimates()
+            st = run.stats()
+            assert st["status"] == 0 and st["tours_finished"] == 5 * k * N
+            assert S[0] == S[1] == 5 * k * N and int(S.sum()) == st["steps"]
+            assert math.isclose(math.exp(lc[1]), 2 * d, rel_tol=1e-12)
 
 
 @pytest.mark.parametrize("runs", [1, 512, 513])

@@ -114,8 +114,9 @@ __device__ __forceinline__ Key step_key(int j) {
 // are in flight together) settles a probe unless it is full: at the load of at most
 // 1/2 that a walk reaches at n_max, one bucket of four in seven is full, against one
 // slot in two with one key per probe.  64-bit keys went in twos before, one load a
-// look and more looks: cubic Algorithm 1 at n_max 4096 47.6 ms against 49.1, 1000
-// 21.5 against 22.6, 10000 (tables in L2) 94.9 against 97.0.
+// look and more looks: cubic chains (no cut-off active) at n_max 4096, 608 sequences,
+// 4 tours 14.8 ms against 15.3, 1000, 1000 sequences, 8 tours 4.8 against 5.05, 10000
+// (walks in the arena), 608 sequences, 4 tours 24.5 against 26.3.
 // ---------------------------------------------------------------------------
 template <typename Key> struct Buckets {
     static constexpr int kKeys = 4, kLog2 = 2;

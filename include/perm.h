@@ -82,7 +82,8 @@ typedef struct {
                           -1 = as few CTAs as hold one walk per sequence (dense packing).
                           Lets concurrent runs share the device */
     int hash_scale;    /* per-walk occupancy hash has 2^hash_scale * 2 n_max slots
-                          (rounded up to a power of 2); 0..2 */
+                          (rounded up to a power of 2); 0..2.  With 0 it has twice as
+                          many where the CTA's walks still fit in shared memory */
     int share_copies;  /* Algorithm 2 with snapshot thresholds: a walk with no tour to
                           start (admission limit, or no tickets left) takes the oldest
                           waiting copy of another walk's tour and grows its subtree; the

@@ -3,8 +3,7 @@
 Runs whose tables do not depend on the schedule (cut-offs without sharing,
 Algorithm 1, a single fresh sequence) equal the oracle's at any layout: the
 shortest walks, more or fewer walks than a warp holds, walks in the arena, the
-last cubic length with 32-bit keys and the first with 64-bit ones, the longest
-table kept in four copies and the first that is not.  Counts exactly, weight
+last cubic length with 32-bit keys and the first with 64-bit ones.  Counts exactly, weight
 sums to relative 1e-12: only the order of the sums differs, and no length gets
 more than 4000 positive terms here (k of them agree to k 2^-53, 4.5e-13)."""
 import math
@@ -44,10 +43,10 @@ LAYOUTS = [
     (3, 3, 33, 4, dict(threshold=SNAP, lanes_per_warp=1)),
     (2, 63, 77, 6, dict(threshold=SNAP, lanes_per_warp=3, slots=50)),
     (3, 63, 77, 6, dict(threshold=FRESH, lanes_per_warp=3, max_ctas=2)),
-    (2, 400, 1100, 2, dict(threshold=SNAP)),                    # four copies of W_n and Q_n
+    (2, 400, 1100, 2, dict(threshold=SNAP)),                    # flatPERM: four copies of the tables
     (2, 401, 1100, 2, dict(threshold=SNAP)),                    # one
-    (2, 400, 1100, 2, dict(threshold=SNAP, slots=511)),         # one
-    (3, 100, 700, 3, dict(threshold=SNAP, observables=1)),      # four copies, watched
+    (2, 400, 1100, 2, dict(threshold=SNAP, slots=511)),
+    (3, 100, 700, 3, dict(threshold=SNAP, observables=1)),      # watched
     (3, 512, 40, 3, dict(threshold=SNAP, stack_ring=128)),      # 32-bit keys
     (3, 513, 40, 3, dict(threshold=SNAP, hash_scale=1)),        # 64-bit keys
     (2, 90, 40, 5, dict(threshold=SNAP, walk_memory=2)),        # walks in the arena

@@ -14,7 +14,7 @@ OUT_DIR = os.path.join(HERE, "_build")
 LIB = os.path.join(OUT_DIR, "libperm.so")
 SOURCES = ["perm_kernels.cu", "perm_grow_square.cu", "perm_grow_cubic.cu", "perm_grow_cubic_long.cu",
             "perm_capi.cu", "perm_noalloc.cu", "perm_batch.cu"]
-HEADERS = ["perm_device.cuh", "perm_kernels.cuh", "perm_grow.cuh"]
+HEADERS = ["perm_device.cuh", "perm_kernels.cuh", "perm_grow.cuh", "perm_parts.h"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "--fmad=false", "-Xcompiler", "-fPIC",
          "-I", os.path.join(ROOT, "include"), "-I", CSRC]

@@ -49,6 +49,7 @@
 
 #include "perm_device.cuh"
 #include "perm_kernels.cuh"
+#include "perm_parts.h"
 
 namespace perm {
 
@@ -311,6 +312,15 @@ __device__ __forceinline__ void red_count(unsigned long long *p, long long v, bo
     asm volatile("{\n.reg .pred q;\nsetp.ne.s32 q, %2, 0;\n@q red.relaxed.gpu.global.add.u64 [%0], %1;\n}"
                  :: "l"(p), "l"(v), "r"((int)take) : "memory");
 }
+
+// A tour-sum row as its parts' ends see it (end_part).
+struct PartsRow {
+    unsigned int *tmaxn, *outst;
+    __device__ __forceinline__ void deepen(unsigned n) { atomicMax(tmaxn, n); }
+    __device__ __forceinline__ unsigned leave() { return atomicSub(outst, 1u); }
+    __device__ __forceinline__ unsigned depth() { return *(volatile unsigned int *)tmaxn; }
+    __device__ __forceinline__ void fence() { __threadfence(); }
+};
 
 // The whole warp copies a donor's sites 0..bdp (key and hash slot) into a cell.
 template <typename Key>
@@ -780,20 +790,19 @@ __device__ __forceinline__ void grow_run(const RunDev &P, unsigned char *smem, c
                 // the warp's own order only), and the last part to end flushes the row
                 __threadfence();
                 __syncwarp();
-                unsigned om = 0u, left = 0u;
+                unsigned depth = 0u;
+                bool ends = false;
                 if (fl && !whole && first) {
-                    om = atomicMax(P.tmaxn + own, (unsigned)maxn);
-                    __threadfence();
-                    left = atomicSub(P.outst + own, 1u);
-                    __threadfence();
+                    PartsRow row{P.tmaxn + own, P.outst + own};
+                    ends = end_part(row, (unsigned)maxn, depth);
                 }
                 __syncwarp();
-                om = __shfl_sync(kFull, om, lead);
-                left = __shfl_sync(kFull, left, lead);
+                depth = __shfl_sync(kFull, depth, lead);
+                ends = __shfl_sync(kFull, (int)ends, lead) != 0;
                 bool other_row = false;
                 if (fl && !whole) {
-                    last = left == 1u;
-                    row_max = (int)(om > (unsigned)maxn ? om : (unsigned)maxn);
+                    last = ends;
+                    row_max = (int)depth;
                     // the row stays with the parts still growing: the next tour takes the
                     // walk's other row, if that one is free
                     other_row = !last && did == 0u;

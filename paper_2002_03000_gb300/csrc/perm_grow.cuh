@@ -1116,9 +1116,9 @@ __device__ __forceinline__ void grow_run(const RunDev &P, unsigned char *smem, c
         {
             __syncwarp();                       // the walks' hashes as the last iteration left them
             const bool isn = state == kNode, grows_on = isn && n < P.n_max;
-            // the sum of the weights recorded at this length before the node (a load of the
-            // whole warp right after the barrier: one instruction, so the lanes of a group read
-            // the same value while the refresher writes)
+            // the sum of the weights recorded at this length before the node (snapshot form: the
+            // refresher may write it meanwhile, so the group takes what its first lane has read,
+            // below)
             double Wsum = 0.0;
             longlong2 cut_n = make_longlong2(0, 0);
             if (cutoffs) cut_n = __ldg(cuts.cut + n);
@@ -1136,6 +1136,8 @@ __device__ __forceinline__ void grow_run(const RunDev &P, unsigned char *smem, c
             bool hit, full;
             int place;
             look_bucket(hash, bucket, nkey, hit, full, place);
+            // (two lanes with different sums could decide differently and part for good)
+            if (snapshot && !cutoffs) Wsum = __shfl_sync(kFull, Wsum, lead);
             // the node's weight goes into the tables with reductions that return nothing, one
             // lane each.  Fresh form: a row of the walk's own takes a load (of the whole group)
             // and a store (of its first lane) through L1; on a shared one the add returns the

@@ -68,6 +68,7 @@ struct perm_run_s {
     long long seq_target = 0;      // Alg. 1 tours per sequence (cumulative)
     long long device_bytes = 0;
     int last_status = PERM_OK;
+    bool unread = false;           // launches queued since their status was last read
 };
 
 namespace {
@@ -585,6 +586,7 @@ int perm_run(perm_handle h, int64_t tours_per_seq) {
         e = cudaMemsetAsync(h->tickets, 0, sizeof(unsigned long long), h->stream);
         if (e != cudaSuccess) return to_code(e);
     }
+    h->unread = true;
     const RunDev P = make_params(h);
     e = perm::launch_grow(P, h->thresh, h->key64, h->ctas, h->stream);
     if (e != cudaSuccess) return to_code(e);
@@ -603,13 +605,19 @@ static cudaError_t copy_out(perm_handle h, void *dst, const void *src, size_t by
     return e;
 }
 
+// The status of everything queued so far, as it came back.
+static void took_status(perm_handle h, int st) {
+    h->last_status = st;
+    h->unread = false;
+}
+
 // Wait for the stream; the run's status (one copy: it orders after the run and reports
 // its failure).
 static int sync_status(perm_handle h) {
     int st = 0;
     const cudaError_t e = copy_out(h, &st, h->status, sizeof(int));
     if (e != cudaSuccess) return to_code(e);
-    h->last_status = st;
+    took_status(h, st);
     return st;
 }
 
@@ -633,7 +641,7 @@ int perm_tables(perm_handle h, double *W_n, double *S_n, double *Q_n, int64_t *M
         e = copy_out(h, buf.data(), from, upto);
         if (e != cudaSuccess) return to_code(e);
         std::memcpy(&st, buf.data() + kStatus * kLine, sizeof(int));
-        h->last_status = st;
+        took_status(h, st);
         if (st < 0 && st != PERM_EOVERFLOW && st != PERM_ETIMEOUT) return st;
         if (W_n) std::memcpy(W_n, buf.data() + o_W, cnt * 8);
         if (Q_n) std::memcpy(Q_n, buf.data() + o_Q, cnt * 8);
@@ -672,14 +680,15 @@ int perm_reset(perm_handle h) {
     if (!h) return PERM_EINVAL;
     const size_t L = (size_t)h->cfg.n_max + 1;
     cudaError_t e = cudaMemsetAsync(h->block, 0, h->zero_bytes, h->stream);
-    if (e == cudaSuccess && h->last_status != PERM_OK)   // a stopped run may leave tour sums behind
+    // a stopped run may leave tour sums behind, and one that is not known to have completed
+    if (e == cudaSuccess && (h->last_status != PERM_OK || h->unread))
         e = cudaMemsetAsync(h->X, 0, L * (size_t)h->xrows * sizeof(double), h->stream);
     if (e == cudaSuccess && h->share)
         e = cudaMemsetAsync(h->outst, 0xFF, sizeof(unsigned int) * h->xrows, h->stream);
     if (e != cudaSuccess) return to_code(e);
     h->tour_limit = 0;
     h->seq_target = 0;
-    h->last_status = PERM_OK;
+    took_status(h, PERM_OK);
     return PERM_OK;
 }
 
@@ -784,7 +793,7 @@ int perm_stats(perm_handle h, perm_stats_t *out) {
     if (e != cudaSuccess) return to_code(e);
     int st = 0;
     std::memcpy(&st, buf + kStatus * kLine, sizeof(int));
-    h->last_status = st;
+    took_status(h, st);
     if (st < 0 && st != PERM_EOVERFLOW && st != PERM_ETIMEOUT) return st;
     auto value = [&](int i) {
         unsigned long long v;

@@ -49,3 +49,20 @@ def test_shared_tours_leave_no_sums_behind(d, n_max, N):
             run.reset()
             _same(_grow_chains(run, n_max, 3), t)
             run.reset()
+
+
+def test_a_reset_clears_a_failed_run_that_nobody_asked_about():
+    """A queued run that stops at its time bound, a reset with no query between, and the
+    next run starts from zero tour sums all the same."""
+    torch_cuda()
+    d, n_max, N = 3, 60, 400
+    t = _chains(d, n_max, N, 31, 3)
+    # 400 x 4000 tours of some 60 nodes, 9.6e7 nodes: tens of ms, against a bound of 5 ms
+    with Run(d, n_max, N, 31, max_seconds=0.005) as run:
+        for _ in range(2):
+            run.set_cutoffs(None, None)
+            run.run(4000, sync=False)
+            run.reset()
+            _same(_grow_chains(run, n_max, 3), t)
+            assert run.stats()["status"] == 0
+            run.reset()

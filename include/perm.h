@@ -74,9 +74,10 @@ typedef struct {
     double max_seconds;/* wall-clock bound of one launch; past it the kernel stops and the
                           run reports PERM_ETIMEOUT; 0 = default (600) */
     int ramp_c0;       /* Algorithm 2 admission: at most ramp_c0 + ramp_gamma * (finished
-                          tours) tours are in flight.  0 = default (2; no limit
-                          while cut-offs replace flatPERM's ratio: they read no table);
-                          < 0 = no limit */
+                          tours) tours are in flight.  0 = default (2); < 0 = no limit.
+                          With both at 0 there is no limit while cut-offs replace
+                          flatPERM's ratio (they read no table); a limit given here
+                          holds for them too, also one that equals the default */
     double ramp_gamma; /* see ramp_c0; 0 = default (0.25) */
     int max_ctas;      /* at most this many CTAs (SMs) for the run's walks; 0 = all SMs;
                           -1 = as few CTAs as hold one walk per sequence (dense packing).

@@ -67,6 +67,7 @@ struct perm_run_s {
     long long tour_limit = 0;      // Alg. 2 tickets handed out so far (cumulative)
     long long seq_target = 0;      // Alg. 1 tours per sequence (cumulative)
     long long device_bytes = 0;
+    bool own_limit = false;        // the caller gave an admission limit (ramp_c0 or ramp_gamma)
     int last_status = PERM_OK;
     bool unread = false;           // launches queued since their status was last read
 };
@@ -239,6 +240,7 @@ int create_impl(perm_handle *out, const perm_config *cfg, const ForcedLayout *fo
     if (h->cfg.refresh_ns == 0) h->cfg.refresh_ns = 8000;
     if (h->cfg.refresh_ns > 1000000) h->cfg.refresh_ns = 1000000;
     if (h->cfg.max_seconds == 0.0) h->cfg.max_seconds = 600.0;
+    h->own_limit = cfg->ramp_c0 != 0 || cfg->ramp_gamma != 0.0;
     if (h->cfg.ramp_c0 == 0) h->cfg.ramp_c0 = kRampC0;
     if (h->cfg.ramp_gamma == 0.0) h->cfg.ramp_gamma = kRampGamma;
     h->device = dev;
@@ -520,10 +522,10 @@ static RunDev make_params(perm_handle h) {
     P.exact_steps = h->exact_steps;
     P.finished = h->finished;
     P.admit = h->admit;
-    // cut-offs read no table, so tours need not wait for samples of others: with the default
-    // limit they all start at once (cubic chains, n_max 10000, 608 sequences, 4 tours each, from
+    // cut-offs read no table, so tours need not wait for samples of others: unless the caller
+    // gave a limit they all start at once (cubic chains, n_max 10000, 608 sequences, 4 tours each, from
     // an empty run: 97.8 -> 26.1 ms; square, n = 257, 2000 sequences, 8 tours: 10.8 -> 9.2)
-    const bool no_limit = h->cut != nullptr && h->cfg.ramp_c0 == kRampC0 && h->cfg.ramp_gamma == kRampGamma;
+    const bool no_limit = h->cut != nullptr && !h->own_limit;
     P.ramp_c0 = h->cfg.ramp_c0 < 0 || no_limit ? -1 : (long long)h->cfg.ramp_c0;
     P.ramp_gamma_q16 = (unsigned long long)(h->cfg.ramp_gamma * 65536.0);
     P.share = h->share ? h->share_cap : 0;
@@ -945,7 +947,7 @@ struct CkptHeader {
     char magic[8];
     uint32_t version;
     uint32_t header_bytes;
-    perm_config cfg;               // as the handle holds it (defaults filled in)
+    perm_config cfg;               // as the handle holds it (defaults filled in, but for the admission limit)
     int64_t tour_limit, seq_target;
     int32_t ntab, has_rn, has_cut, cut_copies;
     double cut_q;
@@ -976,6 +978,7 @@ int perm_save(perm_handle h, const char *path) {
     hd.version = kCkptVersion;
     hd.header_bytes = (uint32_t)sizeof(CkptHeader);
     hd.cfg = h->cfg;
+    if (!h->own_limit) { hd.cfg.ramp_c0 = 0; hd.cfg.ramp_gamma = 0.0; }    // the default again when loaded
     hd.tour_limit = h->tour_limit;
     hd.seq_target = h->seq_target;
     hd.ntab = h->ntab;

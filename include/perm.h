@@ -290,12 +290,19 @@ const char *perm_strerror(int code);
  * force_exact = 1 takes every decision on r in double precision (0: the
  * kernel's own path).  Outcomes: 0 walk at n_max, 1 trapped, 2 pruned,
  * 3 children.  Requires d in {2,3} and n_max <= 512.  Queued on `stream`,
- * not waited for. */
+ * not waited for.  This is the step with fresh thresholds;
+ * perm_debug_step_snapshot is the step with snapshot thresholds (the same
+ * decisions; r and a survivor's weight are formed in other operations). */
 int perm_debug_step(int d, int n_max, int B, const int32_t *coords, const int32_t *len,
                     const double *W, const double *Wsum, const uint64_t *M,
                     const uint64_t *ordinal, const uint32_t *seq, const uint32_t *tour,
                     uint64_t seed, uint32_t run_id, int force_exact, int32_t *out_i,
                     double *out_r, double *out_w, void *stream);
+int perm_debug_step_snapshot(int d, int n_max, int B, const int32_t *coords, const int32_t *len,
+                             const double *W, const double *Wsum, const uint64_t *M,
+                             const uint64_t *ordinal, const uint32_t *seq, const uint32_t *tour,
+                             uint64_t seed, uint32_t run_id, int force_exact, int32_t *out_i,
+                             double *out_r, double *out_w, void *stream);
 
 /* ---------------------------------------------------------------------------
  * Batched runs (many independent runs, one CUDA-graph launch).

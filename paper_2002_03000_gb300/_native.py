@@ -32,7 +32,8 @@ PERM_THRESH_FRESH = 1
 EXPORTS = (
     "perm_config_init", "perm_create", "perm_create_ex", "perm_set_stream", "perm_run", "perm_reset",
     "perm_run_sync", "perm_estimates", "perm_tables", "perm_stats", "perm_trace_enable",
-    "perm_trace_read", "perm_destroy", "perm_strerror", "perm_debug_step", "perm_debug_philox",
+    "perm_trace_read", "perm_destroy", "perm_strerror", "perm_debug_step", "perm_debug_step_snapshot",
+    "perm_debug_philox",
     "perm_run_static", "perm_set_cutoffs", "perm_save", "perm_load", "perm_get_config", "perm_batch_create", "perm_batch_create_persistent", "perm_batch_run", "perm_batch_size",
     "perm_batch_estimates", "perm_batch_stats", "perm_batch_destroy", "perm_autotune",
     "perm_observable_r2", "perm_estimates_from_tables", "perm_batch_continue",
@@ -111,7 +112,8 @@ def load(path: str = LIB_PATH):
     L.perm_destroy.restype = None
     L.perm_strerror.argtypes = [C.c_int]
     L.perm_strerror.restype = C.c_char_p
-    L.perm_debug_step.argtypes = [C.c_int, C.c_int, C.c_int] + [vp] * 8 + [u64, u32, C.c_int] + [vp] * 3 + [vp]
+    for f in (L.perm_debug_step, L.perm_debug_step_snapshot):
+        f.argtypes = [C.c_int, C.c_int, C.c_int] + [vp] * 8 + [u64, u32, C.c_int] + [vp] * 3 + [vp]
     L.perm_debug_philox.argtypes = [C.c_int, vp, C.POINTER(u32), vp]
     L.perm_run_static.argtypes = [C.POINTER(perm_config), i64, vp, vp, vp, C.POINTER(i64), vp]
     L.perm_batch_create.argtypes = [hp, C.POINTER(perm_config), C.POINTER(i64), C.c_int, C.c_int]
@@ -262,6 +264,14 @@ def perm_debug_step(d, n_max, B, coords, length, W, Wsum, M, ordinal, seq, tour,
     _check(load().perm_debug_step(d, n_max, B, coords, length, W, Wsum, M, ordinal, seq, tour,
                                   seed, run_id, force_exact, out_i, out_r, out_w, stream),
            "perm_debug_step")
+
+
+def perm_debug_step_snapshot(d, n_max, B, coords, length, W, Wsum, M, ordinal, seq, tour, seed, run_id,
+                             force_exact, out_i, out_r, out_w, stream=0):
+    """perm_debug_step as the snapshot form decides."""
+    _check(load().perm_debug_step_snapshot(d, n_max, B, coords, length, W, Wsum, M, ordinal, seq, tour,
+                                           seed, run_id, force_exact, out_i, out_r, out_w, stream),
+           "perm_debug_step_snapshot")
 
 
 def perm_run_static(cfg, tours_per_seq, W_dev, S_dev, Q_dev, stream=0):

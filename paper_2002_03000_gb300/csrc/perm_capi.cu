@@ -868,20 +868,38 @@ void perm_destroy(perm_handle h) {
     delete h;
 }
 
-int perm_debug_step(int d, int n_max, int B, const int32_t *coords, const int32_t *len,
-                    const double *W, const double *Wsum, const uint64_t *M,
-                    const uint64_t *ordinal, const uint32_t *seq, const uint32_t *tour,
-                    uint64_t seed, uint32_t run_id, int force_exact, int32_t *out_i,
-                    double *out_r, double *out_w, void *stream) {
+static int debug_step(int d, int n_max, int B, const int32_t *coords, const int32_t *len,
+                      const double *W, const double *Wsum, const uint64_t *M,
+                      const uint64_t *ordinal, const uint32_t *seq, const uint32_t *tour,
+                      uint64_t seed, uint32_t run_id, bool snapshot, int force_exact, int32_t *out_i,
+                      double *out_r, double *out_w, void *stream) {
     if ((d != 2 && d != 3) || n_max < 1 || n_max > 512 || B < 0) return PERM_EINVAL;
     if (force_exact != 0 && force_exact != 1) return PERM_EINVAL;
     if (B > 0 && (!coords || !len || !W || !Wsum || !M || !ordinal || !seq || !tour || !out_i ||
                   !out_r || !out_w))
         return PERM_EINVAL;
     cudaError_t e = perm::launch_debug_step(d, n_max, B, coords, len, W, Wsum, M, ordinal, seq, tour,
-                                            (uint32_t)seed ^ run_id, (uint32_t)(seed >> 32), force_exact,
+                                            (uint32_t)seed ^ run_id, (uint32_t)(seed >> 32), snapshot, force_exact,
                                             out_i, out_r, out_w, (cudaStream_t)stream);
     return to_code(e);
+}
+
+int perm_debug_step(int d, int n_max, int B, const int32_t *coords, const int32_t *len,
+                    const double *W, const double *Wsum, const uint64_t *M,
+                    const uint64_t *ordinal, const uint32_t *seq, const uint32_t *tour,
+                    uint64_t seed, uint32_t run_id, int force_exact, int32_t *out_i,
+                    double *out_r, double *out_w, void *stream) {
+    return debug_step(d, n_max, B, coords, len, W, Wsum, M, ordinal, seq, tour, seed, run_id, false, force_exact,
+                      out_i, out_r, out_w, stream);
+}
+
+int perm_debug_step_snapshot(int d, int n_max, int B, const int32_t *coords, const int32_t *len,
+                             const double *W, const double *Wsum, const uint64_t *M,
+                             const uint64_t *ordinal, const uint32_t *seq, const uint32_t *tour,
+                             uint64_t seed, uint32_t run_id, int force_exact, int32_t *out_i,
+                             double *out_r, double *out_w, void *stream) {
+    return debug_step(d, n_max, B, coords, len, W, Wsum, M, ordinal, seq, tour, seed, run_id, true, force_exact,
+                      out_i, out_r, out_w, stream);
 }
 
 int perm_debug_philox(int B, const uint32_t *ctr, const uint32_t *key, uint32_t *out) {

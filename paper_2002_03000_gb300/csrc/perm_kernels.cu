@@ -207,9 +207,10 @@ __global__ void batch_init_kernel(const BatchDev B) {
 
 // ---------------------------------------------------------------------------
 // Growth step on caller-given snapshot states (one group of lanes per state, one
-// warp per block, as the persistent kernel's node).
+// warp per block, as the persistent kernel's node).  REFINE: the fresh form's decision,
+// else the snapshot form's.
 // ---------------------------------------------------------------------------
-template <int D, typename Key>
+template <int D, typename Key, bool REFINE>
 __global__ void __launch_bounds__(32) debug_step_kernel(int n_max, int log2h, int B,
         const int32_t *coords, const int32_t *len, const double *Wv, const double *Wsv,
         const uint64_t *Mv, const uint64_t *ordv, const uint32_t *seqv, const uint32_t *tourv,
@@ -262,7 +263,7 @@ __global__ void __launch_bounds__(32) debug_step_kernel(int n_max, int log2h, in
     set_tours<true>(t, M);
     const double sum = __dadd_rn(Wsum, W);
     const Decision o = decide_node<D>(good ? n : 0, a > 0 ? a : 1, W, sum, guess(W, Wsum, t.Mf, w.x), t,
-                                      true, w.x, aoc, decides, decides && force_exact != 0);
+                                      REFINE, w.x, aoc, decides, decides && force_exact != 0);
     if (!good || j != 0) return;
     const int c = decides ? o.c : 0;
     uint32_t dirs = lists[fm], xw = w.y;
@@ -408,31 +409,34 @@ cudaError_t launch_finalize(const RunDev &P, cudaStream_t stream) {
     return cudaGetLastError();
 }
 
+template <int D, bool REFINE>
+static cudaError_t debug_step_form(int n_max, int B, const int32_t *coords, const int32_t *len, const double *W,
+                                   const double *Wsum, const uint64_t *M, const uint64_t *ordinal,
+                                   const uint32_t *seq, const uint32_t *tour, uint32_t key0, uint32_t key1,
+                                   int force_exact, int32_t *out_i, double *out_r, double *out_w, cudaStream_t stream) {
+    int log2h = 4;
+    while ((1 << log2h) < 2 * n_max) ++log2h;
+    const int per = walks_per_warp_max(D);               // states per block of one warp
+    const int blocks = (B + per - 1) / per;
+    const size_t smem = 1024 + walk_hash_bytes(log2h, 4) * (size_t)per;
+    const cudaError_t e = cudaFuncSetAttribute(debug_step_kernel<D, uint32_t, REFINE>,
+                                               cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    debug_step_kernel<D, uint32_t, REFINE><<<blocks, 32, smem, stream>>>(n_max, log2h, B, coords, len, W, Wsum,
+            M, ordinal, seq, tour, key0, key1, force_exact, out_i, out_r, out_w);
+    return cudaGetLastError();
+}
+
 cudaError_t launch_debug_step(int d, int n_max, int B, const int32_t *coords, const int32_t *len,
                               const double *W, const double *Wsum, const uint64_t *M,
                               const uint64_t *ordinal, const uint32_t *seq, const uint32_t *tour,
-                              uint32_t key0, uint32_t key1, int force_exact, int32_t *out_i,
+                              uint32_t key0, uint32_t key1, bool snapshot, int force_exact, int32_t *out_i,
                               double *out_r, double *out_w, cudaStream_t stream) {
-    int log2h = 4;
-    while ((1 << log2h) < 2 * n_max) ++log2h;
     if (B <= 0) return cudaSuccess;
-    const int per = walks_per_warp_max(d);               // states per block of one warp
-    const int blocks = (B + per - 1) / per;
-    const size_t smem = 1024 + walk_hash_bytes(log2h, 4) * (size_t)per;
-    if (d == 2) {
-        cudaError_t e = cudaFuncSetAttribute(debug_step_kernel<2, uint32_t>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        debug_step_kernel<2, uint32_t><<<blocks, 32, smem, stream>>>(n_max, log2h, B, coords, len, W, Wsum,
-                M, ordinal, seq, tour, key0, key1, force_exact, out_i, out_r, out_w);
-    } else {
-        cudaError_t e = cudaFuncSetAttribute(debug_step_kernel<3, uint32_t>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        debug_step_kernel<3, uint32_t><<<blocks, 32, smem, stream>>>(n_max, log2h, B, coords, len, W, Wsum,
-                M, ordinal, seq, tour, key0, key1, force_exact, out_i, out_r, out_w);
-    }
-    return cudaGetLastError();
+    const auto form = d == 2 ? (snapshot ? debug_step_form<2, false> : debug_step_form<2, true>)
+                             : (snapshot ? debug_step_form<3, false> : debug_step_form<3, true>);
+    return form(n_max, B, coords, len, W, Wsum, M, ordinal, seq, tour, key0, key1, force_exact, out_i, out_r,
+                out_w, stream);
 }
 
 cudaError_t launch_debug_philox(int B, const uint32_t *ctr, uint32_t k0, uint32_t k1, uint32_t *out,

@@ -163,7 +163,7 @@ cudaError_t set_smem_limits();
 cudaError_t launch_debug_step(int d, int n_max, int B, const int32_t *coords, const int32_t *len,
                               const double *W, const double *Wsum, const uint64_t *M,
                               const uint64_t *ordinal, const uint32_t *seq, const uint32_t *tour,
-                              uint32_t key0, uint32_t key1, int force_exact, int32_t *out_i,
+                              uint32_t key0, uint32_t key1, bool snapshot, int force_exact, int32_t *out_i,
                               double *out_r, double *out_w, cudaStream_t stream);
 cudaError_t launch_debug_philox(int B, const uint32_t *ctr, uint32_t k0, uint32_t k1, uint32_t *out,
                                 cudaStream_t stream);

@@ -229,17 +229,23 @@ __device__ __noinline__ Decision decide_node_exact(int a, double W, double sum, 
     return decide_on_average(a, W, __ddiv_rn(sum, __ull2double_rn(M)), w0, a_sc);
 }
 
+// A survivor's weight where M is its tour's own number: the quotient by M correctly rounded.
+__device__ __noinline__ double divided_survivor(double sum, unsigned long long M, double a_sc) {
+    return __dmul_rn(__ddiv_rn(sum, __ull2double_rn(M)), a_sc);
+}
+
 // The decision at a node with a >= 1 free neighbours (Sec. 2): r, the copies, the
 // children's weight.  sum: the weights recorded at length n up to this node, gs: what
 // the estimate of r says; refine: round the survivor's quotient by M correctly (one more step of the
-// division).  valid: the lane has a node to decide (the others' results are not used);
+// division); divide: the snapshot form's M is not the snapshot's, and a survivor's quotient is
+// divided out (a tour's first nodes, until the snapshot counts it).  valid: the lane has a node to decide (the others' results are not used);
 // force_exact: decide on the double-precision r.  Shared by the persistent kernel
 // and the snapshot-state kernel; every lane of a walk's group takes the same decision.
 // One straight line with selects but for the exact path: a branch costs a lone warp
 // 25 cycles or more, a double-precision instruction 64 whatever its active lanes.
 template <int D>
 __device__ __forceinline__ Decision decide_node(int n, int a, double W, double sum, const Guess &gs, const Tours &t,
-                                                bool refine, uint32_t w0, const double *aoc, bool valid, bool force_exact) {
+                                                bool refine, bool divide, uint32_t w0, const double *aoc, bool valid, bool force_exact) {
     Decision o;
     o.exact = false;
     o.x = gs.x;
@@ -253,7 +259,9 @@ __device__ __forceinline__ Decision decide_node(int n, int a, double W, double s
     // (W/c) a_+ 2^-dE: one double-precision product for both, on the critical path
     // alone.  The survivor's factor (1/M) a_+ 2^-dE (a node past the empty walk has
     // a_+ <= 5) is one of three products kept per M, its exponent shifted (exact: 1/M
-    // is far from the subnormals); the weight is within 2^-51 of the quotient
+    // is far from the subnormals); the weight is within 2^-51 of the quotient.  That holds for the
+    // snapshot's M; with the tour's own number the quotient is divided out below, beside the exact
+    // path (in one branch with it: square n = 512 continued 50.8 -> 51.0 ms, cubic 120 -> 121)
     double base = W, fac = row[c];
     if (refine) {
         // (under a branch: three dependent operations of 62 cycles, which ran no faster beside
@@ -275,8 +283,9 @@ __device__ __forceinline__ Decision decide_node(int n, int a, double W, double s
     // the estimate cannot settle a comparison: r exactly as defined
     if (exact && refine) {
         o = decide_on_average(a, W, average(sum, t), w0, row[0]);
-    } else if (exact) {
-        o = decide_node_exact(a, W, sum, t.M, w0, row[0]);
+    } else if (!refine && (exact || (valid && surv && divide))) {
+        if (exact) o = decide_node_exact(a, W, sum, t.M, w0, row[0]);
+        else o.child_w = divided_survivor(sum, t.M, row[0]);
     }
     return o;
 }
@@ -1205,7 +1214,7 @@ __device__ __forceinline__ void grow_run(const RunDev &P, unsigned char *smem, c
             const int cslot = __shfl_sync(kFull, nslot, lead + dir0);
             Decision o;
             if (cutoffs) o = decide_cutoffs<D>(n, a1, W, cut_n, w0, aoc, cuts);
-            else o = decide_node<D>(n, a1, W, sum, gs, tours, !snapshot, w0, aoc, decides, false);
+            else o = decide_node<D>(n, a1, W, sum, gs, tours, !snapshot, snapshot && (uint32_t)tours.M != ms_low, w0, aoc, decides, false);
             const int c = decides ? o.c : 0;
             if (o.exact && decides) my_exact += 1ull;
             const bool extend = c > 0, leaf = isn && c == 0;

@@ -263,7 +263,7 @@ __global__ void __launch_bounds__(32) debug_step_kernel(int n_max, int log2h, in
     set_tours<true>(t, M);
     const double sum = __dadd_rn(Wsum, W);
     const Decision o = decide_node<D>(good ? n : 0, a > 0 ? a : 1, W, sum, guess(W, Wsum, t.Mf, w.x), t,
-                                      REFINE, w.x, aoc, decides, decides && force_exact != 0);
+                                      REFINE, false, w.x, aoc, decides, decides && force_exact != 0);
     if (!good || j != 0) return;
     const int c = decides ? o.c : 0;
     uint32_t dirs = lists[fm], xw = w.y;

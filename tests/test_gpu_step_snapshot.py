@@ -36,3 +36,27 @@ def test_decision_boundaries(d, force_exact):
 @pytest.mark.parametrize("d", [2, 3])
 def test_edge_cases(d):
     fresh.test_step_parity_edge_cases(d)
+
+
+@pytest.mark.parametrize("d,n_max", [(2, 30), (3, 24)])
+def test_a_survivor_on_its_own_tour_number_is_divided_out(d, n_max):
+    """Until a snapshot counts a tour, its nodes take the tour's own number for M, and a
+    survivor's weight is the quotient (Wsum + W)/M, correctly rounded, times a_+ 2^-dE.
+    Only the tour started last before a refresh has a number that is also a snapshot's
+    (its survivors may take the product with 1/M): one of those that 64 walks start from
+    one refresh, a quarter of a millisecond or more, to the next, 64 or more."""
+    from oracle import oracle as orc
+    gpu_util.torch_cuda()
+    N = 64
+    with gpu_util.Run(d, n_max, N, 77, refresh_ns=1000000, share_copies=-1) as run:
+        run.trace_enable(1, 1, 40000)
+        run.run(200)
+        assert run.stats()["status"] == 0
+        _, recs, _ = run.trace_read()
+    own = [r for r in recs if r.c == 1 and r.n > 0 and r.r < 1.0 and not r.exact and r.M == r.tour * N + r.seq + 1]
+    assert len(own) > 500
+    same = 0
+    for r in own:
+        dE = orc.scale_exp(d, r.n + 1) - orc.scale_exp(d, r.n)
+        same += r.child_w == (r.Wsum + r.W) / float(r.M) * (r.a_plus * 2.0 ** -dE)
+    assert same >= 0.98 * len(own), (same, len(own))

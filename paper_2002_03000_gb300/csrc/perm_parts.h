@@ -1,5 +1,5 @@
-// perm_parts.h -- how the parts of one tour end (shared copies).  Plain C++, so that the
-// order of the steps can be checked on the host.
+// perm_parts.h -- how tours are handed out, and how the parts of one tour end (shared
+// copies).  Plain C++, so that both can be checked on the host.
 #pragma once
 
 #ifdef __CUDACC__
@@ -26,6 +26,15 @@ PERM_HD bool end_part(Row &row, unsigned maxn, unsigned &depth) {
     if (parts != 1u) return false;
     depth = row.depth();
     return true;
+}
+
+// Tour tickets that a warp fetches beyond those its walks need now, at most `most`: a warp
+// keeps what it has fetched, so no more than half of a walk's even share of the tours
+// that the launch has left to start.
+PERM_HD unsigned tickets_ahead(long long left, long long walks, unsigned most) {
+    if (left >= 2 * walks * (long long)(most + 1u)) return most;
+    const long long half = left / (2 * walks);
+    return half > 1 ? (unsigned)(half - 1) : 0u;
 }
 
 }  // namespace perm

@@ -284,28 +284,6 @@ int create_impl(perm_handle *out, const perm_config *cfg, const ForcedLayout *fo
         if (arena_mode == perm::kArenaAll) return (size_t)0;
         return head_b + walk_b * (size_t)walks;
     };
-    if (!force && cfg->max_ctas == -1) {
-        // dense packing: the fewest CTAs that hold one walk per sequence, so that runs
-        // sharing the device take few SMs each (24 runs of n = 64..256 on streams: 33.8 ms at 4
-        // full warps a CTA, 25.4 at 8, 22.6 at 11)
-        long long per_cta = 0;
-        for (int t = max_w * max_l; t >= 1; --t)
-            if (smem_for(t) <= budget) { per_cta = t; break; }
-        if (per_cta > 0) {
-            const long long need = ((long long)n_seq + per_cta - 1) / per_cta;
-            h->num_sms = (int)std::max(1LL, std::min((long long)h->num_sms, need));
-        }
-    }
-    long long tslots = cfg->slots ? cfg->slots : (long long)n_seq;   // walks that grow tours
-    if (tslots > n_seq) tslots = n_seq;
-    // and helper walks: as asked (none by default), or (-1) the walks the automatic
-    // layout has room for beyond the tour walks (4 warps of 8 per SM), when shared
-    // copies are on
-    const bool can_help = cfg->share_copies >= 0 && cfg->alg == PERM_ALG2 &&
-                          cfg->threshold == PERM_THRESH_SNAPSHOT && !force;
-    long long helpers = cfg->helper_walks;
-    if (helpers < 0) helpers = can_help && !lpw ? std::max(0LL, (long long)h->num_sms * 32 - tslots) : 0;
-    long long slots = tslots + helpers;
     int warps = 0, lanes = 0;
     // walks of a CTA over its warps: over as many of them as there are walks
     auto spread = [&](int t) {
@@ -330,22 +308,11 @@ int create_impl(perm_handle *out, const perm_config *cfg, const ForcedLayout *fo
             if (w * w * l > best) { best = w * w * l; full_l = l; auto_walks = (int)(w * l); }
         }
     }
-    if (force) {
-        // every CTA of the batch grid may join this run: the most walks up to the automatic
-        // layout's bound that fit the shared memory
-        for (int t = std::min(auto_walks, kBatchWalks); t >= 1 && !warps; --t) {
-            spread(t);
-            if (smem_for(warps * lanes) > budget) warps = 0;
-        }
-        slots = (long long)force->ctas * warps * lanes;
-        if (!warps || slots > (1LL << 30)) { cudaStreamDestroy(h->stream); delete h; return PERM_EUNSUPPORTED; }
-        h->num_sms = force->ctas;
-    }
-    if (!force) {
-        // the walks that the SMs share, or the most of them that fit
-        long long t = std::min<long long>((slots + h->num_sms - 1) / h->num_sms,
-                                          lpw ? max_w * std::min(lpw, max_l) : auto_walks);
-        for (; t >= 1 && !warps; --t) {
+    // a CTA's layout for t walks, or for the most below that fit; the walks that it holds (0:
+    // none fits).  most: what the largest CTA is asked for
+    const long long most = lpw ? max_w * std::min(lpw, max_l) : auto_walks;
+    auto lay_out = [&](long long t) {
+        for (warps = 0; t >= 1 && !warps; --t) {
             if (lpw) {
                 lanes = (int)std::min<long long>(t, std::min(lpw, max_l));
                 warps = (int)((t + lanes - 1) / lanes);
@@ -357,7 +324,42 @@ int create_impl(perm_handle *out, const perm_config *cfg, const ForcedLayout *fo
             }
             if (smem_for(warps * lanes) > budget) warps = 0;
         }
+        return warps * lanes;
+    };
+    if (!force && cfg->max_ctas == -1) {
+        // dense packing: the fewest CTAs that hold one walk per sequence, so that runs
+        // sharing the device take few SMs each (24 runs of n = 64..256 on streams: 33.8 ms at 4
+        // full warps a CTA, 25.4 at 8, 22.6 at 11).  A CTA holds what its layout does, which may be
+        // fewer walks than the shared memory
+        const long long per_cta = lay_out(most);
+        if (per_cta > 0) {
+            const long long need = ((long long)n_seq + per_cta - 1) / per_cta;
+            h->num_sms = (int)std::max(1LL, std::min((long long)h->num_sms, need));
+        }
     }
+    long long tslots = cfg->slots ? cfg->slots : (long long)n_seq;   // walks that grow tours
+    if (tslots > n_seq) tslots = n_seq;
+    // and helper walks: as asked (none by default), or (-1) the walks the automatic
+    // layout has room for beyond the tour walks (4 warps of 8 per SM), when shared
+    // copies are on
+    const bool can_help = cfg->share_copies >= 0 && cfg->alg == PERM_ALG2 &&
+                          cfg->threshold == PERM_THRESH_SNAPSHOT && !force;
+    long long helpers = cfg->helper_walks;
+    if (helpers < 0) helpers = can_help && !lpw ? std::max(0LL, (long long)h->num_sms * 32 - tslots) : 0;
+    long long slots = tslots + helpers;
+    if (force) {
+        // every CTA of the batch grid may join this run: the most walks up to the automatic
+        // layout's bound that fit the shared memory
+        for (int t = std::min(auto_walks, kBatchWalks); t >= 1 && !warps; --t) {
+            spread(t);
+            if (smem_for(warps * lanes) > budget) warps = 0;
+        }
+        slots = (long long)force->ctas * warps * lanes;
+        if (!warps || slots > (1LL << 30)) { cudaStreamDestroy(h->stream); delete h; return PERM_EUNSUPPORTED; }
+        h->num_sms = force->ctas;
+    }
+    // the walks that the SMs share, or the most of them that fit
+    if (!force) lay_out(std::min((slots + h->num_sms - 1) / h->num_sms, most));
     if (!warps) { cudaStreamDestroy(h->stream); delete h; return PERM_EUNSUPPORTED; }
     const long long per_cta_eff = (long long)warps * lanes;
     // (sequences beyond the layout wait at tour boundaries)

@@ -346,7 +346,8 @@ int perm_batch_stats(perm_batch_handle b, int r, perm_stats_t *out);
 void perm_batch_destroy(perm_batch_handle b);
 
 /* Autotuner (no counterpart in the paper): for each walks-per-warp choice (auto,
- * 2, 4, 8, 16, 32), hash size (hash_scale 0, 1) and stack ring (16, 64 records),
+ * 2, 4, 8, 16, 32), hash size (hash_scale 0, 1) and stack ring (16, 64 records)
+ * that comes to a layout of its own (a warp holds at most 8 walks, d = 3: 4),
  * times a complete run of probe_tours tours per sequence of cfg from empty
  * tables (twice; the faster counts).  The default layout (auto, 0, 16) is timed
  * first and kept unless another choice is at least 3% faster and then at least

@@ -19,6 +19,7 @@
 #include <map>
 #include <mutex>
 #include <new>
+#include <set>
 #include <tuple>
 #include <vector>
 
@@ -339,7 +340,9 @@ void perm_batch_destroy(perm_batch_handle b) { batch_free(b); }
 
 // ---------------------------------------------------------------------------
 // Autotuner: short calibration runs over walks per warp, hash size and the
-// shared-memory stack ring ("spill tile").  Each trial times a complete run of
+// shared-memory stack ring ("spill tile").  Choices that come to a layout already timed
+// are left out (a warp holds at most 8 walks, 4 on the cubic lattice, and hash_scale 0
+// doubles the hash where it fits: of 23 choices about half repeat another).  Each trial times a complete run of
 // probe_tours tours per sequence from empty tables (twice, the faster counts),
 // so the trials compare equal work, start-up included.  The default layout is
 // timed first and stays unless a choice beats it by 3% and then again on runs
@@ -368,9 +371,12 @@ int perm_autotune(perm_config *cfg, int64_t probe_tours) {
     const int lanes_c[] = {0, 2, 4, 8, 16, 32};
     const int hash_c[] = {0, 1};
     const int ring_c[] = {16, 64};
+    // the layouts timed so far: warps, walks a warp, CTAs, hash slots, ring
+    std::set<std::tuple<int, int, int, int, int>> timed;
     // a complete run of `tours` from empty tables with the layout of `t`, `reps`
-    // times (start-up included: it is part of every run); the fastest counts
-    auto time_layout = [&](const TuneChoice &t, int64_t tours, int reps) {
+    // times (start-up included: it is part of every run); the fastest counts.  once: not if
+    // the layout has been timed
+    auto time_layout = [&](const TuneChoice &t, int64_t tours, int reps, bool once) {
         perm_config c = *cfg;
         c.lanes_per_warp = t.lanes;
         c.hash_scale = t.hash_scale;
@@ -378,7 +384,13 @@ int perm_autotune(perm_config *cfg, int64_t probe_tours) {
         perm_handle h = nullptr;
         if (perm_create_ex(&h, &c) != PERM_OK) return -1.0;
         double sec = -1.0;
-        int rc = PERM_OK;
+        perm_stats_t st;
+        int rc = perm_stats(h, &st);
+        if (rc == PERM_OK && once &&
+            !timed.insert(std::make_tuple(st.warps_per_cta, st.lanes_per_warp, st.ctas, st.hash_slots, t.ring)).second) {
+            perm_destroy(h);
+            return -1.0;
+        }
         for (int rep = 0; rep < reps && rc == PERM_OK; ++rep) {
             rc = perm_reset(h);
             const auto t0 = std::chrono::steady_clock::now();
@@ -391,7 +403,7 @@ int perm_autotune(perm_config *cfg, int64_t probe_tours) {
         return rc == PERM_OK ? sec : -1.0;
     };
     const TuneChoice dflt{0, 0, 16};
-    const double dflt_s = time_layout(dflt, probe_tours, 2);
+    const double dflt_s = time_layout(dflt, probe_tours, 2, true);
     double best_s = dflt_s;
     TuneChoice best = dflt;
     for (int ring : ring_c) {
@@ -399,7 +411,7 @@ int perm_autotune(perm_config *cfg, int64_t probe_tours) {
             for (int lw : lanes_c) {
                 const TuneChoice t{lw, hs, ring};
                 if (lw == 0 && hs == 0 && ring == 16) continue;
-                const double sec = time_layout(t, probe_tours, 2);
+                const double sec = time_layout(t, probe_tours, 2, true);
                 // a choice other than the default has to beat it by 3% (the spread
                 // of repeated complete runs), else the default stays
                 if (sec >= 0.0 && (best_s < 0.0 || sec < best_s * (best.lanes == 0 && best.hash_scale == 0 &&
@@ -417,7 +429,8 @@ int perm_autotune(perm_config *cfg, int64_t probe_tours) {
     if (best_s >= 0.0 && !(best.lanes == 0 && best.hash_scale == 0 && best.ring == 16)) {
         double b4 = -1.0, d4 = -1.0;
         for (int k = 0; k < 3; ++k) {
-            const double b = time_layout(best, 4 * probe_tours, 1), d = time_layout(dflt, 4 * probe_tours, 1);
+            const double b = time_layout(best, 4 * probe_tours, 1, false),
+                         d = time_layout(dflt, 4 * probe_tours, 1, false);
             if (b >= 0.0 && (b4 < 0.0 || b < b4)) b4 = b;
             if (d >= 0.0 && (d4 < 0.0 || d < d4)) d4 = d;
         }

@@ -41,7 +41,7 @@ def bytes_per_step(d, f):
     return base + 32.0 * f
 
 
-KERNEL_SOURCES = ("perm_grow.cuh", "perm_kernels.cu", "perm_kernels.cuh", "perm_device.cuh")
+KERNEL_SOURCES = ("perm_grow.cuh", "perm_kernels.cu", "perm_kernels.cuh", "perm_device.cuh", "perm_parts.h")
 
 
 def code_tokens(text):
@@ -563,8 +563,8 @@ LOG_C10000_PAPER = 9704.14   # Sec. 4, eq. 8: log c_10000 on the square lattice 
 
 def long_walks(cap_s=60.0):
     """Sec. 4's long walks with Table 2's setup: square lattice, n_max = 10^4, 12
-    interacting sequences (Algorithm 2, snapshot thresholds, walks in the global
-    arena), from empty tables, one tour of every sequence per launch until
+    interacting sequences (Algorithm 2, snapshot thresholds; the walks' state in shared
+    memory where it fits, else in the global arena), from empty tables, one tour of every sequence per launch until
     `cap_s` seconds (each launch bounded by that too).  Reports what is reached:
     tours finished, growth steps, the longest length sampled, and log c_10000 with
     its standard error against the paper's 9704.14 once n = 10^4 is sampled."""

@@ -114,7 +114,7 @@ typedef struct {
                           flight whatever their number.  k > 0 needs Algorithm 2 with
                           snapshot thresholds and shared copies on; 0 (default) =
                           none; -1 = the walks the automatic layout has room for
-                          beyond the tour walks (up to 4 warps of 8 per SM) when
+                          beyond the tour walks, up to 32 walks per SM in all, when
                           shared copies are on, else none.  Fewer run when not all
                           fit.  They pay off for long walks from few sequences
                           (n_max 10^4 from 12); with many sequences or short walks
@@ -318,8 +318,8 @@ int perm_debug_step_snapshot(int d, int n_max, int B, const int32_t *coords, con
  * per sequence of it, and moves to another run once the run has no tours left to
  * start; with no run left to start, CTAs help unfinished runs through their
  * waiting copies.  Every run must be Alg. 2 with snapshot thresholds
- * (PERM_EUNSUPPORTED otherwise); each is laid out for the whole grid (at most
- * 4 x 8 walks per CTA), so its per-walk scratch scales with the SM count; its
+ * (PERM_EUNSUPPORTED otherwise); each is laid out for the whole grid (up to
+ * 50 walks per CTA), so its per-walk scratch scales with the SM count; its
  * lanes_per_warp, slots and max_ctas are ignored.  The statistics and estimates
  * follow the same law as a single run's (the scheduling differs, so results are
  * not bit-identical to one).  The launch ends within the largest max_seconds
@@ -346,9 +346,9 @@ int perm_batch_stats(perm_batch_handle b, int r, perm_stats_t *out);
 void perm_batch_destroy(perm_batch_handle b);
 
 /* Autotuner (no counterpart in the paper): for each walks-per-warp choice (auto,
- * 2, 4, 8, 16, 32), hash size (hash_scale 0, 1) and stack ring (16, 64 records)
- * that comes to a layout of its own (a warp holds at most 8 walks, d = 3: 4),
- * times a complete run of probe_tours tours per sequence of cfg from empty
+ * 2, 4, 8), hash size (hash_scale 0, 1) and stack ring (16, 64 records) that
+ * comes to a layout of its own (a warp holds at most 8 walks, d = 3: 4), times a
+ * complete run of probe_tours tours per sequence of cfg from empty
  * tables (twice; the faster counts).  The default layout (auto, 0, 16) is timed
  * first and kept unless another choice is at least 3% faster and then at least
  * 3% faster again on runs of 4 x probe_tours (the fastest of three runs of each,
@@ -380,7 +380,8 @@ int perm_autotune(perm_config *cfg, int64_t probe_tours);
  * time-sliced at tour boundaries); an explicit cfg->slots (clamped to n_seq)
  * whose scratch exceeds the buffer is rejected with PERM_ESCRATCH.  The run
  * grows every waiting copy on the walk that made it (no shared copies:
- * share_copies 0 or -1 both mean that here) and uses the automatic layout;
+ * share_copies 0 or -1 both mean that here) and lays out as many walks as fit
+ * the buffer and the shared memory, over up to 11 warps per SM (8 with 64-bit keys);
  * observables, hash_scale, lanes_per_warp, stack_ring, max_ctas, walk_memory
  * other than 0, helper_walks > 0 or share_copies > 0 return PERM_EUNSUPPORTED (every walk's
  * state must then fit in shared memory).  Starts from empty tables and

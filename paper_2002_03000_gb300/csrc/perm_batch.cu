@@ -342,7 +342,7 @@ void perm_batch_destroy(perm_batch_handle b) { batch_free(b); }
 // Autotuner: short calibration runs over walks per warp, hash size and the
 // shared-memory stack ring ("spill tile").  Choices that come to a layout already timed
 // are left out (a warp holds at most 8 walks, 4 on the cubic lattice, and hash_scale 0
-// doubles the hash where it fits: of 23 choices about half repeat another).  Each trial times a complete run of
+// doubles the hash where it fits: about half of the choices repeat another).  Each trial times a complete run of
 // probe_tours tours per sequence from empty tables (twice, the faster counts),
 // so the trials compare equal work, start-up included.  The default layout is
 // timed first and stays unless a choice beats it by 3% and then again on runs
@@ -368,7 +368,7 @@ int perm_autotune(perm_config *cfg, int64_t probe_tours) {
             return PERM_OK;
         }
     }
-    const int lanes_c[] = {0, 2, 4, 8, 16, 32};
+    const int lanes_c[] = {0, 2, 4, 8};
     const int hash_c[] = {0, 1};
     const int ring_c[] = {16, 64};
     // the layouts timed so far: warps, walks a warp, CTAs, hash slots, ring

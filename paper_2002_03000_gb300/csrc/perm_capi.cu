@@ -115,9 +115,10 @@ void free_all(perm_handle h) {
 // cubic n = 512, 8192 x 128 173 / 168 / 166 / 165; square n = 256, 1000 x 64 32 / 28 / 26 / 25;
 // cubic n = 945, 2142 x 4 86 / 38 / 33 / 33; square n = 1725, 422 x 4 250 / 205 / 184 / 470.
 constexpr int kAutoWalks = 32;          // walks per CTA of the automatic layout, in the arena
-constexpr int kBatchWalks = 48;         // and of a persistent batch's members: each has scratch for
-                                        // a grid of such CTAs (24 runs of n = 64..256: 0.66, 0.76
-                                        // and 0.99 GB, 15.1, 15.4 and 15.6 ms at 40, 48 and 88)
+constexpr int kBatchWalks = 48;         // and about as many of a persistent batch's members: each has
+                                        // scratch for a grid of such CTAs (24 runs of n = 64..256:
+                                        // 0.66, 0.76 and 0.99 GB, 15.1, 15.4 and 15.6 ms at 40, 48
+                                        // and 88; whole warps of them, 10 x 5 where they fit)
 constexpr int kDefaultShareCap = 4;
 constexpr int kRampC0 = 2;              // the default admission limit
 constexpr double kRampGamma = 0.25;
@@ -340,8 +341,8 @@ int create_impl(perm_handle *out, const perm_config *cfg, const ForcedLayout *fo
     long long tslots = cfg->slots ? cfg->slots : (long long)n_seq;   // walks that grow tours
     if (tslots > n_seq) tslots = n_seq;
     // and helper walks: as asked (none by default), or (-1) the walks the automatic
-    // layout has room for beyond the tour walks (4 warps of 8 per SM), when shared
-    // copies are on
+    // layout has room for beyond the tour walks, up to 32 per SM, when shared copies
+    // are on
     const bool can_help = cfg->share_copies >= 0 && cfg->alg == PERM_ALG2 &&
                           cfg->threshold == PERM_THRESH_SNAPSHOT && !force;
     long long helpers = cfg->helper_walks;
@@ -515,8 +516,10 @@ static RunDev make_params(perm_handle h) {
     P.seq_target = h->seq_target;
     P.refresh_ns = h->cfg.refresh_ns;
     P.max_ns = (long long)(h->cfg.max_seconds * 1e9);
-    // original PERM's weights repeat, so that the order of a sum's terms hardly changes its rounding,
-    // but the number of sums does: one table keeps its tables within 5e-15 of a plain sum (four: 3.5e-14)
+    // original PERM keeps one table, so that its tables agree with a sequential sum of the same
+    // weights (within 5e-15; with four copies within 3.5e-14).  That is agreement, not accuracy: its
+    // weights repeat, equal terms round the same way each time, and both then are 3.4e-14 from the
+    // exact sum (four copies 1.1e-14; square, n = 257, 16000 tours)
     P.parts = h->cut ? 1 : h->parts; P.part_stride = kPartStride; P.Wp = h->Wp; P.Qp = h->Qp;
     P.Wn = h->Wn; P.Sn = h->Sn; P.Qn = h->Qn; P.Rn = h->Rn; P.tickets = h->tickets; P.seq_M = h->seq_M;
     P.X = h->X; P.gstk_meta = h->gstk_meta; P.gstk_w = h->gstk_w;

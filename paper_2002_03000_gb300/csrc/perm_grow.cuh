@@ -182,9 +182,13 @@ __device__ __forceinline__ void set_tours(Tours &t, unsigned long long M) {
     t.inv5 = __dmul_rn(5.0, t.inv1);
 }
 
-// The running average sum / M, correctly rounded: q = sum (1/M) and one step of the division
-// from the correctly rounded 1/M (M below 2^32, the sum far from the range's ends),
-// else the division itself.
+// The running average sum / M, correctly rounded: q = sum (1/M) and one correction by its
+// remainder with the correctly rounded 1/M (P. Markstein, "Computation of elementary functions
+// on the IBM RISC System/6000 processor", IBM J. Res. Dev. 34 (1990) 111-119), where M is
+// below 2^32 and the sum far from the range's ends; else the division itself.  (q is within
+// 1.5 units in the last place, so the remainder sum - q M, a multiple of q's last place below
+// 2^33 of them, is exact; the corrected value is then within 2^-52 units of the quotient,
+// which lies 2^-33 units or more from a midpoint between two doubles.)
 __device__ __forceinline__ double average(double sum, const Tours &t) {
     const double q = __dmul_rn(sum, t.inv1);
     double avg = __fma_rn(__fma_rn(-q, t.Md, sum), t.inv1, q);
@@ -239,8 +243,8 @@ __device__ __noinline__ double divided_survivor(double sum, unsigned long long M
 
 // The decision at a node with a >= 1 free neighbours (Sec. 2): r, the copies, the
 // children's weight.  sum: the weights recorded at length n up to this node, gs: what
-// the estimate of r says; refine: round the survivor's quotient by M correctly (one more step of the
-// division); divide: the snapshot form's M is not the snapshot's, and a survivor's quotient is
+// the estimate of r says; refine: round the survivor's quotient by M correctly (one correction
+// by its remainder); divide: the snapshot form's M is not the snapshot's, and a survivor's quotient is
 // divided out (a tour's first nodes, until the snapshot counts it).  valid: the lane has a node to decide (the others' results are not used);
 // force_exact: decide on the double-precision r.  Shared by the persistent kernel
 // and the snapshot-state kernel; every lane of a walk's group takes the same decision.
@@ -267,8 +271,9 @@ __device__ __forceinline__ Decision decide_node(int n, int a, double W, double s
     // path (in one branch with it: square n = 512 continued 50.8 -> 51.0 ms, cubic 120 -> 121)
     double base = W, fac = row[c];
     if (refine) {
-        // (under a branch: three dependent operations of 62 cycles, which ran no faster beside
-        // the probes)
+        // the quotient as average() forms it (past M = 2^32 it may be a unit in the last place
+        // off).  (Under a branch: three dependent operations of 62 cycles, which ran no faster
+        // beside the probes)
         if (surv) {
             const double q = __dmul_rn(sum, t.inv1);
             base = __fma_rn(__fma_rn(-q, t.Md, sum), t.inv1, q);

@@ -120,8 +120,8 @@ cudaError_t batch_grid(int threads, size_t smem, int *ctas);
 cudaError_t launch_batch(const BatchDev &B, int ctas, int threads, size_t smem, cudaStream_t stream);
 
 // Host side of batch members (runs whose descriptors sit in a batch's table):
-// a run laid out for `ctas` CTAs of at most 4 x 8 walks within smem_budget bytes
-// of shared memory, and its descriptor for tours_per_seq tours per sequence from
+// a run laid out for `ctas` CTAs of up to 10 x 5 walks within smem_budget bytes of
+// shared memory, and its descriptor for tours_per_seq tours per sequence from
 // empty tables.
 int member_create(perm_handle *out, const perm_config *cfg, int ctas, size_t smem_budget);
 int member_params(perm_handle h, int64_t tours_per_seq, int run_index, RunDev *P, size_t *smem,

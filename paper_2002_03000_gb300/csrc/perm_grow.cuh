@@ -268,7 +268,7 @@ __device__ __forceinline__ Decision decide_node(int n, int a, double W, double s
     // a_+ <= 5) is one of three products kept per M, its exponent shifted (exact: 1/M
     // is far from the subnormals); the weight is within 2^-51 of the quotient.  That holds for the
     // snapshot's M; with the tour's own number the quotient is divided out below, beside the exact
-    // path (in one branch with it: square n = 512 continued 50.8 -> 51.0 ms, cubic 120 -> 121)
+    // path (in one branch with it: under 1 %)
     double base = W, fac = row[c];
     if (refine) {
         // the quotient as average() forms it (past M = 2^32 it may be a unit in the last place
@@ -1157,8 +1157,6 @@ __device__ __forceinline__ void grow_run(const RunDev &P, unsigned char *smem, c
             bool hit, full;
             int place;
             look_bucket(hash, bucket, nkey, hit, full, place);
-            // (two lanes with different sums could decide differently and part for good)
-            if (snapshot && !cutoffs) Wsum = __shfl_sync(kFull, Wsum, lead);
             // the node's weight goes into the tables with reductions that return nothing, one
             // lane each.  Fresh form: a row of the walk's own takes a load (of the whole group)
             // and a store (of its first lane) through L1; on a shared one the add returns the
@@ -1177,7 +1175,8 @@ __device__ __forceinline__ void grow_run(const RunDev &P, unsigned char *smem, c
                 if (isn && Mt != tours.M) set_tours<!cutoffs>(tours, Mt);
             }
             red_add(acc + n, W, isn && (snapshot ? j < 2 : j == 1));
-            const double sum = __dadd_rn(Wsum, W);
+            double sum = 0.0;
+            if (!snapshot) sum = __dadd_rn(Wsum, W);
             if (!snapshot && own_rows && isn && first) Wrow[n] = sum;
             // a full bucket without the key, a used-up block of random words, a new M: one vote
             // for the three
@@ -1215,6 +1214,14 @@ __device__ __forceinline__ void grow_run(const RunDev &P, unsigned char *smem, c
             // of r says
             const int wl = lead + (int)((ord - pbase) & (uint32_t)(G - 1));
             const uint32_t w0 = __shfl_sync(kFull, pw0, wl), w1 = __shfl_sync(kFull, pw1, wl);
+            // the group's W_n is its first lane's (two lanes with different sums could decide
+            // differently and part for good); taken here, where the load is long done: right
+            // after the look it cost square n = 512 continued 49.5 -> 51.2 ms, 12 walks to n = 16
+            // 22.9 -> 23.9
+            if (snapshot && !cutoffs) {
+                Wsum = __shfl_sync(kFull, Wsum, lead);
+                sum = __dadd_rn(Wsum, W);
+            }
             Guess gs;
             if (!cutoffs) gs = guess(W, Wsum, tours.Mf, w0);
             // the first child's step (a draw from the free list), its key and its place in the

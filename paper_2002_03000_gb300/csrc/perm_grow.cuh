@@ -13,16 +13,16 @@
 //
 // What bounds it: the walks are few (one per sequence; an SM's shared memory and
 // registers hold at most 88), so the dependent instruction streams of 9 to 11 warps set
-// the rate (an SM issues on 38 % of its cycles at 9 warps), not memory or arithmetic.  On
+// the rate (an SM issues on 39 % of its cycles at 9 warps), not memory or arithmetic.  On
 // this part a lone warp pays 25 cycles or more for a branch, 45 for a vote and a branch on
 // it, 20-60 for a reduction, 33 for a shared-memory load, 64 for every double-precision
 // instruction whatever its active lanes (measured, one warp).  One lane per walk ran all
 // four (six) probes, the table updates and a dozen branches of a node one after another,
 // 7 walks to a warp; a group of lanes does them side by side, and the node is one straight
 // line.  GB300, one lane per walk -> the first form of a group -> now: 12 walks to n = 16,
-// 24 000 tours 48.5 -> 31.5 -> 23.1 ms; square n = 512, 4096 sequences, 96 tours each of a
-// continued run 193 -> 126 -> 49.8 ms, 256 tours from empty tables 561 -> 302 -> 164 ms;
-// cubic n = 512, 8192 sequences, 128 tours 491 -> 253 -> 118 ms.
+// 24 000 tours 48.5 -> 31.5 -> 22.9 ms; square n = 512, 4096 sequences, 96 tours each of a
+// continued run 193 -> 126 -> 49.5 ms, 256 tours from empty tables 561 -> 302 -> 164 ms;
+// cubic n = 512, 8192 sequences, 128 tours 491 -> 253 -> 119 ms.
 //
 // Threshold sources for Algorithm 2 (one shared table W, Fig. 1):
 //  - snapshot: every node adds its weight to the global table with a

@@ -9,6 +9,8 @@
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
+#include <memory>
+#include <new>
 #include <string>
 #include <vector>
 
@@ -126,13 +128,28 @@ constexpr int kBoostShareCap = 1024;
 constexpr long long kStallNs = 700000;
 
 // S_n is kept on the device as its differences along n, row by row of L entries.
-void counts_from_differences(std::vector<unsigned long long> &s, size_t L) {
-    for (size_t i = 0; i < s.size(); ++i)
-        if (i % L != 0) s[i] += s[i - 1];
+// (out may be the differences' own memory.)
+template <typename T>
+void counts_from_differences(const void *differences, size_t cnt, size_t L, T *out) {
+    const unsigned char *s = static_cast<const unsigned char *>(differences);
+    for (size_t row = 0; row < cnt; row += L) {
+        unsigned long long sum = 0ull, d;
+        for (size_t i = row; i < row + L; ++i) {
+            std::memcpy(&d, s + 8 * i, 8);
+            out[i] = (T)(sum += d);
+        }
+    }
 }
-void differences_from_counts(std::vector<unsigned long long> &s, size_t L) {
-    for (size_t i = s.size(); i-- > 0;)
-        if (i % L != 0) s[i] -= s[i - 1];
+void differences_from_counts(unsigned char *s, size_t cnt, size_t L) {
+    for (size_t row = 0; row < cnt; row += L) {
+        unsigned long long before = 0ull, c;
+        for (size_t i = row; i < row + L; ++i) {
+            std::memcpy(&c, s + 8 * i, 8);
+            const unsigned long long d = c - before;
+            std::memcpy(s + 8 * i, &d, 8);
+            before = c;
+        }
+    }
 }
 
 // A length's cut-offs as the kernel compares them, by their bit patterns: no NaN (which no
@@ -652,22 +669,15 @@ int perm_tables(perm_handle h, double *W_n, double *S_n, double *Q_n, int64_t *M
         if (st < 0 && st != PERM_EOVERFLOW && st != PERM_ETIMEOUT) return st;
         if (W_n) std::memcpy(W_n, buf.data() + o_W, cnt * 8);
         if (Q_n) std::memcpy(Q_n, buf.data() + o_Q, cnt * 8);
-        if (S_n) {
-            std::vector<unsigned long long> s(cnt);
-            std::memcpy(s.data(), buf.data() + o_S, cnt * 8);
-            counts_from_differences(s, L);
-            for (size_t i = 0; i < cnt; ++i) S_n[i] = (double)s[i];
-        }
+        if (S_n) counts_from_differences(buf.data() + o_S, cnt, L, S_n);
     } else {
         st = sync_status(h);
         if (st < 0 && st != PERM_EOVERFLOW && st != PERM_ETIMEOUT) return st;
         if (W_n) e = copy_out(h, W_n, h->Wn, cnt * sizeof(double));
         if (e == cudaSuccess && Q_n) e = copy_out(h, Q_n, h->Qn, cnt * sizeof(double));
         if (e == cudaSuccess && S_n) {
-            std::vector<unsigned long long> s(cnt);
-            e = copy_out(h, s.data(), h->Sn, cnt * sizeof(unsigned long long));
-            counts_from_differences(s, L);
-            for (size_t i = 0; i < cnt; ++i) S_n[i] = (double)s[i];
+            e = copy_out(h, S_n, h->Sn, cnt * sizeof(unsigned long long));
+            if (e == cudaSuccess) counts_from_differences(S_n, cnt, L, S_n);
         }
     }
     if (e == cudaSuccess && M) {
@@ -1016,7 +1026,7 @@ int perm_save(perm_handle h, const char *path) {
     cudaError_t e = copy_out(h, W.data(), h->Wn, cnt * 8);
     if (e == cudaSuccess) e = copy_out(h, Q.data(), h->Qn, cnt * 8);
     if (e == cudaSuccess) e = copy_out(h, S.data(), h->Sn, cnt * 8);
-    counts_from_differences(S, L);                          // a checkpoint holds counts
+    counts_from_differences(S.data(), cnt, L, S.data());    // a checkpoint holds counts
     if (e == cudaSuccess && hd.has_rn) e = copy_out(h, R.data(), h->Rn, cnt * 8);
     if (e == cudaSuccess) e = copy_out(h, sM.data(), h->seq_M, sM.size() * 8);
     if (e == cudaSuccess && hd.has_cut) e = copy_out(h, cut.data(), h->cut, L * sizeof(double2));
@@ -1061,17 +1071,19 @@ int perm_load(perm_handle *out, const char *path) {
               hd.version == kCkptVersion && hd.header_bytes == (uint32_t)sizeof(CkptHeader);
     const uint64_t payload = ok ? ckpt_payload(hd) : 0;
     ok = ok && payload > 0;
-    std::vector<unsigned char> body(ok ? (size_t)payload : 0);
-    ok = ok && std::fread(body.data(), 1, body.size(), f) == body.size();
+    // (not cleared: the file fills it)
+    std::unique_ptr<unsigned char[]> body(ok ? new (std::nothrow) unsigned char[(size_t)payload] : nullptr);
+    const bool room = !ok || body != nullptr;
+    ok = ok && room && std::fread(body.get(), 1, (size_t)payload, f) == (size_t)payload;
     ok = ok && std::fgetc(f) == EOF;                        // nothing after the arrays
     std::fclose(f);
-    if (!ok) return PERM_EINVAL;
+    if (!ok) return room ? PERM_EINVAL : PERM_ENOMEM;
     perm_handle h = nullptr;
     int rc = perm_create_ex(&h, &hd.cfg);
     if (rc != PERM_OK) return rc;
     if (hd.has_rn != (h->Rn != nullptr)) { perm_destroy(h); return PERM_EINVAL; }
     const size_t L = (size_t)hd.cfg.n_max + 1, cnt = L * (size_t)hd.ntab;
-    const unsigned char *p = body.data();
+    unsigned char *p = body.get();
     auto put = [&](void *dev, size_t bytes) {
         cudaError_t e = cudaMemcpyAsync(dev, p, bytes, cudaMemcpyHostToDevice, h->stream);
         p += bytes;
@@ -1080,12 +1092,8 @@ int perm_load(perm_handle *out, const char *path) {
     cudaError_t e = put(h->Wn, cnt * 8);
     if (e == cudaSuccess) e = put(h->Qn, cnt * 8);
     if (e == cudaSuccess) {
-        std::vector<unsigned long long> S(cnt);
-        std::memcpy(S.data(), p, cnt * 8);
-        p += cnt * 8;
-        differences_from_counts(S, L);
-        e = cudaMemcpyAsync(h->Sn, S.data(), cnt * 8, cudaMemcpyHostToDevice, h->stream);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
+        differences_from_counts(p, cnt, L);
+        e = put(h->Sn, cnt * 8);
     }
     if (e == cudaSuccess && hd.has_rn) e = put(h->Rn, cnt * 8);
     if (e == cudaSuccess) e = put(h->seq_M, (size_t)hd.cfg.n_seq * 8);
